@@ -42,13 +42,17 @@ struct ConvIn {
 // warps) computes 128 consecutive voxels (M = 128) times all output channels
 // (N = Cout) into a float32 accumulator in tensor memory; K = 27 taps x C_in
 // runs in chunks of 16 channels, one tcgen05.mma (kind::f16, bf16 inputs) per
-// chunk.  Every thread gathers its voxel's 16 channels of the chunk (zero
-// outside the grid: the convolution's padding) and the first N threads the
-// weights' rows into this CTA's shared memory, in the K-major layout without
-// swizzling (core matrices of 8 rows x 16 bytes; neighbours along K 128
-// bytes apart, along M/N 256 bytes apart).  Two stages alternate: while the
-// tensor core works on one, the threads fill the other; the MMA's completion
-// is signalled to an mbarrier by tcgen05.commit.  The epilogue reads the
+// chunk, GRP chunks to a stage.  Every thread gathers its voxel's 16 channels
+// of each chunk (zero outside the grid: the convolution's padding) and the
+// first N threads the weights' rows, into registers while the tensor core
+// still reads the stage, then into this CTA's shared memory, in the K-major
+// layout without swizzling (core matrices of 8 rows x 16 bytes; neighbours
+// along K 128 bytes apart, along M/N 256 bytes apart).  Two stages alternate;
+// the MMAs' completion is signalled to an mbarrier by tcgen05.commit.  What
+// bounds it: the latency of a stage's gathers and barrier (9 stages per 16
+// input channels); with one chunk to a stage there were 27 of them, and the 19
+// convolutions of a gradient at 64^3 took 1086 us; now 780 us.  The
+// accumulation order is that of the chunks either way.  The epilogue reads the
 // accumulator rows back with tcgen05.ld (warp w owns lanes 32w..32w+31), adds
 // the bias, applies the ReLU and stores bf16.  Every mbarrier wait is
 // bounded: on expiry the kernel sets *err, skips the epilogue and still
@@ -111,10 +115,12 @@ __device__ __forceinline__ void in16(const ConvIn& a, int Z, int Y, int X, int z
   hi = *reinterpret_cast<const uint4*>(p + 8);
 }
 
+static constexpr int GRP = 3;  // chunks per stage (their number is 27 C_in / 16)
+
 template <int N>
 __global__ void __launch_bounds__(128) k_conv3_tc(ConvIn a, const bf16* __restrict__ W, const float* __restrict__ bias,
                                                   bf16* out, int Z, int Y, int X, int relu, int* err) {
-  constexpr int A_BYTES = 128 * 32, B_BYTES = N * 32, STAGE = A_BYTES + B_BYTES;
+  constexpr int A_BYTES = 128 * 32, B_BYTES = N * 32, CHUNK = A_BYTES + B_BYTES, STAGE = GRP * CHUNK;
   constexpr int TM_COLS = N <= 32 ? 32 : (N <= 64 ? 64 : 128);
   __shared__ __align__(1024) unsigned char sm[2 * STAGE];
   __shared__ __align__(8) unsigned long long mbar[2];
@@ -139,49 +145,60 @@ __global__ void __launch_bounds__(128) k_conv3_tc(ConvIn a, const bf16* __restri
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_slot;
-  const int chunks_per_tap = Cin / 16, nchunk = 27 * chunks_per_tap;
+  const int chunks_per_tap = Cin / 16, ngroup = 27 * chunks_per_tap / GRP;
   constexpr uint32_t IDESC = tc::instr_desc(128, N);
   bool ok = true;
-  for (int c = 0; c < nchunk && ok; ++c) {
-    const int s = c & 1;
-    if (c >= 2) ok = tc::mbar_wait(tc::saddr(&mbar[s]), ((c - 2) >> 1) & 1);  // stage s free again
-    if (!ok) break;
-    const int tap = c / chunks_per_tap, cb = (c - tap * chunks_per_tap) * 16;
-    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-    unsigned char* As = sm + s * STAGE;
-    unsigned char* Bs = As + A_BYTES;
-    uint4 lo, hi;
-    if (vok) {
-      in16(a, Z, Y, X, z + dz, y + dy, x + dx, cb, lo, hi);
-    } else {
-      lo = make_uint4(0u, 0u, 0u, 0u);
-      hi = lo;
+  for (int gq = 0; gq < ngroup && ok; ++gq) {
+    const int s = gq & 1;
+    // the group's operands into registers: every load in flight at once
+    uint4 al[GRP], ah[GRP], bl[GRP], bh[GRP];
+#pragma unroll
+    for (int q = 0; q < GRP; ++q) {
+      const int c = gq * GRP + q, tap = c / chunks_per_tap, cb = (c - tap * chunks_per_tap) * 16;
+      const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+      al[q] = make_uint4(0u, 0u, 0u, 0u);
+      ah[q] = al[q];
+      if (vok) in16(a, Z, Y, X, z + dz, y + dy, x + dx, cb, al[q], ah[q]);
+      if (tid < N) {
+        const uint4* wr = reinterpret_cast<const uint4*>(W + ((size_t)tap * N + tid) * Cin + cb);
+        bl[q] = wr[0];
+        bh[q] = wr[1];
+      }
     }
-    *reinterpret_cast<uint4*>(As + tc::tile_off(tid, 0)) = lo;
-    *reinterpret_cast<uint4*>(As + tc::tile_off(tid, 8)) = hi;
-    if (tid < N) {
-      const bf16* wr = W + ((size_t)tap * N + tid) * Cin + cb;
-      *reinterpret_cast<uint4*>(Bs + tc::tile_off(tid, 0)) = *reinterpret_cast<const uint4*>(wr);
-      *reinterpret_cast<uint4*>(Bs + tc::tile_off(tid, 8)) = *reinterpret_cast<const uint4*>(wr + 8);
+    if (gq >= 2) ok = tc::mbar_wait(tc::saddr(&mbar[s]), ((gq - 2) >> 1) & 1);  // stage s free again
+    if (!ok) break;
+#pragma unroll
+    for (int q = 0; q < GRP; ++q) {
+      unsigned char* As = sm + s * STAGE + q * CHUNK;
+      unsigned char* Bs = As + A_BYTES;
+      *reinterpret_cast<uint4*>(As + tc::tile_off(tid, 0)) = al[q];
+      *reinterpret_cast<uint4*>(As + tc::tile_off(tid, 8)) = ah[q];
+      if (tid < N) {
+        *reinterpret_cast<uint4*>(Bs + tc::tile_off(tid, 0)) = bl[q];
+        *reinterpret_cast<uint4*>(Bs + tc::tile_off(tid, 8)) = bh[q];
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint64_t ad = tc::smem_desc(tc::saddr(As), 128, 256), bd = tc::smem_desc(tc::saddr(Bs), 128, 256);
-      const uint32_t acc = c > 0 ? 1u : 0u;
-      asm volatile(
-          "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-          "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
+#pragma unroll
+      for (int q = 0; q < GRP; ++q) {
+        const uint32_t as = tc::saddr(sm + s * STAGE + q * CHUNK);
+        const uint64_t ad = tc::smem_desc(as, 128, 256), bd = tc::smem_desc(as + A_BYTES, 128, 256);
+        const uint32_t acc = (gq > 0 || q > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+            "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
+      }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
           tc::saddr(&mbar[s])));
     }
   }
-  // every issued chunk has completed once the last two commits have arrived
+  // every issued group has completed once the last two commits have arrived
   if (ok) {
-    for (int c = (nchunk >= 2 ? nchunk - 2 : 0); c < nchunk && ok; ++c)
-      ok = tc::mbar_wait(tc::saddr(&mbar[c & 1]), (c >> 1) & 1);
+    for (int gq = ngroup - 2; gq < ngroup && ok; ++gq) ok = tc::mbar_wait(tc::saddr(&mbar[gq & 1]), (gq >> 1) & 1);
   }
   if (!ok && tid == 0) atomicExch(err, 1);
   asm volatile("tcgen05.fence::after_thread_sync;");
@@ -259,16 +276,38 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* out, int Z, int Y, int
   }
 }
 
-// d_fine (+)= pool adjoint of d_coarse: each child gets 1/8 of its parent
-__global__ void k_pool_bwd(const bf16* __restrict__ dc, bf16* df, int Z, int Y, int X, int C, int accumulate) {
-  size_t n = (size_t)Z * Y * X * C;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    int c = (int)(t % C);
-    size_t v = t / C;
-    int x = (int)(v % X), y = (int)((v / X) % Y), z = (int)(v / ((size_t)X * Y));
-    float g = 0.125f * __bfloat162float(dc[(((size_t)(z >> 1) * (Y >> 1) + (y >> 1)) * (X >> 1) + (x >> 1)) * C + c]);
-    if (accumulate) g += __bfloat162float(df[t]);
-    df[t] = __float2bfloat16(g);
+// The element-wise passes of the backward pass handle eight channels (16
+// bytes) per thread; every channel count and offset is a multiple of 16.
+__device__ __forceinline__ void unpack8(uint4 r, float f[8]) {
+  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&r);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    f[2 * t] = __low2float(h[t]);
+    f[2 * t + 1] = __high2float(h[t]);
+  }
+}
+__device__ __forceinline__ uint4 pack8(const float f[8]) {
+  uint4 r;
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&r);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) h[t] = __floats2bfloat162_rn(f[2 * t], f[2 * t + 1]);
+  return r;
+}
+__device__ __forceinline__ uint4 ld8(const bf16* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ void st8(bf16* p, uint4 v) { *reinterpret_cast<uint4*>(p) = v; }
+
+// d_fine += pool adjoint of d_coarse: each child gets 1/8 of its parent
+__global__ void k_pool_bwd(const bf16* __restrict__ dc, bf16* df, int Z, int Y, int X, int C) {
+  const unsigned c8 = C / 8, n = (unsigned)((size_t)Z * Y * X * c8);
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const unsigned c = t % c8 * 8, v = t / c8;
+    const int x = (int)(v % X), y = (int)(v / X % Y), z = (int)(v / ((unsigned)X * Y));
+    float g[8], d[8];
+    unpack8(ld8(dc + (((size_t)(z >> 1) * (Y >> 1) + (y >> 1)) * (X >> 1) + (x >> 1)) * C + c), g);
+    unpack8(ld8(df + (size_t)t * 8), d);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) g[q] = 0.125f * g[q] + d[q];
+    st8(df + (size_t)t * 8, pack8(g));
   }
 }
 
@@ -290,26 +329,26 @@ __global__ void k_up_bwd(const bf16* __restrict__ df, bf16* dc, int Z, int Y, in
   }
 }
 
-// d[v][c] = (y[v][c] > 0) ? d : 0, optionally reading d from channels
-// [coff, coff + C) of a wider tensor (Ct channels) into a packed one
-__global__ void k_relu_mask(const bf16* __restrict__ d, int Ct, int coff, const bf16* __restrict__ y, bf16* out,
-                            size_t V, int C) {
-  size_t n = V * C;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    int c = (int)(t % C);
-    size_t v = t / C;
-    float g = __bfloat162float(d[v * Ct + coff + c]);
-    out[t] = __bfloat162float(y[t]) > 0.f ? __float2bfloat16(g) : __float2bfloat16(0.f);
+// d[v][c] = (y[v][c] > 0) ? d : 0
+__global__ void k_relu_mask(const bf16* __restrict__ d, const bf16* __restrict__ y, bf16* out, size_t n8) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n8; t += (size_t)gridDim.x * blockDim.x) {
+    float g[8], a[8];
+    unpack8(ld8(d + t * 8), g);
+    unpack8(ld8(y + t * 8), a);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) g[q] = a[q] > 0.f ? g[q] : 0.f;
+    st8(out + t * 8, pack8(g));
   }
 }
 
-// dst += src (bf16, same shape), for gradients meeting at a skip connection
-__global__ void k_add_from(bf16* dst, const bf16* __restrict__ src, int Cs, int soff, size_t V, int C) {
-  size_t n = V * C;
+// dst = channels [soff, soff + C) of src (Cs channels): the gradient that
+// reaches a skip connection
+__global__ void k_take(bf16* dst, const bf16* __restrict__ src, int Cs, int soff, size_t V, int C) {
+  const int c8 = C / 8;
+  const size_t n = V * c8;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    int c = (int)(t % C);
-    size_t v = t / C;
-    dst[t] = __float2bfloat16(__bfloat162float(dst[t]) + __bfloat162float(src[v * Cs + soff + c]));
+    const size_t v = t / c8;
+    st8(dst + t * 8, ld8(src + v * Cs + soff + (t - v * c8) * 8));
   }
 }
 
@@ -676,14 +715,13 @@ void unet_forward(UNetImpl* u, cudaStream_t st) {
   { k_head<<<nblk(V), 256, 0, st>>>(u->ua2, u->w + u->headw, u->w + u->headb, u->out, V, c0); WSI_COUNT(); }
 }
 
-// One layer's backward: G (gradient of its output, channels [goff, goff+Cout)
-// of a tensor with Gt channels) -> weight/bias gradients, and (if dX) the
-// input gradient [V][C0 + C1] into dX.
-static void layer_bwd(UNetImpl* u, int l, const bf16* in0, const bf16* in1, const bf16* y, const bf16* G, int Gt,
-                      int goff, bf16* M, bf16* dX, int z, int yy, int x, cudaStream_t st) {
+// One layer's backward: G (gradient of its output) -> weight/bias gradients,
+// and (if dX) the input gradient [V][C0 + C1] into dX.
+static void layer_bwd(UNetImpl* u, int l, const bf16* in0, const bf16* in1, const bf16* y, const bf16* G, bf16* M,
+                      bf16* dX, int z, int yy, int x, cudaStream_t st) {
   ConvLayer& L = u->L[l];
   size_t V = (size_t)z * yy * x;
-  { k_relu_mask<<<nblk(V * L.Cout), 256, 0, st>>>(G, Gt, goff, y, M, V, L.Cout); WSI_COUNT(); }
+  { k_relu_mask<<<nblk(V * L.Cout / 8), 256, 0, st>>>(G, y, M, V * L.Cout / 8); WSI_COUNT(); }
   ConvIn a{in0, L.C0, L.up0, in1, L.C1};
   // bricks spread over about four blocks per SM of each (o, c) tile's share
   const int bx = cdiv(x, DWX), by = cdiv(yy, DWY), nbr = bx * by * cdiv(z, DWZ);
@@ -705,36 +743,37 @@ void unet_backward(UNetImpl* u, cudaStream_t st) {
   { k_head_bwd<<<std::min(nblk(V), 152 * 2), 256, 0, st>>>(u->out, u->tgt, u->ua2, u->w + u->headw, V, c0, u->g + u->headw,
                                         u->g + u->headb, u->g0, u->loss); WSI_COUNT(); }
   // full resolution decoder
-  layer_bwd(u, 9, u->ua1, nullptr, u->ua2, u->g0, c0, 0, u->g1, u->g2, Z, Y, X, st);           // d ua1 -> g2
-  layer_bwd(u, 8, u->ub2, u->a2, u->ua1, u->g2, c0, 0, u->g1, u->g0, Z, Y, X, st);             // d [up(ub2), a2] -> g0
+  layer_bwd(u, 9, u->ua1, nullptr, u->ua2, u->g0, u->g1, u->g2, Z, Y, X, st);           // d ua1 -> g2
+  layer_bwd(u, 8, u->ub2, u->a2, u->ua1, u->g2, u->g1, u->g0, Z, Y, X, st);             // d [up(ub2), a2] -> g0
   // skip gradient of a2: gA = g0[:, c1:] (its ReLU mask is applied with the
   // pooled-path gradient, in layer a2's backward)
-  cudaMemsetAsync(u->gA, 0, V * c0 * sizeof(bf16), st);
-  { k_add_from<<<nblk(V * c0), 256, 0, st>>>(u->gA, u->g0, c1 + c0, c1, V, c0); WSI_COUNT(); }
+  { k_take<<<nblk(V * c0 / 8), 256, 0, st>>>(u->gA, u->g0, c1 + c0, c1, V, c0); WSI_COUNT(); }
   { k_up_bwd<<<nblk(V2 * c1), 256, 0, st>>>(u->g0, u->g2, Z / 2, Y / 2, X / 2, c1 + c0, c1); WSI_COUNT(); }  // d ub2
   // half resolution decoder
-  layer_bwd(u, 7, u->ub1, nullptr, u->ub2, u->g2, c1, 0, u->g1, u->g0, Z / 2, Y / 2, X / 2, st);  // d ub1 -> g0
-  layer_bwd(u, 6, u->cc2, u->b2, u->ub1, u->g0, c1, 0, u->g1, u->g2, Z / 2, Y / 2, X / 2, st);    // d [up(cc2), b2] -> g2
-  cudaMemsetAsync(u->gB, 0, V2 * c1 * sizeof(bf16), st);
-  { k_add_from<<<nblk(V2 * c1), 256, 0, st>>>(u->gB, u->g2, c2 + c1, c2, V2, c1); WSI_COUNT(); }
+  layer_bwd(u, 7, u->ub1, nullptr, u->ub2, u->g2, u->g1, u->g0, Z / 2, Y / 2, X / 2, st);  // d ub1 -> g0
+  layer_bwd(u, 6, u->cc2, u->b2, u->ub1, u->g0, u->g1, u->g2, Z / 2, Y / 2, X / 2, st);    // d [up(cc2), b2] -> g2
+  { k_take<<<nblk(V2 * c1 / 8), 256, 0, st>>>(u->gB, u->g2, c2 + c1, c2, V2, c1); WSI_COUNT(); }
   { k_up_bwd<<<nblk(V4 * c2), 256, 0, st>>>(u->g2, u->g0, Z / 4, Y / 4, X / 4, c2 + c1, c2); WSI_COUNT(); }  // d cc2
   // bottom
-  layer_bwd(u, 5, u->cc1, nullptr, u->cc2, u->g0, c2, 0, u->g1, u->g2, Z / 4, Y / 4, X / 4, st);  // d cc1 -> g2
-  layer_bwd(u, 4, u->pb, nullptr, u->cc1, u->g2, c2, 0, u->g1, u->g0, Z / 4, Y / 4, X / 4, st);   // d pb -> g0
-  { k_pool_bwd<<<nblk(V2 * c1), 256, 0, st>>>(u->g0, u->gB, Z / 2, Y / 2, X / 2, c1, 1); WSI_COUNT(); }  // d b2
+  layer_bwd(u, 5, u->cc1, nullptr, u->cc2, u->g0, u->g1, u->g2, Z / 4, Y / 4, X / 4, st);  // d cc1 -> g2
+  layer_bwd(u, 4, u->pb, nullptr, u->cc1, u->g2, u->g1, u->g0, Z / 4, Y / 4, X / 4, st);   // d pb -> g0
+  { k_pool_bwd<<<nblk(V2 * c1 / 8), 256, 0, st>>>(u->g0, u->gB, Z / 2, Y / 2, X / 2, c1); WSI_COUNT(); }  // d b2
   // half resolution encoder
-  layer_bwd(u, 3, u->b1, nullptr, u->b2, u->gB, c1, 0, u->g1, u->g2, Z / 2, Y / 2, X / 2, st);    // d b1 -> g2
-  layer_bwd(u, 2, u->pa, nullptr, u->b1, u->g2, c1, 0, u->g1, u->g0, Z / 2, Y / 2, X / 2, st);    // d pa -> g0
-  { k_pool_bwd<<<nblk(V * c0), 256, 0, st>>>(u->g0, u->gA, Z, Y, X, c0, 1); WSI_COUNT(); }        // d a2
+  layer_bwd(u, 3, u->b1, nullptr, u->b2, u->gB, u->g1, u->g2, Z / 2, Y / 2, X / 2, st);    // d b1 -> g2
+  layer_bwd(u, 2, u->pa, nullptr, u->b1, u->g2, u->g1, u->g0, Z / 2, Y / 2, X / 2, st);    // d pa -> g0
+  { k_pool_bwd<<<nblk(V * c0 / 8), 256, 0, st>>>(u->g0, u->gA, Z, Y, X, c0); WSI_COUNT(); }        // d a2
   // full resolution encoder
-  layer_bwd(u, 1, u->a1, nullptr, u->a2, u->gA, c0, 0, u->g1, u->g2, Z, Y, X, st);                // d a1 -> g2
-  layer_bwd(u, 0, u->x, nullptr, u->a1, u->g2, c0, 0, u->g1, nullptr, Z, Y, X, st);
+  layer_bwd(u, 1, u->a1, nullptr, u->a2, u->gA, u->g1, u->g2, Z, Y, X, st);                // d a1 -> g2
+  layer_bwd(u, 0, u->x, nullptr, u->a1, u->g2, u->g1, nullptr, Z, Y, X, st);
 }
 
 // float [V][3] -> the network's bf16 [V][16] input (channels 3..15 zero)
 __global__ void k_input3(const float* __restrict__ x3, bf16* x, size_t V) {
-  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x)
-    for (int c = 0; c < 16; ++c) x[v * 16 + c] = __float2bfloat16(c < 3 ? x3[v * 3 + c] : 0.f);
+  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
+    const float f[8] = {x3[v * 3], x3[v * 3 + 1], x3[v * 3 + 2], 0.f, 0.f, 0.f, 0.f, 0.f};
+    st8(x + v * 16, pack8(f));
+    st8(x + v * 16 + 8, make_uint4(0u, 0u, 0u, 0u));
+  }
 }
 
 void unet_set_input3(UNetImpl* u, const float* x3, cudaStream_t st) {
