@@ -125,7 +125,9 @@ struct wsi_ctx {
   UNetImpl* unet_impl = nullptr;
   int unet_level = 0;
   bool unet_on = false;
-  SpreadWork sw;                  // deterministic spreading work arrays (allocated on first use)
+  unsigned long long* sacc = nullptr;  // deterministic spreading: one integer per face (on first use)
+  MarkerBins bins;                // markers sorted by cell (grown on first use)
+  void* bins_mem = nullptr;
   double* mbox = nullptr;         // 6 doubles: marker extent
   UNetImpl* gunet_impl = nullptr;  // initial-guess network (wsi_attach_unet_guess)
   int gunet_level = 0;
@@ -169,16 +171,42 @@ double* dalloc(wsi_ctx* c, size_t n) {
   return (double*)p;
 }
 
-// deterministic spreading work arrays (zero-filled; they are left zero by
-// every spreading call)
+// room for n markers in the bins
+bool ensure_bins(wsi_ctx* c, int n) {
+  MarkerBins& b = c->bins;
+  if (!b.cnt) {
+    b.cnt = (int*)dalloc(c, c->ncell / 2 + 1);
+    b.ctr = (int*)dalloc(c, BIN_CTR_BYTES / 8);
+    b.fmx = (unsigned long long*)(b.ctr + 4);
+    if (!b.cnt || !b.ctr) {
+      b.cnt = nullptr;
+      return false;
+    }
+  }
+  if (n <= b.cap) return true;
+  int* p = nullptr;
+  if (cudaMalloc(&p, (size_t)n * 7 * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (c->bins_mem) {
+    cudaStreamSynchronize(c->st);
+    cudaFree(c->bins_mem);
+  }
+  c->bins_mem = p;
+  int** q[7] = {&b.cellof, &b.rank, &b.perm, &b.lcell, &b.lstart, &b.lcnt, &b.irr};
+  for (int a = 0; a < 7; ++a) *q[a] = p + (size_t)a * n;
+  b.cap = n;
+  return true;
+}
+
+// deterministic spreading work array (zero-filled; left zero by every
+// spreading call)
 bool ensure_spread_work(wsi_ctx* c) {
-  if (c->sw.acc) return true;
-  c->sw.acc = (unsigned long long*)dalloc(c, c->nvel);
-  c->sw.cnt = (int*)dalloc(c, c->ncell / 2 + 1);
-  c->sw.qexp = (int*)dalloc(c, 1);
-  c->sw.part = dalloc(c, 6 * 152);
+  if (c->sacc) return true;
   c->mbox = dalloc(c, 6);
-  return c->sw.acc && c->sw.cnt && c->sw.qexp && c->sw.part && c->mbox;
+  c->sacc = (unsigned long long*)dalloc(c, c->nvel);
+  return c->sacc && c->mbox;
 }
 
 void vel_parts(wsi_ctx* c, double* base, double* out[3]) {
@@ -490,16 +518,16 @@ bool solve3(double A[3][3], const double b[3], double x[3]) {
 // Rigidity projection at marker positions Xuse: vel += S(U_b - J vel).
 int dlm_project(wsi_ctx* c, double* velv, const double* Xuse) {
   Body& B = c->body;
-  double* vq[3];
-  vel_parts(c, velv, vq);
-  const double* cq[3] = {vq[0], vq[1], vq[2]};
-  if (!ensure_spread_work(c)) return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
-  launch_marker_mean(Xuse, B.n, B.xc, B.scratch, c->st);
-  launch_ib_interp(c->g, cq, Xuse, B.n, B.U, c->st);
-  launch_rigid_sums(Xuse, B.U, B.n, B.xc, B.sums, B.scratch, c->st);
-  launch_marker_box(Xuse, B.n, c->mbox, c->sw.part, c->st);
-  double hs[15], xc[3], mm[6];
-  cudaMemcpyAsync(hs, B.sums, sizeof(hs), cudaMemcpyDeviceToHost, c->st);
+  if (!ensure_spread_work(c) || !ensure_bins(c, B.n)) return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
+  launch_marker_mean_box(Xuse, B.n, B.xc, c->mbox, B.scratch, c->st);
+  launch_marker_bins(c->g, Xuse, B.n, c->bins, c->st);
+  launch_ib_interp(c->g, velv, Xuse, B.n, c->bins, B.U, c->st);
+  // the fitted motion of a fully locked body is not used
+  bool locked = true;
+  for (int d = 0; d < 6; ++d) locked = locked && B.lock[d];
+  if (!locked) launch_rigid_sums(Xuse, B.U, B.n, B.xc, B.sums, B.scratch, c->st);
+  double hs[12] = {0}, xc[3], mm[6];
+  if (!locked) cudaMemcpyAsync(hs, B.sums, sizeof(hs), cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(xc, B.xc, sizeof(xc), cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(mm, c->mbox, sizeof(mm), cudaMemcpyDeviceToHost, c->st);
   if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "dlm sums");
@@ -517,8 +545,9 @@ int dlm_project(wsi_ctx* c, double* velv, const double* Xuse) {
   }
   double rg[6] = {Ur[0], Ur[1], Ur[2], Wr[0], Wr[1], Wr[2]};
   cudaMemcpyAsync(B.rig, rg, sizeof(rg), cudaMemcpyHostToDevice, c->st);
-  launch_body_velocity(Xuse, B.U, B.n, B.rig, B.xc, B.Ub, B.F, c->st);
-  launch_ib_spread(c->g, B.F, Xuse, B.n, B.dV, vq, c->sw, spread_box(c->g, mm), c->st);
+  launch_body_velocity(Xuse, B.U, B.n, B.rig, B.xc, B.Ub, B.F, c->bins, c->st);
+  launch_ib_spread(c->g, B.F, Xuse, B.n, B.dV, velv, c->sacc, c->bins, spread_box(c->g, mm), c->st);
+  launch_marker_bins_clear(B.n, c->bins, c->st);
   for (int d = 0; d < 3; ++d) {
     B.U_r[d] = Ur[d];
     B.W_r[d] = Wr[d];
@@ -914,6 +943,7 @@ void wsi_destroy(wsi_ctx* c) {
   if (c->st) cudaStreamSynchronize(c->st);
   precond_free<double>(c->P64);
   precond_free<float>(c->P32);
+  cudaFree(c->bins_mem);
   df_operands_release(c->df);
   for (void* p : c->allocs) cudaFree(p);
   delete c;
@@ -1076,7 +1106,7 @@ int wsi_step(wsi_ctx* c, double dt, const wsi_solve_opts* o, wsi_step_stats* s) 
                          B.U_pres[0] == 0.0 && B.U_pres[1] == 0.0 && B.U_pres[2] == 0.0 && B.W_pres[0] == 0.0 &&
                          B.W_pres[1] == 0.0 && B.W_pres[2] == 0.0;
     if (c->has_body && (B.shape == 1 || B.shape == 2) && !(at_rest && c->psi_static_done)) {
-      launch_marker_mean(B.X, B.n, B.xc, B.scratch, st);
+      launch_marker_mean_box(B.X, B.n, B.xc, nullptr, B.scratch, st);
       if (B.shape == 1)
         launch_box_sdf(g, B.xc, B.half, c->psi_new, st);
       else
@@ -1438,15 +1468,16 @@ int wsi_reinit(wsi_ctx* c, double* phi, int iters) {
 int wsi_interp(wsi_ctx* c, const double* vel, const double* X, int n, double* U) {
   if (valid_ctx(c)) return WSI_ERR_INVALID_ARG;
   if (n <= 0) return WSI_OK;
+  if (!ensure_bins(c, n)) return fail(c, WSI_ERR_OOM, "out of device memory for markers");
   double* dX = dalloc(c, (size_t)n * 3);
   double* dU = dalloc(c, (size_t)n * 3);
   if (!dX || !dU) return fail(c, WSI_ERR_OOM, "out of device memory");
   int rc = copy_in(c, c->vel_half, vel, c->nvel);
   if (!rc) rc = copy_in(c, dX, X, (size_t)n * 3);
   if (rc) return rc;
-  const double* vh[3];
-  vel_parts(c, (const double*)c->vel_half, vh);
-  launch_ib_interp(c->g, vh, dX, n, dU, c->st);
+  launch_marker_bins(c->g, dX, n, c->bins, c->st);
+  launch_ib_interp(c->g, c->vel_half, dX, n, c->bins, dU, c->st);
+  launch_marker_bins_clear(n, c->bins, c->st);
   rc = copy_out(c, U, dU, (size_t)n * 3);
   cudaStreamSynchronize(c->st);
   // release the temporaries (last two allocations)
@@ -1461,7 +1492,8 @@ int wsi_spread(wsi_ctx* c, const double* F, const double* X, int n, double dV, d
   if (valid_ctx(c)) return WSI_ERR_INVALID_ARG;
   // the work arrays first: the two staging buffers below must stay the last
   // two allocations (they are released at the end)
-  if (!ensure_spread_work(c)) return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
+  if (!ensure_spread_work(c) || !ensure_bins(c, std::max(n, 1)))
+    return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
   double* dX = dalloc(c, (size_t)std::max(n, 1) * 3);
   double* dF = dalloc(c, (size_t)std::max(n, 1) * 3);
   if (!dX || !dF) return fail(c, WSI_ERR_OOM, "out of device memory");
@@ -1472,13 +1504,16 @@ int wsi_spread(wsi_ctx* c, const double* F, const double* X, int n, double dV, d
   }
   if (!rc) {
     cudaMemsetAsync(c->vel_half, 0, c->nvel * sizeof(double), c->st);
-    double* vq[3];
-    vel_parts(c, c->vel_half, vq);
-    double mm[6];
-    launch_marker_box(dX, n, c->mbox, c->sw.part, c->st);
-    cudaMemcpyAsync(mm, c->mbox, sizeof(mm), cudaMemcpyDeviceToHost, c->st);
-    cudaStreamSynchronize(c->st);
-    launch_ib_spread(c->g, dF, dX, n, dV, vq, c->sw, spread_box(c->g, mm), c->st);
+    if (n > 0) {
+      double mm[6];
+      launch_marker_mean_box(dX, n, c->red, c->mbox, c->red + 8, c->st);
+      launch_marker_bins(c->g, dX, n, c->bins, c->st);
+      launch_force_max(dF, n, c->bins, c->st);
+      cudaMemcpyAsync(mm, c->mbox, sizeof(mm), cudaMemcpyDeviceToHost, c->st);
+      cudaStreamSynchronize(c->st);
+      launch_ib_spread(c->g, dF, dX, n, dV, c->vel_half, c->sacc, c->bins, spread_box(c->g, mm), c->st);
+      launch_marker_bins_clear(n, c->bins, c->st);
+    }
     rc = copy_out(c, vel, c->vel_half, c->nvel);
   }
   cudaStreamSynchronize(c->st);

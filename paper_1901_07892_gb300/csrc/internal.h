@@ -325,32 +325,44 @@ template <typename T>
 void precond_coarse_part(Precond<T>& P, const Opts& o, int l, cudaStream_t st);
 
 // ---------------------------------------------------------------- dlm.cu
-void launch_ib_interp(const GridDev& g, const double* const vel[3], const double* X, int n, double* U,
-                      cudaStream_t st);
-// deterministic spreading (fixed-point integer sums): work arrays that stay
-// zero between calls, and the box of cells the markers' taps can reach
-struct SpreadWork {
-  unsigned long long* acc = nullptr;  // one per face of the packed velocity
-  int* cnt = nullptr;                 // one per cell
-  int* qexp = nullptr;                // quantum exponent of the current call
-  double* part = nullptr;             // reduction partials (6 x 152 doubles)
+// Markers binned by the cell that holds them: sorted order (perm), the list of
+// non-empty cells (cell, first place in perm, count) and the irregular markers
+// (outside the grid or not finite), with device counters.  cnt (one per cell)
+// is zero between uses.
+enum { BIN_CELLS = 0, BIN_TOTAL = 1, BIN_IRR = 2, BIN_CMAX = 3 };
+static constexpr int BIN_CTR_BYTES = 4 * 4 + 8;  // the four counters and fmx
+struct MarkerBins {
+  int cap = 0;  // markers the arrays hold
+  int *cnt = nullptr, *cellof = nullptr, *rank = nullptr, *perm = nullptr, *lcell = nullptr, *lstart = nullptr,
+      *lcnt = nullptr, *irr = nullptr, *ctr = nullptr;
+  unsigned long long* fmx = nullptr;  // bits of max|F|, zeroed with the counters
 };
+void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBins& b, cudaStream_t st);
+void launch_marker_bins_clear(int n, const MarkerBins& b, cudaStream_t st);
+// vel: packed velocity vector
+void launch_ib_interp(const GridDev& g, const double* vel, const double* X, int n, const MarkerBins& b,
+                      double* U, cudaStream_t st);
+// box of cells the markers' taps can reach, from the marker extent
+// mm = (min x, y, z, max x, y, z)
 struct SpreadBox {
   int lo[3], hi[3];  // cells, inclusive
 };
-// box from the marker extent mm = (min x, y, z, max x, y, z)
 SpreadBox spread_box(const GridDev& g, const double mm[6]);
-void launch_marker_box(const double* X, int n, double* out6, double* scratch, cudaStream_t st);
-void launch_ib_spread(const GridDev& g, const double* F, const double* X, int n, double dV, double* const vel[3],
-                      const SpreadWork& w, const SpreadBox& b, cudaStream_t st);
-// rigid sums: out[0..2] sum U, [3..5] sum R x U, [6..11] sum of R.R I - R (x) R (xx,yy,zz,xy,xz,yz),
-// [12..14] sum X; R relative to xc_dev
+// mean of the markers and (box6 not null) their extent
+void launch_marker_mean_box(const double* X, int n, double* xc_dev, double* box6, double* scratch, cudaStream_t st);
+// max|F| into b.fmx
+void launch_force_max(const double* F, int n, const MarkerBins& b, cudaStream_t st);
+// deterministic spreading (fixed-point integer sums) of the binned markers;
+// acc: one integer per face of the packed velocity, zero between calls
+void launch_ib_spread(const GridDev& g, const double* F, const double* X, int n, double dV, double* vel,
+                      unsigned long long* acc, const MarkerBins& b, const SpreadBox& box, cudaStream_t st);
+// rigid sums: out[0..2] sum U; with xc_dev also [3..5] sum R x U, [6..11] sum of
+// R.R I - R (x) R (xx,yy,zz,xy,xz,yz), R relative to xc_dev
 void launch_rigid_sums(const double* X, const double* U, int n, const double* xc_dev, double* out, double* scratch,
                        cudaStream_t st);
-void launch_marker_mean(const double* X, int n, double* xc_dev, double* scratch, cudaStream_t st);
-// F = U_r + W_r x (X - xc) - U   (body velocity minus interpolated); Ub also stored
+// Ub = U_r + W_r x (X - xc), F = Ub - U, max|F| into b.fmx
 void launch_body_velocity(const double* X, const double* U, int n, const double* rigid_dev, const double* xc_dev,
-                          double* Ub, double* F, cudaStream_t st);
+                          double* Ub, double* F, const MarkerBins& b, cudaStream_t st);
 // X = X^n + dt (U_b^{n+1} + U_b^n) / 2; *flag |= 1 when a marker leaves the box
 // (by more than half a cell) or is not finite (flag may be null)
 void launch_marker_update(const GridDev& g, const double* Xn, const double* Ub_new, const double* Ub_old, int n,
