@@ -176,9 +176,10 @@ bool ensure_bins(wsi_ctx* c, int n) {
   MarkerBins& b = c->bins;
   if (!b.cnt) {
     b.cnt = (int*)dalloc(c, c->ncell / 2 + 1);
+    b.bcnt = (int*)dalloc(c, c->ncell / 2 + 1);
     b.ctr = (int*)dalloc(c, BIN_CTR_BYTES / 8);
     b.fmx = (unsigned long long*)(b.ctr + 4);
-    if (!b.cnt || !b.ctr) {
+    if (!b.cnt || !b.bcnt || !b.ctr) {
       b.cnt = nullptr;
       return false;
     }

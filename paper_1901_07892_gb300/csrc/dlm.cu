@@ -155,11 +155,10 @@ __device__ __forceinline__ long long fixed_of(float f, int E) {
   return (long long)((unsigned long long)(long long)((int)u < 0 ? -r : r) << max(sh, 0));
 }
 
-// E of the current call from the largest cell count, the irregular markers and
-// the bits of max|F|
+// E of the current call from the largest cell count and the bits of max|F|
 __device__ __forceinline__ int spread_exponent(const int* __restrict__ ctr, const unsigned long long* __restrict__ fmx,
                                                double scale) {
-  const double c = (double)(ctr[BIN_CMAX] + ctr[BIN_IRR]), f = __longlong_as_double((long long)fmx[0]);
+  const double c = (double)ctr[BIN_CMAX], f = __longlong_as_double((long long)fmx[0]);
   const double B = 128.0 * c * f * scale;
   int e = 0;
   const bool pos = B > 0.0 && B < 1e300;
@@ -208,13 +207,23 @@ __global__ void __launch_bounds__(128) k_spread_list(GridDev g, const double* __
 }
 
 // ------------------------------------------------------------- binning by cell
+// the cell of a marker for the quantum's bound: float64, clamped into the grid
+__device__ __forceinline__ int bound_cell(const GridDev& g, const double* __restrict__ X, int m) {
+  int c[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) c[d] = clampi((int)floor(X[3 * m + d] * g.ih[d]), 0, g.n[d] - 1);
+  return (int)fidx(g, 3, c[0], c[1], c[2]);
+}
+
 // Pass 1: cell of each marker and its rank in that cell (the arrival order of
 // an atomic; results don't depend on it: interpolation treats each marker by
-// itself, spreading adds integers)
-__global__ void __launch_bounds__(256) k_bin_count(GridDev g, const double* __restrict__ X, int n, int* cnt,
+// itself, spreading adds integers).  The cell follows the taps' double-float
+// positions; bcnt counts by the float64 ones, which may differ on a cell face.
+__global__ void __launch_bounds__(256) k_bin_count(GridDev g, const double* __restrict__ X, int n, int* cnt, int* bcnt,
                                                    int* cellof, int* rank, int* irr, int* ctr) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
+  atomicAdd(&bcnt[bound_cell(g, X, m)], 1);
   int c[3];
   bool in = true;
 #pragma unroll
@@ -235,15 +244,17 @@ __global__ void __launch_bounds__(256) k_bin_count(GridDev g, const double* __re
 }
 
 // Pass 2: the first marker of each cell takes a range of the sorted order and a
-// place in the cell list (two atomics per block); cnt then holds the range's start
-__global__ void __launch_bounds__(256) k_bin_alloc(int n, const int* __restrict__ cellof, const int* __restrict__ rank,
-                                                   int* cnt, int* lcell, int* lstart, int* lcnt, int* ctr) {
+// place in the cell list (two atomics per block); cnt then holds the range's
+// start.  Also the largest of the bound's counts.
+__global__ void __launch_bounds__(256) k_bin_alloc(GridDev g, const double* __restrict__ X, int n,
+                                                   const int* __restrict__ bcnt, const int* __restrict__ cellof,
+                                                   const int* __restrict__ rank, int* cnt, int* lcell, int* lstart, int* lcnt, int* ctr) {
   __shared__ int sm[8], sc[8], sx[8], base[2];
   const int m = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cell = m < n ? cellof[m] : -1;
   const bool first = cell >= 0 && rank[m] == 0;
   const int k = first ? cnt[cell] : 0;
-  int a = k, b = first ? 1 : 0, x = k;  // inclusive scans of markers and cells, largest count
+  int a = k, b = first ? 1 : 0, x = m < n ? bcnt[bound_cell(g, X, m)] : 0;  // inclusive scans of markers and cells
   for (int o = 1; o < 32; o <<= 1) {
     const int ua = __shfl_up_sync(0xffffffffu, a, o), ub = __shfl_up_sync(0xffffffffu, b, o);
     if (lane >= o) {
@@ -282,11 +293,13 @@ __global__ void __launch_bounds__(256) k_bin_alloc(int n, const int* __restrict_
   }
 }
 
-// Pass 3: markers in cell order
-__global__ void __launch_bounds__(256) k_bin_fill(int n, const int* __restrict__ cellof, const int* __restrict__ rank,
-                                                  const int* __restrict__ cnt, int* perm) {
+// Pass 3: markers in cell order; the bound's counts back to zero
+__global__ void __launch_bounds__(256) k_bin_fill(GridDev g, const double* __restrict__ X, int n,
+                                                  const int* __restrict__ cellof, const int* __restrict__ rank,
+                                                  const int* __restrict__ cnt, int* bcnt, int* perm) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
+  bcnt[bound_cell(g, X, m)] = 0;
   const int cell = cellof[m];
   if (cell >= 0) perm[cnt[cell] + rank[m]] = m;
 }
@@ -295,9 +308,10 @@ void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBi
   if (n <= 0) return;
   cudaMemsetAsync(b.ctr, 0, BIN_CTR_BYTES, st);
   const int blocks = cdiv(n, 256);
-  { k_bin_count<<<blocks, 256, 0, st>>>(g, X, n, b.cnt, b.cellof, b.rank, b.irr, b.ctr); WSI_COUNT(); }
-  { k_bin_alloc<<<blocks, 256, 0, st>>>(n, b.cellof, b.rank, b.cnt, b.lcell, b.lstart, b.lcnt, b.ctr); WSI_COUNT(); }
-  { k_bin_fill<<<blocks, 256, 0, st>>>(n, b.cellof, b.rank, b.cnt, b.perm); WSI_COUNT(); }
+  { k_bin_count<<<blocks, 256, 0, st>>>(g, X, n, b.cnt, b.bcnt, b.cellof, b.rank, b.irr, b.ctr); WSI_COUNT(); }
+  { k_bin_alloc<<<blocks, 256, 0, st>>>(g, X, n, b.bcnt, b.cellof, b.rank, b.cnt, b.lcell, b.lstart, b.lcnt,
+                                           b.ctr); WSI_COUNT(); }
+  { k_bin_fill<<<blocks, 256, 0, st>>>(g, X, n, b.cellof, b.rank, b.cnt, b.bcnt, b.perm); WSI_COUNT(); }
 }
 
 // counts of the listed cells back to zero for the next binning

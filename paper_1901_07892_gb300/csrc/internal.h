@@ -327,13 +327,13 @@ void precond_coarse_part(Precond<T>& P, const Opts& o, int l, cudaStream_t st);
 // ---------------------------------------------------------------- dlm.cu
 // Markers binned by the cell that holds them: sorted order (perm), the list of
 // non-empty cells (cell, first place in perm, count) and the irregular markers
-// (outside the grid or not finite), with device counters.  cnt (one per cell)
-// is zero between uses.
+// (outside the grid or not finite), with device counters.  cnt and bcnt (one per
+// cell) are zero between uses.
 enum { BIN_CELLS = 0, BIN_TOTAL = 1, BIN_IRR = 2, BIN_CMAX = 3 };
 static constexpr int BIN_CTR_BYTES = 4 * 4 + 8;  // the four counters and fmx
 struct MarkerBins {
   int cap = 0;  // markers the arrays hold
-  int *cnt = nullptr, *cellof = nullptr, *rank = nullptr, *perm = nullptr, *lcell = nullptr, *lstart = nullptr,
+  int *cnt = nullptr, *bcnt = nullptr, *cellof = nullptr, *rank = nullptr, *perm = nullptr, *lcell = nullptr, *lstart = nullptr,
       *lcnt = nullptr, *irr = nullptr, *ctr = nullptr;
   unsigned long long* fmx = nullptr;  // bits of max|F|, zeroed with the counters
 };
