@@ -1925,14 +1925,12 @@ int wsi_pressure_solve(wsi_ctx* c, const double* y, double* x, double rtol, int 
     if (c->mixed()) {
       MGLevel<float>& L0 = c->P32.lev[0];
       launch_lincomb_to_f32(n, 1.0 / rn, r, 0.0, nullptr, 0.0, nullptr, L0.b, st);
-      cudaMemsetAsync(L0.x, 0, n * sizeof(float), st);
-      precond_vcycle<float>(c->P32, c->opts, st);
+      precond_vcycle<float>(c->P32, c->opts, true, st);
       launch_lincomb_mix(n, 1.0, xv, rn, L0.x, 0.0, L0.x, xv, st);
     } else {
       MGLevel<double>& L0 = c->P64.lev[0];
       cudaMemcpyAsync(L0.b, r, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
-      cudaMemsetAsync(L0.x, 0, n * sizeof(double), st);
-      precond_vcycle<double>(c->P64, c->opts, st);
+      precond_vcycle<double>(c->P64, c->opts, true, st);
       launch_lincomb(n, 1.0, xv, 1.0, L0.x, 0.0, nullptr, xv, st);
     }
     last_learned = use;

@@ -238,6 +238,7 @@ struct Precond {
   std::vector<MGLevel<T>> lev;
   double* coarse_inv = nullptr;  // dense float64 inverse of the regularised coarsest operator
   int ncoarse = 0;
+  int coarse_ctas = 8;           // blocks of the fused lower cycle's cluster
   // fine-level viscous coefficients in T
   T* rho_face[3] = {nullptr, nullptr, nullptr};
   T* mu_cc = nullptr;
@@ -317,9 +318,10 @@ const double* learned_guess_loss(const Precond<float>& P);
 // lev[from].x carried to level 0: each finer x set to the prolongation
 template <typename T>
 void precond_prolong_chain(Precond<T>& P, int from, cudaStream_t st);
-// one V-cycle on level 0 of the hierarchy (x, b of level 0)
+// one V-cycle on level 0 of the hierarchy (x, b of level 0; zero: from x = 0,
+// whatever x holds)
 template <typename T>
-void precond_vcycle(Precond<T>& P, const Opts& o, cudaStream_t st);
+void precond_vcycle(Precond<T>& P, const Opts& o, bool zero, cudaStream_t st);
 // everything of a V-cycle on level l but the post-smoothing (x, b of level l)
 template <typename T>
 void precond_coarse_part(Precond<T>& P, const Opts& o, int l, cudaStream_t st);

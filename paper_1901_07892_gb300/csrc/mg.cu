@@ -32,6 +32,20 @@ static constexpr int BX = 32, BY = 8;
 static inline dim3 grid3(int nx, int ny, int nz) { return dim3(cdiv(nx, BX), cdiv(ny, BY), nz); }
 
 template <typename T>
+struct CoarseCycle;
+template <typename T, int NT>
+__global__ void k_coarse_cycle(const __grid_constant__ CoarseCycle<T> c);
+// cells of a level that one block works on in shared memory, and of one that the
+// fused lower cycle takes at all; float64 updates are bound by the narrow pipe of
+// the SMs that take part, so fewer of them go to one block or one cluster
+template <typename T>
+static constexpr int coarse_smem_cells() { return 512; }
+template <typename T>
+static constexpr int coarse_max_cells() { return sizeof(T) == 4 ? 65536 : 4096; }
+template <typename T>
+static constexpr int coarse_threads() { return 512; }
+
+template <typename T>
 static T* dalloc(std::vector<void*>& allocs, size_t n, std::string& err) {
   void* p = nullptr;
   if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
@@ -133,6 +147,29 @@ int precond_alloc(Precond<T>& P, const GridDev& g0, std::string& err) {
   for (int e = 0; e < 3; ++e) P.mu_e[e] = dalloc<T>(P.allocs, esize(g0, e), err);
   P.rp = dalloc<T>(P.allocs, fsize(g0, 3), err);
   P.y = dalloc<T>(P.allocs, fsize(g0, 3), err);
+  // the fused lower cycle's shared memory: x and b of its small levels (each at
+  // most half the cells of the one above) and the dense solve's vector
+  cudaFuncSetAttribute(k_coarse_cycle<T, coarse_threads<T>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       4 * std::max(coarse_smem_cells<T>(), 1024) * (int)sizeof(T) + 1024 * 8);
+  P.coarse_ctas = 8;
+  if (cudaFuncSetAttribute(k_coarse_cycle<T, coarse_threads<T>()>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+      cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(coarse_threads<T>());
+    cfg.dynamicSmemBytes = 4 * std::max(coarse_smem_cells<T>(), 1024) * (int)sizeof(T) + 1024 * 8;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 16;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int ncl = 0;
+    if (cudaOccupancyMaxActiveClusters(&ncl, k_coarse_cycle<T, coarse_threads<T>()>, &cfg) == cudaSuccess && ncl > 0)
+      P.coarse_ctas = 16;
+  }
+  cudaGetLastError();
   P.dscratch = dalloc<double>(P.allocs, 4096, err);
   P.dsum = dalloc<double>(P.allocs, 8, err);
   if (!P.coarse_inv || !P.mu_cc || !P.rp || !P.y || !P.dscratch || !P.dsum) return WSI_ERR_OOM;
@@ -433,70 +470,79 @@ int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, cud
 // ------------------------------------------------------------ V-cycle kernels
 static inline dim3 grid_rb(const GridDev& g) { return dim3(cdiv(cdiv(g.n[0], 2), BX), cdiv(g.n[1], BY), g.n[2]); }
 
-// one colour of a red-black Gauss-Seidel sweep: thread t of a row owns the
-// t-th cell of that colour, i = 2t + ((j + k + color) & 1)
+// The pressure operator of one level as the smoothing kernels use it
 template <typename T>
-__global__ void k_rbgs_p(GridDev g, const T* __restrict__ bx, const T* __restrict__ by, const T* __restrict__ bz,
-                         T* x, const T* __restrict__ b, int color) {
-  const int j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + color) & 1);
-  if (i >= g.n[0] || j >= g.n[1]) return;
-  size_t id = fidx(g, 3, i, j, k);
-  T ihx2 = ginv2<T>(g, 0), ihy2 = ginv2<T>(g, 1), ihz2 = ginv2<T>(g, 2);
-  T s = T(0), d = T(0);
-  if (i + 1 < g.n[0]) { T c = bx[fidx(g, 0, i + 1, j, k)] * ihx2; s += c * x[id + 1]; d += c; }
-  if (i > 0) { T c = bx[fidx(g, 0, i, j, k)] * ihx2; s += c * x[id - 1]; d += c; }
-  if (j + 1 < g.n[1]) { T c = by[fidx(g, 1, i, j + 1, k)] * ihy2; s += c * x[id + g.n[0]]; d += c; }
-  if (j > 0) { T c = by[fidx(g, 1, i, j, k)] * ihy2; s += c * x[id - g.n[0]]; d += c; }
-  size_t pl = (size_t)g.n[0] * g.n[1];
-  if (k + 1 < g.n[2]) { T c = bz[fidx(g, 2, i, j, k + 1)] * ihz2; s += c * x[id + pl]; d += c; }
-  else if (g.open_top) d += T(2) * bz[fidx(g, 2, i, j, k + 1)] * ihz2;  // ghost -x above the open top
-  if (k > 0) { T c = bz[fidx(g, 2, i, j, k)] * ihz2; s += c * x[id - pl]; d += c; }
-  if (d > T(0)) x[id] = (s - b[id]) / d;
-}
+struct PLevel {
+  int n[3], open_top;
+  T ih2[3];
+  const T *bx, *by, *bz, *b;
+};
 
 template <typename T>
-__device__ __forceinline__ T lap_at(const GridDev& g, const T* __restrict__ bx, const T* __restrict__ by,
-                                    const T* __restrict__ bz, const T* __restrict__ x, int i, int j, int k) {
-  size_t id = fidx(g, 3, i, j, k);
-  T xc = x[id];
-  T ihx2 = ginv2<T>(g, 0), ihy2 = ginv2<T>(g, 1), ihz2 = ginv2<T>(g, 2);
+static PLevel<T> plevel(const MGLevel<T>& L) {
+  PLevel<T> p;
+  for (int a = 0; a < 3; ++a) {
+    p.n[a] = L.g.n[a];
+    p.ih2[a] = ginv2<T>(L.g, a);
+  }
+  p.open_top = L.g.open_top;
+  p.bx = L.beta[0];
+  p.by = L.beta[1];
+  p.bz = L.beta[2];
+  p.b = L.b;
+  return p;
+}
+
+// face coefficients around cell (i, j, k); those of walls are not used
+template <typename T>
+struct Faces {
+  T xh, xl, yh, yl, zh, zl;
+};
+template <typename T>
+__device__ __forceinline__ Faces<T> load_faces(const PLevel<T>& p, int i, int j, int k) {
+  const int r = k * p.n[1] + j, ox = r * (p.n[0] + 1) + i, oy = (r + k) * p.n[0] + i, oz = r * p.n[0] + i;
+  Faces<T> f{p.bx[ox + 1], p.bx[ox], p.by[oy + p.n[0]], p.by[oy], T(0), T(0)};
+  if (k + 1 < p.n[2] || p.open_top) f.zh = p.bz[oz + p.n[0] * p.n[1]];  // (a 2-D grid reads neither)
+  if (k > 0) f.zl = p.bz[oz];
+  return f;
+}
+
+// Gauss-Seidel value of cell (i, j, k): x(di, dj, dk) returns the neighbours;
+// a cell without any face keeps x(0, 0, 0)
+template <typename T, typename X>
+__device__ __forceinline__ T gs_value(const PLevel<T>& p, const Faces<T>& f, int i, int j, int k, T b, X x) {
+  T s = T(0), d = T(0);
+  if (i + 1 < p.n[0]) { T c = f.xh * p.ih2[0]; s += c * x(1, 0, 0); d += c; }
+  if (i > 0) { T c = f.xl * p.ih2[0]; s += c * x(-1, 0, 0); d += c; }
+  if (j + 1 < p.n[1]) { T c = f.yh * p.ih2[1]; s += c * x(0, 1, 0); d += c; }
+  if (j > 0) { T c = f.yl * p.ih2[1]; s += c * x(0, -1, 0); d += c; }
+  if (k + 1 < p.n[2]) { T c = f.zh * p.ih2[2]; s += c * x(0, 0, 1); d += c; }
+  else if (p.open_top) d += T(2) * f.zh * p.ih2[2];  // ghost -x above the open top
+  if (k > 0) { T c = f.zl * p.ih2[2]; s += c * x(0, 0, -1); d += c; }
+  if (d > T(0)) return (s - b) / d;
+  return x(0, 0, 0);
+}
+
+// L x at cell (i, j, k), x as above
+template <typename T, typename X>
+__device__ __forceinline__ T lap_value(const PLevel<T>& p, const Faces<T>& f, int i, int j, int k, X x) {
+  const T xc = x(0, 0, 0);
   T s = T(0);
-  if (i + 1 < g.n[0]) s += bx[fidx(g, 0, i + 1, j, k)] * (x[id + 1] - xc) * ihx2;
-  if (i > 0) s -= bx[fidx(g, 0, i, j, k)] * (xc - x[id - 1]) * ihx2;
-  if (j + 1 < g.n[1]) s += by[fidx(g, 1, i, j + 1, k)] * (x[id + g.n[0]] - xc) * ihy2;
-  if (j > 0) s -= by[fidx(g, 1, i, j, k)] * (xc - x[id - g.n[0]]) * ihy2;
-  size_t pl = (size_t)g.n[0] * g.n[1];
-  if (k + 1 < g.n[2]) s += bz[fidx(g, 2, i, j, k + 1)] * (x[id + pl] - xc) * ihz2;
-  else if (g.open_top) s -= T(2) * bz[fidx(g, 2, i, j, k + 1)] * xc * ihz2;
-  if (k > 0) s -= bz[fidx(g, 2, i, j, k)] * (xc - x[id - pl]) * ihz2;
+  if (i + 1 < p.n[0]) s += f.xh * (x(1, 0, 0) - xc) * p.ih2[0];
+  if (i > 0) s -= f.xl * (xc - x(-1, 0, 0)) * p.ih2[0];
+  if (j + 1 < p.n[1]) s += f.yh * (x(0, 1, 0) - xc) * p.ih2[1];
+  if (j > 0) s -= f.yl * (xc - x(0, -1, 0)) * p.ih2[1];
+  if (k + 1 < p.n[2]) s += f.zh * (x(0, 0, 1) - xc) * p.ih2[2];
+  else if (p.open_top) s -= T(2) * f.zh * xc * p.ih2[2];
+  if (k > 0) s -= f.zl * (xc - x(0, 0, -1)) * p.ih2[2];
   return s;
 }
 
-// coarse b = mean over children of (b - L x) on the fine grid
-template <typename T>
-__global__ void k_restrict_res(GridDev gf, GridDev gc, int r0, int r1, int r2, const T* __restrict__ bx,
-                               const T* __restrict__ by, const T* __restrict__ bz, const T* __restrict__ x,
-                               const T* __restrict__ b, T* bcoarse) {
-  int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y, K = blockIdx.z;
-  if (I >= gc.n[0] || J >= gc.n[1]) return;
-  T s = T(0);
-  for (int c = 0; c < r2; ++c)
-    for (int bb = 0; bb < r1; ++bb)
-      for (int a = 0; a < r0; ++a) {
-        int i = I * r0 + a, j = J * r1 + bb, k = K * r2 + c;
-        s += b[fidx(gf, 3, i, j, k)] - lap_at<T>(gf, bx, by, bz, x, i, j, k);
-      }
-  bcoarse[fidx(gc, 3, I, J, K)] = s / T(r0 * r1 * r2);
-}
-
-// x_fine += P x_coarse (linear in cell centres along coarsened axes)
-template <typename T>
-__global__ void k_prolong_add(GridDev gf, GridDev gc, int r0, int r1, int r2, const T* __restrict__ xc, T* xf) {
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= gf.n[0] || j >= gf.n[1]) return;
-  int r[3] = {r0, r1, r2};
-  int f3[3] = {i, j, k};
+// prolongation (linear in cell centres along coarsened axes) at fine cell
+// (i, j, k): xc(I, J, K) returns the coarse values; m: the coarse extents
+template <typename T, typename X>
+__device__ __forceinline__ T prolong_value(const int r[3], const int m[3], int i, int j, int k, X xc) {
+  const int f3[3] = {i, j, k};
   int c0[3], c1[3];
   T w0[3];
 #pragma unroll
@@ -504,7 +550,7 @@ __global__ void k_prolong_add(GridDev gf, GridDev gc, int r0, int r1, int r2, co
     if (r[a] == 2) {
       c0[a] = f3[a] >> 1;
       int nb = (f3[a] & 1) ? c0[a] + 1 : c0[a] - 1;
-      c1[a] = clampi(nb, 0, gc.n[a] - 1);
+      c1[a] = clampi(nb, 0, m[a] - 1);
       w0[a] = T(0.75);
     } else {
       c0[a] = f3[a];
@@ -525,9 +571,223 @@ __global__ void k_prolong_add(GridDev gf, GridDev gc, int r0, int r1, int r2, co
         T w = wx * wy * wz;
         if (w == T(0)) continue;
         int a = cx ? c1[0] : c0[0], b = cy ? c1[1] : c0[1], c = cz ? c1[2] : c0[2];
-        s += w * xc[fidx(gc, 3, a, b, c)];
+        s += w * xc(a, b, c);
       }
-  xf[fidx(gf, 3, i, j, k)] += s;
+  return s;
+}
+
+// one colour of a red-black Gauss-Seidel sweep: thread t of a row owns the
+// t-th cell of that colour, i = 2t + ((j + k + color) & 1)
+template <typename T>
+__global__ void k_rbgs_p(PLevel<T> p, T* x, int color) {
+  const int j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + color) & 1);
+  if (i >= p.n[0] || j >= p.n[1]) return;
+  const int id = (k * p.n[1] + j) * p.n[0] + i, pl = p.n[0] * p.n[1];
+  x[id] = gs_value<T>(p, load_faces<T>(p, i, j, k), i, j, k, p.b[id],
+                      [&](int a, int b, int c) { return x[id + a + b * p.n[0] + c * pl]; });
+}
+
+// Four neighbouring cells at a time (rows of a multiple of four cells, so that
+// every row of a cell or y/z-face array starts on a 16-byte boundary; x-face
+// rows have one element more and are read one by one)
+template <typename T>
+struct Quad {
+  T v[4];
+};
+template <typename T>
+__device__ __forceinline__ Quad<T> load4(const T* a) {
+  Quad<T> q;
+  if constexpr (sizeof(T) == 4) {
+    const float4 f = *reinterpret_cast<const float4*>(a);
+    q.v[0] = f.x, q.v[1] = f.y, q.v[2] = f.z, q.v[3] = f.w;
+  } else {
+    const double2 f = reinterpret_cast<const double2*>(a)[0], h = reinterpret_cast<const double2*>(a)[1];
+    q.v[0] = f.x, q.v[1] = f.y, q.v[2] = h.x, q.v[3] = h.y;
+  }
+  return q;
+}
+template <typename T>
+__device__ __forceinline__ void store4(T* a, const Quad<T>& q) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(a) = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]);
+  } else {
+    reinterpret_cast<double2*>(a)[0] = make_double2(q.v[0], q.v[1]);
+    reinterpret_cast<double2*>(a)[1] = make_double2(q.v[2], q.v[3]);
+  }
+}
+
+// One colour of a red-black sweep, four cells (two of the colour) per thread:
+// 15 loads for two updates instead of 28, and whole sectors written (the other
+// colour's values go back as they were read).  ZERO: x is zero on entry and not
+// read.  HBM-bound: x, b and the three coefficient arrays stream once per half
+// sweep, 24 bytes per cell; at 256^3 58.6 us, 6.9 TB/s (one cell per
+// thread, 64-bit indices: 98 us).  float32 only: in float64 the pipe bounds the
+// update and two updates in a row per thread cost 5 % more.
+template <typename T, bool ZERO>
+__global__ void __launch_bounds__(256) k_rbgs_p4(PLevel<T> p, T* x, int color) {
+  const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nq = nx >> 2;
+  const int t = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
+  const int j = t / nq;
+  if (j >= ny) return;
+  const int i0 = 4 * (t - j * nq), pl = nx * ny;
+  const int r = k * ny + j, id = r * nx + i0, oy = id + k * nx, ox = id + r;
+  const int q = (j + k + color) & 1;  // cells i0 + q and i0 + q + 2
+  const Quad<T> b = load4(p.b + id);
+  Quad<T> xc, xyl, xyh, xzl, xzh, yl, yh, zl, zh;
+  T xe = T(0), fx[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) fx[a] = p.bx[ox + q + a];
+  yl = load4(p.by + oy);
+  yh = load4(p.by + oy + nx);
+  zl = load4(p.bz + id);
+  zh = load4(p.bz + id + pl);
+  if (!ZERO) {
+    xc = load4(x + id);
+    if (j > 0) xyl = load4(x + id - nx);
+    if (j + 1 < ny) xyh = load4(x + id + nx);
+    if (k > 0) xzl = load4(x + id - pl);
+    if (k + 1 < nz) xzh = load4(x + id + pl);
+    if (q ? i0 + 4 < nx : i0 > 0) xe = q ? x[id + 4] : x[id - 1];
+  } else {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) xc.v[a] = T(0);
+  }
+  auto update = [&](auto QC) {
+    constexpr int Q = decltype(QC)::value;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int m = Q + 2 * h;  // place in the quad
+      const Faces<T> f{fx[2 * h + 1], fx[2 * h], yh.v[m], yl.v[m], zh.v[m], zl.v[m]};
+      xc.v[m] = gs_value<T>(p, f, i0 + m, j, k, b.v[m], [&](int a, int c, int d) {
+        if (ZERO) return T(0);
+        if (a == 1) return m == 3 ? xe : xc.v[m < 3 ? m + 1 : 3];
+        if (a == -1) return m == 0 ? xe : xc.v[m > 0 ? m - 1 : 0];
+        if (c == 1) return xyh.v[m];
+        if (c == -1) return xyl.v[m];
+        if (d == 1) return xzh.v[m];
+        if (d == -1) return xzl.v[m];
+        return xc.v[m];
+      });
+    }
+  };
+  if (q) update(std::integral_constant<int, 1>{});
+  else update(std::integral_constant<int, 0>{});
+  store4(x + id, xc);
+}
+
+// coarse b = mean over children of (b - L x) on the fine grid
+template <typename T>
+__global__ void k_restrict_res(PLevel<T> p, int m0, int m1, int r0, int r1, int r2, const T* __restrict__ x,
+                               T* bcoarse) {
+  int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y, K = blockIdx.z;
+  if (I >= m0 || J >= m1) return;
+  const int pl = p.n[0] * p.n[1];
+  T s = T(0);
+  for (int c = 0; c < r2; ++c)
+    for (int bb = 0; bb < r1; ++bb)
+      for (int a = 0; a < r0; ++a) {
+        const int i = I * r0 + a, j = J * r1 + bb, k = K * r2 + c, id = (k * p.n[1] + j) * p.n[0] + i;
+        s += p.b[id] - lap_value<T>(p, load_faces<T>(p, i, j, k), i, j, k,
+                                    [&](int da, int db, int dc) { return x[id + da + db * p.n[0] + dc * pl]; });
+      }
+  bcoarse[(K * m1 + J) * m0 + I] = s / T(r0 * r1 * r2);
+}
+
+// x_fine += P x_coarse
+template <typename T>
+__global__ void k_prolong_add(GridDev gf, GridDev gc, int r0, int r1, int r2, const T* __restrict__ xc, T* xf) {
+  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  if (i >= gf.n[0] || j >= gf.n[1]) return;
+  const int r[3] = {r0, r1, r2};
+  xf[fidx(gf, 3, i, j, k)] +=
+      prolong_value<T>(r, gc.n, i, j, k, [&](int a, int b, int c) { return xc[fidx(gc, 3, a, b, c)]; });
+}
+
+// The same with every axis coarsened, two coarse cells (a fine quad of 2 x 2
+// rows) per thread: 56 loads for 16 fine cells instead of 224 (84 -> 56 us at
+// 256^3).
+template <typename T>
+__global__ void __launch_bounds__(128) k_restrict_res4(PLevel<T> p, const T* __restrict__ x, T* bcoarse) {
+  const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nq = nx >> 2, m1 = ny >> 1;
+  const int t = blockIdx.x * 128 + threadIdx.x, K = blockIdx.y;
+  const int J = t / nq;
+  if (J >= m1) return;
+  const int i0 = 4 * (t - J * nq), j0 = 2 * J, k0 = 2 * K, pl = nx * ny;
+  T s[2] = {T(0), T(0)};
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int k = k0 + c;
+    Quad<T> xr[4];  // rows j0 - 1 .. j0 + 2
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int j = j0 - 1 + a;
+      if (j >= 0 && j < ny) xr[a] = load4(x + (k * ny + j) * nx + i0);
+    }
+    Quad<T> fy[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) fy[a] = load4(p.by + (k * (ny + 1) + j0 + a) * nx + i0);
+#pragma unroll
+    for (int bb = 0; bb < 2; ++bb) {
+      const int j = j0 + bb, r = k * ny + j, id = r * nx + i0;
+      const Quad<T> b = load4(p.b + id), zl = load4(p.bz + id), zh = load4(p.bz + id + pl);
+      Quad<T> xzl, xzh;
+      if (k > 0) xzl = load4(x + id - pl);
+      if (k + 1 < nz) xzh = load4(x + id + pl);
+      const T xm = i0 > 0 ? x[id - 1] : T(0), xp = i0 + 4 < nx ? x[id + 4] : T(0);
+      T fx[5];
+#pragma unroll
+      for (int a = 0; a < 5; ++a) fx[a] = p.bx[id + r + a];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const Faces<T> f{fx[m + 1], fx[m], fy[bb + 1].v[m], fy[bb].v[m], zh.v[m], zl.v[m]};
+        s[m >> 1] += b.v[m] - lap_value<T>(p, f, i0 + m, j, k, [&](int da, int db, int dc) {
+          if (da == 1) return m == 3 ? xp : xr[bb + 1].v[m < 3 ? m + 1 : 3];
+          if (da == -1) return m == 0 ? xm : xr[bb + 1].v[m > 0 ? m - 1 : 0];
+          if (db == 1) return xr[bb + 2].v[m];
+          if (db == -1) return xr[bb].v[m];
+          if (dc == 1) return xzh.v[m];
+          if (dc == -1) return xzl.v[m];
+          return xr[bb + 1].v[m];
+        });
+      }
+    }
+  }
+  const int o = (K * m1 + J) * (nx >> 1) + (i0 >> 1);
+  bcoarse[o] = s[0] / T(8);
+  bcoarse[o + 1] = s[1] / T(8);
+}
+
+// x_fine += P x_coarse with every axis coarsened, four fine cells per thread
+// (16 coarse loads instead of 32; 149 -> 44 us per cycle over all levels at 256^3)
+template <typename T>
+__global__ void __launch_bounds__(256) k_prolong_add4(int nx, int ny, int m2, const T* __restrict__ xc, T* xf) {
+  const int nq = nx >> 2, t = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y, j = t / nq;
+  if (j >= ny) return;
+  const int i0 = 4 * (t - j * nq), mx = nx >> 1, my = ny >> 1;
+  const int I0 = i0 >> 1, J0 = j >> 1, K0 = k >> 1;
+  const int J1 = clampi((j & 1) ? J0 + 1 : J0 - 1, 0, my - 1), K1 = clampi((k & 1) ? K0 + 1 : K0 - 1, 0, m2 - 1);
+  const int Im = max(I0 - 1, 0), Ip = min(I0 + 2, mx - 1);
+  const int id = (k * ny + j) * nx + i0;
+  Quad<T> f = load4(xf + id), s;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) s.v[m] = T(0);
+#pragma unroll
+  for (int cz = 0; cz < 2; ++cz)
+#pragma unroll
+    for (int cy = 0; cy < 2; ++cy) {
+      const T* row = xc + ((cz ? K1 : K0) * my + (cy ? J1 : J0)) * mx;
+      const T a[4] = {row[Im], row[I0], row[I0 + 1], row[Ip]};
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const T wyz = (cy ? T(0.25) : T(0.75)) * (cz ? T(0.25) : T(0.75));
+        s.v[m] += T(0.75) * wyz * a[1 + (m >> 1)];
+        s.v[m] += T(0.25) * wyz * a[(m & 1) ? 2 + (m >> 1) : (m >> 1)];
+      }
+    }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) f.v[m] += s.v[m];
+  store4(xf + id, f);
 }
 
 // x = Minv (-b), one block
@@ -541,6 +801,266 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Minv, const T* 
     for (int c = 0; c < n; ++c) s += Minv[(size_t)r * n + c] * sb[c];
     x[r] = (T)s;
   }
+}
+
+// The lower part of a V-cycle in one launch: every level from the first one of
+// at most coarse_max_cells down to the coarsest, pre-smoothing, restriction, the
+// dense solve, prolongation and post-smoothing, the same operations in the same
+// order as a launch each.  Levels of more than coarse_smem_cells are worked on
+// by a cluster of sixteen blocks (eight where the device holds no more) in global memory (x and the restricted b through
+// L2, a cluster barrier between half sweeps); the smaller ones by its first
+// block with x and b in shared memory.  A launch per half sweep costs 2.5 to 4 us
+// on these levels whatever their size (11 launches per level): a cycle
+// over 40x32x48 cells 95 us instead of about 170, the levels of 32^3 and below of
+// a 256^3 cycle 67 us instead of about 95.  Bound by latency: an exchange through
+// L2 and a cluster barrier per half sweep.  Above 65536 cells the whole GPU's
+// bandwidth wins.
+static constexpr int COARSE_LEVELS = 14;
+
+// quotient by a level extent: exact for t, d <= 65536
+struct FastDiv {
+  unsigned m;
+  int d;
+  void set(int v) {
+    d = v;
+    m = v > 1 ? (unsigned)(((1ull << 32) + v - 1) / v) : 0u;
+  }
+  __device__ __forceinline__ int div(int t) const { return d > 1 ? (int)__umulhi((unsigned)t, m) : t; }
+};
+struct LevelDiv {
+  FastDiv hx, nx, ny;  // cells of one colour per row, cells per row, rows per plane
+};
+
+template <typename T>
+struct CoarseCycle {
+  PLevel<T> lev[COARSE_LEVELS];
+  T* x[COARSE_LEVELS];
+  T* b[COARSE_LEVELS];
+  int r[COARSE_LEVELS][3];
+  LevelDiv dv[COARSE_LEVELS];
+  int off[COARSE_LEVELS];  // place of the level's x in shared memory (its b follows)
+  int nl, first;           // levels, first one in shared memory
+  int pre, post, zero, ncoarse, nb;  // nb: doubles before the levels in shared memory
+  const double* minv;
+};
+
+template <typename T>
+struct GlobalX {  // written by other blocks: through L2
+  T* p;
+  __device__ __forceinline__ T get(int i) const { return __ldcg(p + i); }
+  __device__ __forceinline__ void set(int i, T v) const { __stcg(p + i, v); }
+};
+template <typename T>
+struct SharedX {
+  T* p;
+  __device__ __forceinline__ T get(int i) const { return p[i]; }
+  __device__ __forceinline__ void set(int i, T v) const { p[i] = v; }
+};
+
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// x around a cell, loaded before any of it is used (beyond walls: the cell's
+// own value, which is not used)
+template <typename T>
+struct Around {
+  T c, xh, xl, yh, yl, zh, zl;
+  __device__ __forceinline__ T operator()(int a, int b, int d) const {
+    return a == 1 ? xh : (a == -1 ? xl : (b == 1 ? yh : (b == -1 ? yl : (d == 1 ? zh : (d == -1 ? zl : c)))));
+  }
+};
+template <typename T, typename X>
+__device__ __forceinline__ Around<T> load_around(const PLevel<T>& p, X x, int i, int j, int k, int id) {
+  const int nx = p.n[0], pl = nx * p.n[1];
+  return Around<T>{x.get(id),
+                   x.get(i + 1 < nx ? id + 1 : id),
+                   x.get(i > 0 ? id - 1 : id),
+                   x.get(j + 1 < p.n[1] ? id + nx : id),
+                   x.get(j > 0 ? id - nx : id),
+                   x.get(k + 1 < p.n[2] ? id + pl : id),
+                   x.get(k > 0 ? id - pl : id)};
+}
+
+// zero: 0 x as stored; 1 x = 0 everywhere; 2 x = 0 on this colour
+template <typename T, typename X, typename B>
+__device__ __forceinline__ void coarse_half(const PLevel<T>& p, const LevelDiv& dv, X x, B b, int color, int zero,
+                                            int t0, int nt) {
+  const int nx = p.n[0], ny = p.n[1], hx = (nx + 1) >> 1, total = hx * ny * p.n[2];
+#pragma unroll 2
+  for (int t = t0; t < total; t += nt) {
+    const int rr = dv.hx.div(t), k = dv.ny.div(rr), j = rr - k * ny;
+    const int i = 2 * (t - rr * hx) + ((j + k + color) & 1), id = rr * nx + i;
+    if (i < nx) {
+      const Faces<T> f = load_faces<T>(p, i, j, k);
+      const T bv = b.get(id);
+      Around<T> n{T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+      if (zero != 1) {
+        n = load_around<T>(p, x, i, j, k, id);
+        if (zero) n.c = T(0);
+      }
+      x.set(id, gs_value<T>(p, f, i, j, k, bv, n));
+    }
+  }
+}
+
+template <typename T, typename X, typename B, typename BC>
+__device__ __forceinline__ void coarse_restrict(const PLevel<T>& p, const int r[3], const int m[3], const LevelDiv& dm,
+                                                X x, B b, BC bc, int t0, int nt) {
+  const int nx = p.n[0], ny = p.n[1];
+  for (int t = t0; t < m[0] * m[1] * m[2]; t += nt) {
+    const int rr = dm.nx.div(t), K = dm.ny.div(rr), J = rr - K * m[1], I = t - rr * m[0];
+    T s = T(0);
+    for (int c = 0; c < r[2]; ++c)
+      for (int bb = 0; bb < r[1]; ++bb) {
+        const int i = I * r[0], j = J * r[1] + bb, k = K * r[2] + c, id = (k * ny + j) * nx + i;
+        const bool two = r[0] == 2;
+        const Faces<T> f0 = load_faces<T>(p, i, j, k);
+        const Around<T> n0 = load_around<T>(p, x, i, j, k, id);
+        const T b0 = b.get(id);
+        Faces<T> f1;
+        Around<T> n1;
+        T b1 = T(0);
+        if (two) {
+          f1 = load_faces<T>(p, i + 1, j, k);
+          n1 = load_around<T>(p, x, i + 1, j, k, id + 1);
+          b1 = b.get(id + 1);
+        }
+        s += b0 - lap_value<T>(p, f0, i, j, k, n0);
+        if (two) s += b1 - lap_value<T>(p, f1, i + 1, j, k, n1);
+      }
+    bc.set(t, s / T(r[0] * r[1] * r[2]));
+  }
+}
+
+template <typename T, typename X, typename XC>
+__device__ __forceinline__ void coarse_prolong(const PLevel<T>& p, const LevelDiv& dv, const int r[3], const int m[3],
+                                               X x, XC xc, int t0, int nt) {
+  const int nx = p.n[0], ny = p.n[1];
+  for (int t = t0; t < nx * ny * p.n[2]; t += nt) {
+    const int rr = dv.nx.div(t), k = dv.ny.div(rr), j = rr - k * ny, i = t - rr * nx;
+    x.set(t, x.get(t) + prolong_value<T>(r, m, i, j, k, [&](int a, int b, int c) { return xc.get((c * m[1] + b) * m[0] + a); }));
+  }
+}
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) k_coarse_cycle(const __grid_constant__ CoarseCycle<T> c) {
+  extern __shared__ __align__(16) double coarse_smem[];
+  T* const sm = reinterpret_cast<T*>(coarse_smem + c.nb);
+  const int tid = threadIdx.x, t0 = blockIdx.x * NT + tid, nt = gridDim.x * NT;
+  for (int l = 0; l < c.first; ++l) {
+    const GlobalX<T> x{c.x[l]}, b{c.b[l]};
+    for (int s = 0; s < c.pre; ++s)
+      for (int q = 0; q < 2; ++q) {
+        coarse_half<T>(c.lev[l], c.dv[l], x, b, q, s == 0 && (c.zero || l > 0) ? q + 1 : 0, t0, nt);
+        cluster_sync_all();
+      }
+    coarse_restrict<T>(c.lev[l], c.r[l], c.lev[l + 1].n, c.dv[l + 1], x, b, GlobalX<T>{c.b[l + 1]}, t0, nt);
+    cluster_sync_all();
+  }
+  if (blockIdx.x == 0) {
+    const int lf = c.first;
+    const int nf = c.lev[lf].n[0] * c.lev[lf].n[1] * c.lev[lf].n[2];
+    auto X = [&](int l) { return SharedX<T>{sm + c.off[l]}; };
+    auto Bs = [&](int l) { return SharedX<T>{sm + c.off[l] + c.lev[l].n[0] * c.lev[l].n[1] * c.lev[l].n[2]}; };
+    for (int t = tid; t < nf; t += NT) {
+      Bs(lf).set(t, __ldcg(c.b[lf] + t));
+      if (!c.zero && lf == 0) X(lf).set(t, __ldcg(c.x[lf] + t));
+    }
+    __syncthreads();
+    for (int l = lf; l + 1 < c.nl; ++l) {
+      for (int s = 0; s < c.pre; ++s)
+        for (int q = 0; q < 2; ++q) {
+          coarse_half<T>(c.lev[l], c.dv[l], X(l), Bs(l), q, s == 0 && (c.zero || l > 0) ? q + 1 : 0, tid, NT);
+          __syncthreads();
+        }
+      coarse_restrict<T>(c.lev[l], c.r[l], c.lev[l + 1].n, c.dv[l + 1], X(l), Bs(l), Bs(l + 1), tid, NT);
+      __syncthreads();
+    }
+    {  // x = Minv (-b)
+      const int n = c.ncoarse;
+      const SharedX<T> x = X(c.nl - 1), b = Bs(c.nl - 1);
+      for (int t = tid; t < n; t += NT) coarse_smem[t] = -(double)b.get(t);
+      __syncthreads();
+      for (int rI = tid; rI < n; rI += NT) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int q = 0; q < n; ++q) s += c.minv[(size_t)rI * n + q] * coarse_smem[q];
+        x.set(rI, (T)s);
+      }
+      __syncthreads();
+    }
+    for (int l = c.nl - 2; l >= lf; --l) {
+      coarse_prolong<T>(c.lev[l], c.dv[l], c.r[l], c.lev[l + 1].n, X(l), X(l + 1), tid, NT);
+      __syncthreads();
+      for (int s = 0; s < c.post; ++s)
+        for (int q = 1; q >= 0; --q) {
+          coarse_half<T>(c.lev[l], c.dv[l], X(l), Bs(l), q, 0, tid, NT);
+          __syncthreads();
+        }
+    }
+    for (int t = tid; t < nf; t += NT) __stcg(c.x[lf] + t, X(lf).get(t));
+  }
+  for (int l = c.first - 1; l >= 0; --l) {
+    cluster_sync_all();
+    const GlobalX<T> x{c.x[l]}, b{c.b[l]};
+    coarse_prolong<T>(c.lev[l], c.dv[l], c.r[l], c.lev[l + 1].n, x, GlobalX<T>{c.x[l + 1]}, t0, nt);
+    for (int s = 0; s < c.post; ++s)
+      for (int q = 1; q >= 0; --q) {
+        cluster_sync_all();
+        coarse_half<T>(c.lev[l], c.dv[l], x, b, q, 0, t0, nt);
+      }
+  }
+}
+
+// level l and everything below in one launch; false when the hierarchy does not
+// fit the kernel (then a launch per operation)
+template <typename T>
+static bool coarse_cycle(Precond<T>& P, const Opts& o, size_t l0, bool zero, cudaStream_t st) {
+  const size_t nl = P.lev.size() - l0;
+  if (fsize(P.lev[l0].g, 3) > (size_t)coarse_max_cells<T>() || nl > (size_t)COARSE_LEVELS) return false;
+  CoarseCycle<T> c;
+  int off = 0;
+  c.nl = (int)nl;
+  c.first = (int)nl;
+  for (size_t l = 0; l < nl; ++l) {
+    MGLevel<T>& L = P.lev[l0 + l];
+    c.lev[l] = plevel(L);
+    c.x[l] = L.x;
+    c.b[l] = L.b;
+    for (int a = 0; a < 3; ++a) c.r[l][a] = L.r[a];
+    c.dv[l].hx.set((L.g.n[0] + 1) / 2);
+    c.dv[l].nx.set(L.g.n[0]);
+    c.dv[l].ny.set(L.g.n[1]);
+    c.off[l] = off;
+    if (fsize(L.g, 3) <= (size_t)coarse_smem_cells<T>() || l + 1 == nl) {
+      c.first = std::min(c.first, (int)l);
+      off += 2 * (int)fsize(L.g, 3);
+    }
+  }
+  c.pre = o.mg_pre;
+  c.post = o.mg_post;
+  c.zero = zero ? 1 : 0;
+  c.ncoarse = P.ncoarse;
+  c.nb = (P.ncoarse + 1) & ~1;
+  c.minv = P.coarse_inv;
+  const size_t smem = c.nb * sizeof(double) + off * sizeof(T);
+  constexpr int NT = coarse_threads<T>();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(c.first > 0 ? P.coarse_ctas : 1);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cfg.gridDim.x;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_coarse_cycle<T, NT>, c);
+  WSI_COUNT();
+  return true;
 }
 
 // One pass of the Chebyshev smoother on A = -L (positive semi-definite)
@@ -585,23 +1105,36 @@ __global__ void k_cheb_finish(size_t n, const T* __restrict__ x, const T* __rest
 // cannot represent.
 static constexpr double CHEB_HI = 2.0, CHEB_LO = 0.25;
 
-// m passes of smoothing on level l: red-black Gauss-Seidel sweeps (pre: red
+// one colour of a sweep over level L (zero: x is zero, whatever it holds)
+template <typename T>
+static void half_sweep(MGLevel<T>& L, int color, bool zero, cudaStream_t st) {
+  const GridDev& g = L.g;
+  ktimer_begin(KC_RBGS_P, st);
+  if (sizeof(T) == 4 && g.n[0] % 4 == 0) {
+    const dim3 grid(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]);
+    if (zero) k_rbgs_p4<T, true><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
+    else k_rbgs_p4<T, false><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
+  } else {
+    if (zero) cudaMemsetAsync(L.x, 0, fsize(g, 3) * sizeof(T), st);
+    k_rbgs_p<T><<<grid_rb(g), dim3(BX, BY), 0, st>>>(plevel(L), L.x, color);
+  }
+  WSI_COUNT();
+  ktimer_end(KC_RBGS_P, st);
+}
+
+// m passes of smoothing on level l (zero: of x = 0, whatever x holds): red-black Gauss-Seidel sweeps (pre: red
 // then black; post: black then red) or a degree-m Chebyshev polynomial
 template <typename T>
-static void smooth(Precond<T>& P, const Opts& o, size_t l, int m, bool pre, cudaStream_t st) {
+static void smooth(Precond<T>& P, const Opts& o, size_t l, int m, bool pre, cudaStream_t st, bool zero = false) {
   MGLevel<T>& L = P.lev[l];
   const GridDev& g = L.g;
-  if (m <= 0) return;
   if (o.mg_smoother != WSI_SMOOTH_CHEBYSHEV) {
+    const int c0 = pre ? 0 : 1;
     for (int s = 0; s < m; ++s)
-      for (int q = 0; q < 2; ++q) {
-        const int c = pre ? q : 1 - q;
-        ktimer_begin(KC_RBGS_P, st);
-        { k_rbgs_p<T><<<grid_rb(g), dim3(BX, BY), 0, st>>>(g, L.beta[0], L.beta[1], L.beta[2], L.x, L.b, c); WSI_COUNT(); }
-        ktimer_end(KC_RBGS_P, st);
-      }
+      for (int q = 0; q < 2; ++q) half_sweep(L, q ^ c0, zero && s == 0 && q == 0, st);
     return;
   }
+  if (zero) cudaMemsetAsync(L.x, 0, fsize(g, 3) * sizeof(T), st);
   const double theta = 0.5 * (CHEB_HI + CHEB_LO), delta = 0.5 * (CHEB_HI - CHEB_LO), sigma = theta / delta;
   double rho_prev = 1.0 / sigma;
   T* xs[2] = {L.x, L.cx2};
@@ -628,39 +1161,53 @@ static void smooth(Precond<T>& P, const Opts& o, size_t l, int m, bool pre, cuda
 }
 
 template <typename T>
-static void vcycle(Precond<T>& P, const Opts& o, size_t l, cudaStream_t st);
+static void vcycle(Precond<T>& P, const Opts& o, size_t l, bool zero, cudaStream_t st);
 
 // pre-smoothing, residual restriction, the coarser cycle and prolongation on
-// level l (everything of a V-cycle at l but the post-smoothing)
+// level l (everything of a V-cycle at l but the post-smoothing); zero: the
+// cycle starts from x = 0, whatever x holds
 template <typename T>
-static void coarse_part(Precond<T>& P, const Opts& o, size_t l, cudaStream_t st) {
+static void coarse_part(Precond<T>& P, const Opts& o, size_t l, bool zero, cudaStream_t st) {
   MGLevel<T>& L = P.lev[l];
   const GridDev& g = L.g;
   dim3 gr = grid3(g.n[0], g.n[1], g.n[2]);
-  smooth(P, o, l, o.mg_pre, true, st);
+  smooth(P, o, l, o.mg_pre, true, st, zero);
   MGLevel<T>& Cl = P.lev[l + 1];
   const GridDev& gc = Cl.g;
   ktimer_begin(KC_RESTRICT, st);
-  { k_restrict_res<T><<<grid3(gc.n[0], gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(
-      g, gc, L.r[0], L.r[1], L.r[2], L.beta[0], L.beta[1], L.beta[2], L.x, L.b, Cl.b); WSI_COUNT(); }
+  const bool quads = sizeof(T) == 4 && g.n[0] % 4 == 0 && L.r[0] == 2 && L.r[1] == 2 && L.r[2] == 2;
+  if (quads)
+    k_restrict_res4<T><<<dim3(cdiv((long long)(g.n[0] / 4) * gc.n[1], 128), gc.n[2]), 128, 0, st>>>(plevel(L), L.x, Cl.b);
+  else
+    k_restrict_res<T><<<grid3(gc.n[0], gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(plevel(L), gc.n[0], gc.n[1], L.r[0],
+                                                                              L.r[1], L.r[2], L.x, Cl.b);
+  WSI_COUNT();
   ktimer_end(KC_RESTRICT, st);
-  cudaMemsetAsync(Cl.x, 0, fsize(gc, 3) * sizeof(T), st);
-  vcycle(P, o, l + 1, st);
+  vcycle(P, o, l + 1, true, st);
   ktimer_begin(KC_PROLONG, st);
-  { k_prolong_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, gc, L.r[0], L.r[1], L.r[2], Cl.x, L.x); WSI_COUNT(); }
+  if (quads)
+    k_prolong_add4<T><<<dim3(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]), 256, 0, st>>>(g.n[0], g.n[1], gc.n[2],
+                                                                                               Cl.x, L.x);
+  else
+    k_prolong_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, gc, L.r[0], L.r[1], L.r[2], Cl.x, L.x);
+  WSI_COUNT();
   ktimer_end(KC_PROLONG, st);
 }
 
 template <typename T>
 void precond_coarse_part(Precond<T>& P, const Opts& o, int l, cudaStream_t st) {
-  coarse_part(P, o, (size_t)l, st);
+  coarse_part(P, o, (size_t)l, false, st);
 }
 template void precond_coarse_part<float>(Precond<float>&, const Opts&, int, cudaStream_t);
 
 template <typename T>
-static void vcycle(Precond<T>& P, const Opts& o, size_t l, cudaStream_t st) {
+static void vcycle(Precond<T>& P, const Opts& o, size_t l, bool zero, cudaStream_t st) {
   MGLevel<T>& L = P.lev[l];
   const GridDev& g = L.g;
+  bool learned_below = false;  // a network works on this level or below
+  if constexpr (std::is_same<T, float>::value)
+    learned_below = P.learn.on && P.learn.ready && (size_t)P.learn.level >= l;
+  if (o.mg_smoother == WSI_SMOOTH_RBGS && !learned_below && coarse_cycle(P, o, l, zero, st)) return;
   if (l + 1 == P.lev.size()) {
     { k_coarse_solve<T><<<1, 256, P.ncoarse * sizeof(double), st>>>(P.ncoarse, P.coarse_inv, L.b, L.x); WSI_COUNT(); }
     return;
@@ -674,7 +1221,7 @@ static void vcycle(Precond<T>& P, const Opts& o, size_t l, cudaStream_t st) {
       return;
     }
   }
-  coarse_part(P, o, l, st);
+  coarse_part(P, o, l, zero, st);
   if constexpr (std::is_same<T, float>::value) {
     // learned augmentation: the network's correction of the residual left
     // by the plain coarse-grid correction
@@ -690,11 +1237,11 @@ static void vcycle(Precond<T>& P, const Opts& o, size_t l, cudaStream_t st) {
 }
 
 template <typename T>
-void precond_vcycle(Precond<T>& P, const Opts& o, cudaStream_t st) {
-  vcycle(P, o, 0, st);
+void precond_vcycle(Precond<T>& P, const Opts& o, bool zero, cudaStream_t st) {
+  vcycle(P, o, 0, zero, st);
 }
-template void precond_vcycle<double>(Precond<double>&, const Opts&, cudaStream_t);
-template void precond_vcycle<float>(Precond<float>&, const Opts&, cudaStream_t);
+template void precond_vcycle<double>(Precond<double>&, const Opts&, bool, cudaStream_t);
+template void precond_vcycle<float>(Precond<float>&, const Opts&, bool, cudaStream_t);
 
 template <typename T>
 void precond_prolong_chain(Precond<T>& P, int from, cudaStream_t st) {
@@ -893,8 +1440,7 @@ void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, co
   // phi = L^{-1} y
   MGLevel<T>& L0 = P.lev[0];
   cudaMemcpyAsync(L0.b, P.y, ncell * sizeof(T), cudaMemcpyDeviceToDevice, st);
-  cudaMemsetAsync(L0.x, 0, ncell * sizeof(T), st);
-  for (int c = 0; c < o.mg_cycles; ++c) vcycle(P, o, 0, st);
+  for (int c = 0; c < o.mg_cycles; ++c) vcycle(P, o, 0, c == 0, st);
   // velocity and pressure updates
   { k_vel_update<0, T><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[0], L0.beta[0], L0.x,
                                                                                  z + pk.off[0]); WSI_COUNT(); }
