@@ -291,18 +291,19 @@ int copy_out(wsi_ctx* c, double* dst, const double* src, size_t n) {
 }
 
 int ensure_pc(wsi_ctx* c) {
+  const bool visc = c->opts.visc_mg > 0;
   if (!c->pc_alloc) {
     // allocated on first use: grids that are only used for operator applies
     // need no multigrid hierarchy
-    int rc = c->desc.precision == WSI_PREC_MIXED ? precond_alloc<float>(c->P32, c->g, c->err)
-                                                 : precond_alloc<double>(c->P64, c->g, c->err);
+    int rc = c->desc.precision == WSI_PREC_MIXED ? precond_alloc<float>(c->P32, c->g, visc, c->err)
+                                                 : precond_alloc<double>(c->P64, c->g, visc, c->err);
     if (rc) return rc;
     c->pc_alloc = true;
   }
   if (!c->pc_dirty) return WSI_OK;
   Coef<double> cf = coef_now(c);
-  int rc = c->desc.precision == WSI_PREC_MIXED ? precond_setup<float>(c->P32, c->g, cf, c->st, c->err)
-                                               : precond_setup<double>(c->P64, c->g, cf, c->st, c->err);
+  int rc = c->desc.precision == WSI_PREC_MIXED ? precond_setup<float>(c->P32, c->g, cf, visc, c->st, c->err)
+                                               : precond_setup<double>(c->P64, c->g, cf, visc, c->st, c->err);
   if (rc == WSI_OK && c->mixed()) {
     rc = learned_alloc(c->P32, c->unet_impl, c->unet_level, c->gunet_impl, c->gunet_level, c->err);
     if (rc == WSI_OK && (c->unet_impl || c->gunet_impl))
@@ -407,8 +408,8 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
       // Classical Gram-Schmidt.  One pass gives h = V^T w together with w.w
       // (w is V_{j+1}, the last row), so ||w - V h||^2 = w.w - |h|^2 needs no
       // second pass; when that cancels by more than half (the DGKS test) the
-      // vector is orthogonalised a second time.  The final axpy also
-      // normalises.
+      // vector is orthogonalised a second time.  The final axpy, which
+      // also normalises, is left out where no iteration follows.
       const size_t o2 = (size_t)m + 2, osc = 2 * (size_t)m + 4;
       launch_mdot(V, n, j + 2, w, n, hd, red, c->st);
       cudaMemcpyAsync(hcol.data(), hd, (j + 2) * sizeof(double), cudaMemcpyDeviceToHost, c->st);
@@ -434,9 +435,6 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
       }
       double hn = sqrt(std::max(hn2, 0.0));
       if (!std::isfinite(hn)) return fail(c, WSI_ERR_NAN, "non-finite Krylov vector");
-      double ihn = hn > 0.0 ? 1.0 / hn : 0.0;
-      cudaMemcpyAsync(hd + osc, &ihn, sizeof(double), cudaMemcpyHostToDevice, c->st);
-      launch_maxpy(V, n, j + 1, hcoef, w, n, 1.0, c->st, hd + osc);
       for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hsum[i];
       H[(size_t)(j + 1) * m + j] = hn;
       // previous rotations
@@ -458,6 +456,12 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
         ++j;
         done = true;
         break;
+      }
+      // the next basis vector, unless the cycle ends here
+      if (j + 1 < m) {
+        const double ihn = 1.0 / hn;
+        cudaMemcpyAsync(hd + osc, &ihn, sizeof(double), cudaMemcpyHostToDevice, c->st);
+        launch_maxpy(V, n, j + 1, hcoef, w, n, 1.0, c->st, hd + osc);
       }
     }
     if (!done) j = m;

@@ -247,8 +247,6 @@ struct Precond {
   T* ru[3] = {nullptr, nullptr, nullptr};
   T* ut[3] = {nullptr, nullptr, nullptr};
   T* rp = nullptr;
-  T* y = nullptr;
-  T* gp[3] = {nullptr, nullptr, nullptr};
   double* dscratch = nullptr;  // reductions
   double* dsum = nullptr;
   bool built = false;
@@ -266,12 +264,13 @@ struct Opts {
 };
 
 template <typename T>
-int precond_alloc(Precond<T>& P, const GridDev& g, std::string& err);
+int precond_alloc(Precond<T>& P, const GridDev& g, bool visc, std::string& err);  // visc: with viscous V-cycles
 template <typename T>
 void precond_free(Precond<T>& P);
 // rebuild level coefficients from the float64 fine coefficients
 template <typename T>
-int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, cudaStream_t st, std::string& err);
+int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, cudaStream_t st,
+                  std::string& err);
 // z = P^{-1} v  (packed float64 Stokes vectors)
 template <typename T>
 void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,

@@ -32,6 +32,10 @@ static constexpr int BX = 32, BY = 8;
 static inline dim3 grid3(int nx, int ny, int nz) { return dim3(cdiv(nx, BX), cdiv(ny, BY), nz); }
 
 template <typename T>
+__global__ void k_coarse_inverse(GridDev g, const T* __restrict__ bx, const T* __restrict__ by,
+                                 const T* __restrict__ bz, int n, double* inv);
+static constexpr int INV_MAX = 160;  // cells of a coarsest level that is inverted on the device
+template <typename T>
 struct CoarseCycle;
 template <typename T, int NT>
 __global__ void k_coarse_cycle(const __grid_constant__ CoarseCycle<T> c);
@@ -81,7 +85,7 @@ static int vlev_alloc(Precond<T>& P, std::string& err) {
 }
 
 template <typename T>
-int precond_alloc(Precond<T>& P, const GridDev& g0, std::string& err) {
+int precond_alloc(Precond<T>& P, const GridDev& g0, bool visc, std::string& err) {
   precond_free(P);
   GridDev g = g0;
   for (;;) {
@@ -139,14 +143,14 @@ int precond_alloc(Precond<T>& P, const GridDev& g0, std::string& err) {
   P.coarse_inv = dalloc<double>(P.allocs, (size_t)P.ncoarse * P.ncoarse, err);
   for (int c = 0; c < 3; ++c) {
     P.rho_face[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
-    P.ru[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
+    if (!std::is_same<T, double>::value) P.ru[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
     P.ut[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
-    P.gp[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
   }
   P.mu_cc = dalloc<T>(P.allocs, fsize(g0, 3), err);
   for (int e = 0; e < 3; ++e) P.mu_e[e] = dalloc<T>(P.allocs, esize(g0, e), err);
-  P.rp = dalloc<T>(P.allocs, fsize(g0, 3), err);
-  P.y = dalloc<T>(P.allocs, fsize(g0, 3), err);
+  if (!std::is_same<T, double>::value) P.rp = dalloc<T>(P.allocs, fsize(g0, 3), err);
+  cudaFuncSetAttribute(k_coarse_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (INV_MAX + 1) * INV_MAX * (int)sizeof(double));
   // the fused lower cycle's shared memory: x and b of its small levels (each at
   // most half the cells of the one above) and the dense solve's vector
   cudaFuncSetAttribute(k_coarse_cycle<T, coarse_threads<T>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -172,8 +176,10 @@ int precond_alloc(Precond<T>& P, const GridDev& g0, std::string& err) {
   cudaGetLastError();
   P.dscratch = dalloc<double>(P.allocs, 4096, err);
   P.dsum = dalloc<double>(P.allocs, 8, err);
-  if (!P.coarse_inv || !P.mu_cc || !P.rp || !P.y || !P.dscratch || !P.dsum) return WSI_ERR_OOM;
-  return vlev_alloc(P, err);
+  if (!P.coarse_inv || !P.mu_cc || (!P.rp && !std::is_same<T, double>::value) || !P.dscratch || !P.dsum) return WSI_ERR_OOM;
+  if (visc) return vlev_alloc(P, err);
+  P.vlev.assign(P.lev.size(), VLevel<T>{});
+  return WSI_OK;
 }
 
 template <typename T>
@@ -193,9 +199,9 @@ void precond_free(Precond<T>& P) {
 
 // ------------------------------------------------------------ coefficients
 template <int C, typename T>
-__global__ void k_coarsen_beta(GridDev gf, GridDev gc, int r0, int r1, int r2, const T* __restrict__ bf, T* bc) {
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= ext(gc, C, 0) || j >= ext(gc, C, 1)) return;
+__device__ __forceinline__ void coarsen_face(const GridDev& gf, const GridDev& gc, int r0, int r1, int r2,
+                                             const T* __restrict__ bf, T* bc, int i, int j, int k) {
+  if (i >= ext(gc, C, 0) || j >= ext(gc, C, 1) || k >= ext(gc, C, 2)) return;
   int r[3] = {r0, r1, r2};
   int base[3] = {i * r[0], j * r[1], k * r[2]};
   int span[3] = {r[0], r[1], r[2]};
@@ -205,6 +211,23 @@ __global__ void k_coarsen_beta(GridDev gf, GridDev gc, int r0, int r1, int r2, c
     for (int b = 0; b < span[1]; ++b)
       for (int a = 0; a < span[0]; ++a) s += bf[fidx(gf, C, base[0] + a, base[1] + b, base[2] + c)];
   bc[fidx(gc, C, i, j, k)] = s / T(span[0] * span[1] * span[2]);
+}
+
+// the three face arrays in one launch: blockIdx.z walks the z-planes of each
+template <typename T>
+__global__ void k_coarsen_faces(GridDev gf, GridDev gc, int r0, int r1, int r2, CVel<T> f, Vel<T> c) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, n2 = gc.n[2] + 1;
+  const int q = blockIdx.z / n2, k = blockIdx.z - q * n2;
+  if (q == 0) coarsen_face<0, T>(gf, gc, r0, r1, r2, f.q[0], c.q[0], i, j, k);
+  else if (q == 1) coarsen_face<1, T>(gf, gc, r0, r1, r2, f.q[1], c.q[1], i, j, k);
+  else coarsen_face<2, T>(gf, gc, r0, r1, r2, f.q[2], c.q[2], i, j, k);
+}
+
+template <typename T>
+static void coarsen_faces(const MGLevel<T>& F, const GridDev& gc, const T* const f[3], T* const c[3], cudaStream_t st) {
+  const dim3 grid(cdiv(gc.n[0] + 1, BX), cdiv(gc.n[1] + 1, BY), 3 * (gc.n[2] + 1));
+  { k_coarsen_faces<T><<<grid, dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1], F.r[2], CVel<T>{{f[0], f[1], f[2]}},
+                                                      Vel<T>{{c[0], c[1], c[2]}}); WSI_COUNT(); }
 }
 
 // coarse cell viscosity: mean of the children
@@ -359,8 +382,72 @@ static void spd_inverse(std::vector<double>& A, int n) {
   A.swap(I);
 }
 
+// The dense coarsest operator M = -L + c 1 1^T of the level and its inverse
+// (Gauss-Jordan in place, no pivoting: M is symmetric positive definite), one
+// block, the matrix in shared memory; the same operations as the host form
+// above.  float64-pipe bound, n^3 multiply-adds on one SM: about 80 us at 64
+// cells, but nothing waits for it on the host (read back, inverted there and
+// sent down it cost two synchronisations and about 0.4 ms per set-up).
 template <typename T>
-int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, cudaStream_t st, std::string& err) {
+__global__ void __launch_bounds__(1024) k_coarse_inverse(GridDev g, const T* __restrict__ bx, const T* __restrict__ by,
+                                                         const T* __restrict__ bz, int n, double* inv) {
+  extern __shared__ double W[];  // n x n, then a column
+  double* col = W + n * n;
+  __shared__ double dmax_w[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int t = tid; t < n * n; t += 1024) W[t] = 0.0;
+  __syncthreads();
+  double dg = 0.0;
+  for (int row = tid; row < n; row += 1024) {
+    const int i = row % g.n[0], j = row / g.n[0] % g.n[1], k = row / (g.n[0] * g.n[1]);
+    const int c3[3] = {i, j, k}, sd[3] = {1, g.n[0], g.n[0] * g.n[1]};
+    double d = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const T* b = a == 0 ? bx : (a == 1 ? by : bz);
+      const double ih2 = 1.0 / (g.h[a] * g.h[a]);
+      const double hi = (double)b[fidx(g, a, i + (a == 0), j + (a == 1), k + (a == 2))];
+      if (c3[a] + 1 < g.n[a]) {
+        W[row * n + row + sd[a]] -= hi * ih2;
+        d += hi * ih2;
+      }
+      if (c3[a] > 0) {
+        const double lo = (double)b[fidx(g, a, i, j, k)];
+        W[row * n + row - sd[a]] -= lo * ih2;
+        d += lo * ih2;
+      }
+      if (a == 2 && k + 1 == g.n[2] && g.open_top) d += 2.0 * hi * ih2;  // p = 0 on the open top: ghost -p
+    }
+    W[row * n + row] = d;
+    dg = d;
+  }
+  for (int o = 16; o > 0; o >>= 1) dg = fmax(dg, __shfl_xor_sync(0xffffffffu, dg, o));
+  if (lane == 0) dmax_w[warp] = dg;
+  __syncthreads();
+  double dmax = 0.0;
+  for (int w = 0; w < 32; ++w) dmax = fmax(dmax, dmax_w[w]);
+  const double creg = g.open_top ? 0.0 : dmax / n;
+  for (int t = tid; t < n * n; t += 1024) W[t] += creg;
+  for (int p = 0; p < n; ++p) {
+    __syncthreads();
+    const double id = 1.0 / W[p * n + p];
+    for (int r = tid; r < n; r += 1024) col[r] = W[r * n + p];
+    __syncthreads();
+    for (int c = tid; c < n; c += 1024) W[p * n + c] = c == p ? id : W[p * n + c] * id;
+    __syncthreads();
+    for (int r = warp; r < n; r += 32) {
+      const double f = col[r];
+      if (r == p || f == 0.0) continue;
+      for (int c = lane; c < n; c += 32) W[r * n + c] = fma(-f, W[p * n + c], c == p ? 0.0 : W[r * n + c]);
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < n * n; t += 1024) inv[t] = W[t];
+}
+
+template <typename T>
+int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, cudaStream_t st,
+                  std::string& err) {
   // fine coefficients in T (one launch for the ten arrays)
   {
     CastSet<double, T> cs;
@@ -383,24 +470,16 @@ int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, cud
     MGLevel<T>& F = P.lev[l];
     MGLevel<T>& Cl = P.lev[l + 1];
     const GridDev& gc = Cl.g;
-    { k_coarsen_beta<0, T><<<grid3(gc.n[0] + 1, gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], F.beta[0], Cl.beta[0]); WSI_COUNT(); }
-    { k_coarsen_beta<1, T><<<grid3(gc.n[0], gc.n[1] + 1, gc.n[2]), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], F.beta[1], Cl.beta[1]); WSI_COUNT(); }
-    { k_coarsen_beta<2, T><<<grid3(gc.n[0], gc.n[1], gc.n[2] + 1), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], F.beta[2], Cl.beta[2]); WSI_COUNT(); }
+    const T* bf[3] = {F.beta[0], F.beta[1], F.beta[2]};
+    coarsen_faces<T>(F, gc, bf, Cl.beta, st);
+    if (!visc) continue;  // the viscous hierarchy is used by viscous V-cycles only
     // viscous coefficients: face density like beta (coplanar mean), cell
     // viscosity the mean of the children, edge viscosity harmonic again
     const T* rf[3] = {l == 0 ? P.rho_face[0] : P.vlev[l].rho_face[0], l == 0 ? P.rho_face[1] : P.vlev[l].rho_face[1],
                       l == 0 ? P.rho_face[2] : P.vlev[l].rho_face[2]};
     const T* mf = l == 0 ? P.mu_cc : P.vlev[l].mu_cc;
     VLevel<T>& VC = P.vlev[l + 1];
-    { k_coarsen_beta<0, T><<<grid3(gc.n[0] + 1, gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], rf[0], VC.rho_face[0]); WSI_COUNT(); }
-    { k_coarsen_beta<1, T><<<grid3(gc.n[0], gc.n[1] + 1, gc.n[2]), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], rf[1], VC.rho_face[1]); WSI_COUNT(); }
-    { k_coarsen_beta<2, T><<<grid3(gc.n[0], gc.n[1], gc.n[2] + 1), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1],
-                                                                                        F.r[2], rf[2], VC.rho_face[2]); WSI_COUNT(); }
+    coarsen_faces<T>(F, gc, rf, VC.rho_face, st);
     { k_vmu_down<T><<<grid3(gc.n[0], gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1], F.r[2], mf,
                                                                              VC.mu_cc); WSI_COUNT(); }
     { k_vedges<0, T><<<grid3(gc.n[0] + 1, gc.n[1] + 1, gc.n[2]), dim3(BX, BY), 0, st>>>(gc, VC.mu_cc, VC.mu_e[0]); WSI_COUNT(); }
@@ -411,6 +490,12 @@ int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, cud
   const MGLevel<T>& Lc = P.lev.back();
   const GridDev& gc = Lc.g;
   int n = P.ncoarse;
+  if (n <= INV_MAX) {
+    { k_coarse_inverse<T><<<1, 1024, (size_t)(n + 1) * n * sizeof(double), st>>>(gc, Lc.beta[0], Lc.beta[1], Lc.beta[2], n,
+                                                                              P.coarse_inv); WSI_COUNT(); }
+    P.built = true;
+    return WSI_OK;
+  }
   std::vector<T> hb[3];
   for (int c = 0; c < 3; ++c) {
     hb[c].resize(fsize(gc, c));
@@ -1402,19 +1487,23 @@ template <typename T>
 void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,
                    cudaStream_t st) {
   Packing pk = packing(g);
-  {
+  MGLevel<T>& L0 = P.lev[0];
+  const T *ru[3], *rp;
+  for (int c = 0; c < 3; ++c) cudaMemsetAsync(P.ut[c], 0, fsize(g, c) * sizeof(T), st);
+  if constexpr (std::is_same<T, double>::value) {
+    for (int c = 0; c < 3; ++c) ru[c] = v + pk.off[c];
+    rp = v + pk.off[3];
+  } else {
     CastSet<double, T> cs;
     cs.count = 4;
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 4; ++c) {
       cs.a[c] = v + pk.off[c];
-      cs.b[c] = P.ru[c];
+      cs.b[c] = c < 3 ? P.ru[c] : P.rp;
       cs.n[c] = fsize(g, c);
-      cudaMemsetAsync(P.ut[c], 0, fsize(g, c) * sizeof(T), st);
     }
-    cs.a[3] = v + pk.off[3];
-    cs.b[3] = P.rp;
-    cs.n[3] = fsize(g, 3);
     cast_set(cs, st);  // one launch for the four parts
+    for (int c = 0; c < 3; ++c) ru[c] = P.ru[c];
+    rp = P.rp;
   }
   Coef<T> cf;
   for (int c = 0; c < 3; ++c) {
@@ -1426,20 +1515,18 @@ void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, co
   T inv_dt = (T)(1.0 / dt), theta = (T)o.theta;
   // u~ = A^{-1} r_u (approximately): red-black sweeps, or viscous V-cycles
   if (o.visc_mg > 0) {
-    for (int c = 0; c < o.visc_mg; ++c) vcycle_visc<T>(P, o, 0, cf, P.ut, P.ru, inv_dt, theta, st);
+    for (int c = 0; c < o.visc_mg; ++c) vcycle_visc<T>(P, o, 0, cf, P.ut, ru, inv_dt, theta, st);
   } else {
     for (int s = 0; s < o.visc_sweeps; ++s)
-      for (int c = 0; c < 2; ++c) launch_viscous_rbgs<T>(g, cf, inv_dt, theta, P.ut, P.ru, c, st);
+      for (int c = 0; c < 2; ++c) launch_viscous_rbgs<T>(g, cf, inv_dt, theta, P.ut, ru, c, st);
   }
   // y = r_p + D u~, mean-free in a closed box (the pressure problem's
   // compatibility condition; an open top fixes the pressure instead)
   dim3 gr = grid3(g.n[0], g.n[1], g.n[2]);
-  { k_div_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, P.ut[0], P.ut[1], P.ut[2], P.rp, P.y); WSI_COUNT(); }
+  { k_div_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, P.ut[0], P.ut[1], P.ut[2], rp, L0.b); WSI_COUNT(); }
   size_t ncell = fsize(g, 3);
-  if (!g.open_top) sub_mean<T>(P.y, ncell, P.dsum, P.dscratch, st);
-  // phi = L^{-1} y
-  MGLevel<T>& L0 = P.lev[0];
-  cudaMemcpyAsync(L0.b, P.y, ncell * sizeof(T), cudaMemcpyDeviceToDevice, st);
+  if (!g.open_top) sub_mean<T>(L0.b, ncell, P.dsum, P.dscratch, st);
+  // phi = L^{-1} y (the cycles leave their right-hand side as it is)
   for (int c = 0; c < o.mg_cycles; ++c) vcycle(P, o, 0, c == 0, st);
   // velocity and pressure updates
   { k_vel_update<0, T><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[0], L0.beta[0], L0.x,
@@ -1449,16 +1536,18 @@ void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, co
   { k_vel_update<2, T><<<grid3(g.n[0], g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, P.ut[2], L0.beta[2], L0.x,
                                                                                  z + pk.off[2]); WSI_COUNT(); }
   int blocks = (int)std::min<size_t>((ncell + 255) / 256, 152 * 16);
-  { k_p_update<T><<<std::max(blocks, 1), 256, 0, st>>>(ncell, L0.x, P.mu_cc, P.y, 1.0 / dt, o.theta, z + pk.off[3]); WSI_COUNT(); }
+  { k_p_update<T><<<std::max(blocks, 1), 256, 0, st>>>(ncell, L0.x, P.mu_cc, L0.b, 1.0 / dt, o.theta, z + pk.off[3]); WSI_COUNT(); }
   if (!g.open_top) sub_mean<double>(z + pk.off[3], ncell, P.dsum, P.dscratch, st);
 }
 
-template int precond_alloc<double>(Precond<double>&, const GridDev&, std::string&);
-template int precond_alloc<float>(Precond<float>&, const GridDev&, std::string&);
+template int precond_alloc<double>(Precond<double>&, const GridDev&, bool, std::string&);
+template int precond_alloc<float>(Precond<float>&, const GridDev&, bool, std::string&);
 template void precond_free<double>(Precond<double>&);
 template void precond_free<float>(Precond<float>&);
-template int precond_setup<double>(Precond<double>&, const GridDev&, const Coef<double>&, cudaStream_t, std::string&);
-template int precond_setup<float>(Precond<float>&, const GridDev&, const Coef<double>&, cudaStream_t, std::string&);
+template int precond_setup<double>(Precond<double>&, const GridDev&, const Coef<double>&, bool, cudaStream_t,
+                                   std::string&);
+template int precond_setup<float>(Precond<float>&, const GridDev&, const Coef<double>&, bool, cudaStream_t,
+                                  std::string&);
 template void precond_apply<double>(Precond<double>&, const GridDev&, const Opts&, double, const double*, double*,
                                     cudaStream_t);
 template void precond_apply<float>(Precond<float>&, const GridDev&, const Opts&, double, const double*, double*,
