@@ -110,6 +110,10 @@ struct wsi_ctx {
   // float64 part of the momentum right-hand side fixed over a step's cycles
   double* b0 = nullptr;
   double* inv_mu = nullptr;  // materials scratch: 1/mu per cell
+  // mixed path: the preconditioned vectors of a cycle, and the float32 copy of
+  // the basis vector the preconditioner takes
+  std::vector<ZVec> zv;
+  float* v32 = nullptr;
   // mixed path: split (hi, lo) copies of the operator coefficients (refreshed
   // at the start of every solve) and of the matvec input
   DfOperands df;
@@ -290,8 +294,12 @@ int copy_out(wsi_ctx* c, double* dst, const double* src, size_t n) {
   return WSI_OK;
 }
 
-int ensure_pc(wsi_ctx* c) {
+// fill: *fill tells whether the caller still has to fill in the finest level's
+// float32 density and viscosities (df_coef_refresh does both at once)
+int ensure_pc(wsi_ctx* c, bool* fill = nullptr) {
   const bool visc = c->opts.visc_mg > 0;
+  if (fill) *fill = false;
+  const bool later = fill && c->mixed() && !visc;
   if (!c->pc_alloc) {
     // allocated on first use: grids that are only used for operator applies
     // need no multigrid hierarchy
@@ -302,35 +310,34 @@ int ensure_pc(wsi_ctx* c) {
   }
   if (!c->pc_dirty) return WSI_OK;
   Coef<double> cf = coef_now(c);
-  int rc = c->desc.precision == WSI_PREC_MIXED ? precond_setup<float>(c->P32, c->g, cf, visc, c->st, c->err)
-                                               : precond_setup<double>(c->P64, c->g, cf, visc, c->st, c->err);
+  int rc = c->desc.precision == WSI_PREC_MIXED ? precond_setup<float>(c->P32, c->g, cf, visc, later, c->st, c->err)
+                                               : precond_setup<double>(c->P64, c->g, cf, visc, false, c->st, c->err);
   if (rc == WSI_OK && c->mixed()) {
     rc = learned_alloc(c->P32, c->unet_impl, c->unet_level, c->gunet_impl, c->gunet_level, c->err);
     if (rc == WSI_OK && (c->unet_impl || c->gunet_impl))
       rc = learned_setup(c->P32, c->rho_cc, c->phi_cur ? c->phi_cur : c->phi, c->st, c->err);
     c->P32.learn.on = c->unet_on;
   }
-  if (rc == WSI_OK) c->pc_dirty = false;
+  if (rc == WSI_OK) {
+    c->pc_dirty = false;
+    if (fill) *fill = later;
+  }
   return rc;
 }
 
-void pc_apply(wsi_ctx* c, double dt, const double* v, double* z) {
-  if (c->desc.precision == WSI_PREC_MIXED)
-    precond_apply<float>(c->P32, c->g, c->opts, dt, v, z, c->st);
-  else
-    precond_apply<double>(c->P64, c->g, c->opts, dt, v, z, c->st);
-}
-
 // split copies of the coefficients for the double-float matvec (mixed path);
-// the face density is stored times 1/dt
-void df_coef_refresh(wsi_ctx* c, const Coef<double>& cf, double inv_dt) {
+// the face density is stored times 1/dt; f32: also the preconditioner's float32
+// copies
+void df_coef_refresh(wsi_ctx* c, const Coef<double>& cf, double inv_dt, bool f32) {
   if (!c->mixed()) return;
-  df_split_coefs(c->df, cf.rho_face, cf.mu_e, cf.mu_cc, inv_dt, c->st);  // one launch for the seven arrays
+  Precond<float>& P = c->P32;
+  float* const d[7] = {P.rho_face[0], P.rho_face[1], P.rho_face[2], P.mu_cc, P.mu_e[0], P.mu_e[1], P.mu_e[2]};
+  df_split_coefs(c->df, cf.rho_face, cf.mu_e, cf.mu_cc, inv_dt, f32 ? d : nullptr, c->st);  // one launch
 }
 
-// K x: float64 on the plain path; on the mixed path in double-float
-// arithmetic (same accuracy class, a fraction of the float64 instructions)
-// from the coefficients split by the last df_coef_refresh
+// K x: float64 on the plain path; on the mixed path in
+// double-float arithmetic (same accuracy class, a fraction of the float64
+// instructions) from the coefficients split by the last df_coef_refresh
 void stokes_mv(wsi_ctx* c, const Coef<double>& cf, double inv_dt, double theta, const double* x, double* y,
                cudaStream_t st) {
   if (c->mixed()) {
@@ -356,13 +363,14 @@ int df_check(wsi_ctx* c) {
 // with classical Gram-Schmidt (see the iteration for the re-orthogonalisation
 // rule).
 int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_opts* o, wsi_solve_stats* s) {
-  int rc = ensure_pc(c);
+  bool fill = false;
+  int rc = ensure_pc(c, &fill);
   if (rc) return rc;
   const size_t n = c->nstk;
   const int m = c->m;
   const double inv_dt = 1.0 / dt, theta = c->desc.theta;
   Coef<double> cf = coef_now(c);
-  df_coef_refresh(c, cf, inv_dt);
+  df_coef_refresh(c, cf, inv_dt, fill);
   double* V = c->V;
   double* Z = c->Z;
   double* hd = c->hdev;
@@ -382,8 +390,7 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
   if (!o->use_x0) cudaMemsetAsync(x, 0, n * sizeof(double), c->st);
   // r = b - K x  into V_0
   stokes_mv(c, cf, inv_dt, theta, x, Vj(0), c->st);
-  launch_lincomb(n, 1.0, b, -1.0, Vj(0), 0.0, nullptr, Vj(0), c->st);
-  double beta = host_norm2(Vj(0), n, red, c->st);
+  double beta = host_residual_norm2(b, Vj(0), n, red, c->st);
   const double tol = o->rtol * bnorm;
   std::vector<double> H((size_t)(m + 1) * m, 0.0), cs(m), sn(m), gv(m + 1), hcol(2 * (m + 1) + 1);
   int result = WSI_OK;
@@ -396,15 +403,20 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
     }
     double ib = 1.0 / beta;
     cudaMemcpyAsync(hd, &ib, sizeof(double), cudaMemcpyHostToDevice, c->st);
-    launch_scale(Vj(0), n, hd, false, c->st);
+    launch_scale(Vj(0), n, hd, c->st, c->v32);
     std::fill(gv.begin(), gv.end(), 0.0);
     gv[0] = beta;
     int j = 0;
     bool done = false;
     for (; j < m; ++j) {
-      pc_apply(c, dt, Vj(j), Zj(j));
       double* w = Vj(j + 1);
-      stokes_mv(c, cf, inv_dt, theta, Zj(j), w, c->st);
+      if (c->mixed()) {
+        precond_apply(c->P32, c->g, c->opts, dt, c->v32, c->zv[j], c->df, c->st);
+        launch_stokes_df_z(c->g, c->df, c->zv[j], theta, w, c->df_err, c->st);
+      } else {
+        precond_apply(c->P64, c->g, c->opts, dt, Vj(j), Zj(j), c->st);
+        stokes_mv(c, cf, inv_dt, theta, Zj(j), w, c->st);
+      }
       // Classical Gram-Schmidt.  One pass gives h = V^T w together with w.w
       // (w is V_{j+1}, the last row), so ||w - V h||^2 = w.w - |h|^2 needs no
       // second pass; when that cancels by more than half (the DGKS test) the
@@ -421,8 +433,7 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
       std::vector<double> hsum(hcol.begin(), hcol.begin() + (j + 1));
       const double* hcoef = hd;
       if (!(hn2 >= 0.5 * ww)) {
-        launch_maxpy(V, n, j + 1, hd, w, n, 1.0, c->st);
-        launch_mdot(V, n, j + 2, w, n, hd + o2, red, c->st);
+        launch_orth(V, n, j + 1, hd, w, n, hd + o2, red, c->st);
         cudaMemcpyAsync(hcol.data(), hd + o2, (j + 2) * sizeof(double), cudaMemcpyDeviceToHost, c->st);
         if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check(c, "fgmres reorthogonalisation");
         double ww2 = hcol[j + 1], hh2 = 0.0;
@@ -461,7 +472,7 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
       if (j + 1 < m) {
         const double ihn = 1.0 / hn;
         cudaMemcpyAsync(hd + osc, &ihn, sizeof(double), cudaMemcpyHostToDevice, c->st);
-        launch_maxpy(V, n, j + 1, hcoef, w, n, 1.0, c->st, hd + osc);
+        launch_maxpy(V, n, j + 1, hcoef, w, n, 1.0, c->st, hd + osc, c->v32);
       }
     }
     if (!done) j = m;
@@ -473,11 +484,15 @@ int fgmres(wsi_ctx* c, const double* b, double* x, double dt, const wsi_solve_op
       y[i] = sacc / H[(size_t)i * m + i];
     }
     cudaMemcpyAsync(hd, y.data(), j * sizeof(double), cudaMemcpyHostToDevice, c->st);
-    launch_maxpy(Z, n, j, hd, x, n, -1.0, c->st);
-    // true residual
-    stokes_mv(c, cf, inv_dt, theta, x, Vj(0), c->st);
-    launch_lincomb(n, 1.0, b, -1.0, Vj(0), 0.0, nullptr, Vj(0), c->st);
-    beta = host_norm2(Vj(0), n, red, c->st);
+    // x and its true residual
+    if (c->mixed()) {
+      launch_x_update(c->g, c->df, c->zv.data(), j, hd, x, c->st);
+      launch_stokes_df_ready(c->g, c->df, theta, Vj(0), c->df_err, c->st);
+    } else {
+      launch_maxpy(Z, n, j, hd, x, n, -1.0, c->st);
+      stokes_mv(c, cf, inv_dt, theta, x, Vj(0), c->st);
+    }
+    beta = host_residual_norm2(b, Vj(0), n, red, c->st);
   }
   // zero-mean pressure in a closed box (an open top fixes the pressure)
   if (!c->g.open_top) {
@@ -897,7 +912,7 @@ int wsi_create_grid(const wsi_grid_desc* d, void* stream, wsi_ctx** out) {
   c->b = A(c->nstk);
   c->x = A(c->nstk);
   c->V = A(c->nstk * (size_t)(c->m + 1));
-  c->Z = A(c->nstk * (size_t)c->m);
+  if (d->precision != WSI_PREC_MIXED) c->Z = A(c->nstk * (size_t)c->m);
   c->hdev = A(4 * (c->m + 2) + 8);
   c->b0 = A(c->nvel);
   c->inv_mu = A(c->ncell);
@@ -920,9 +935,24 @@ int wsi_create_grid(const wsi_grid_desc* d, void* stream, wsi_ctx** out) {
     df_operands_shape(g, c->df);
     for (int a = 0; a < DF_NARR; ++a) c->df.a[a] = (float2*)A(df_operand_elems(c->df, a));
     c->df_err = (int*)A(1);
+    c->v32 = F(c->nstk);
+    // the preconditioned vectors in one allocation (parts on 256 bytes)
+    c->zv.resize(c->m);
+    size_t zo[4], zn = 0;
+    for (int q = 0; q < 4; ++q) {
+      zo[q] = zn;
+      zn += (q < 3 ? (zvec_elems(c->df, q) + 63) / 64 : (c->ncell + 31) / 32) * 32;  // doubles
+    }
+    double* zb = A(zn * (size_t)c->m);
+    for (int j = 0; ok && j < c->m; ++j) {
+      for (int q = 0; q < 3; ++q) c->zv[j].v[q] = (float*)(zb + zn * j + zo[q]);
+      c->zv[j].p = zb + zn * j + zo[3];
+    }
     if (ok) {
       cudaMemsetAsync(c->df_err, 0, sizeof(int), c->st);
-      if (df_operands_encode(c->df) != WSI_OK) {
+      bool enc = df_operands_encode(c->df) == WSI_OK;
+      for (ZVec& z : c->zv) enc = enc && zvec_encode(c->df, z) == WSI_OK;
+      if (!enc) {
         c->err = "tile-copy descriptors of the matvec operands could not be encoded";
         wsi_destroy(c);
         return WSI_ERR_CUDA;
@@ -949,6 +979,7 @@ void wsi_destroy(wsi_ctx* c) {
   precond_free<double>(c->P64);
   precond_free<float>(c->P32);
   cudaFree(c->bins_mem);
+  for (ZVec& z : c->zv) zvec_release(z);
   df_operands_release(c->df);
   for (void* p : c->allocs) cudaFree(p);
   delete c;
@@ -1334,7 +1365,7 @@ int wsi_apply(wsi_ctx* c, int op, const double* in, double* out, double dt) {
   vel_parts(c, xout, qo);
   switch (op) {
     case WSI_OP_STOKES:
-      df_coef_refresh(c, cf, 1.0 / dt);
+      df_coef_refresh(c, cf, 1.0 / dt, false);
       stokes_mv(c, cf, 1.0 / dt, c->desc.theta, xin, xout, c->st);
       break;
     case WSI_OP_VISCOUS: launch_viscous<double>(c->g, cf, 1.0 / dt, c->desc.theta, qi, qo, c->st, false); break;
@@ -1905,7 +1936,7 @@ int wsi_pressure_solve(wsi_ctx* c, const double* y, double* x, double rtol, int 
   const int plain_cycles = 2;
   bool learned = c->mixed() && c->unet_on;
   bool last_learned = false;
-  double* xb = c->Z;  // iterate before a learned cycle
+  double* xb = c->V + n;  // iterate before a learned cycle
   double rn = ynorm, prev = ynorm, rho_plain = 1.0;
   int cycles = 0;
   while (true) {

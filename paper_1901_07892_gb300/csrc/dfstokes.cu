@@ -43,6 +43,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "df.cuh"
 #include "internal.h"
@@ -56,9 +57,21 @@ static constexpr int TX = 34;    // tile columns: x = FX bx - 2 .. FX bx + 31
 static constexpr int TY = FBY + 2;  // tile rows: y = FBY by - 1 .. FBY by + FBY
 static constexpr int TILE = 208;    // float2 slots per tile (TX TY = 204, padded to a multiple of 128 bytes)
 static constexpr int NST = 3;       // levels in the ring: two read, one in flight
-static constexpr int STAGE = DF_NARR * TILE;
-static constexpr int SMEM_BYTES = NST * STAGE * 8 + NST * 8;
-static constexpr uint32_t STAGE_TX = DF_NARR * TX * TY * 8;  // bytes the copies of one level deliver
+// float32 velocity tiles of a preconditioned vector: TMA starts them on a
+// multiple of four columns, at most two left of the others' origin
+static constexpr int ZTX = 36;
+static constexpr int ZTILE = 224;   // floats per tile (ZTX TY = 216, padded to a multiple of 128 bytes)
+
+// Layout of a ring level.  HF: the velocity comes as float32 (tails zero), so
+// the level holds the pressure and the seven coefficients as pairs, then three
+// float32 tiles.
+template <bool HF>
+struct Ring {
+  static constexpr int FIRST = HF ? DF_P : 0;  // first array held as pairs
+  static constexpr int BYTES = (DF_NARR - FIRST) * TILE * 8 + (HF ? 3 * ZTILE * 4 : 0);
+  static constexpr uint32_t TXB = (DF_NARR - FIRST) * TX * TY * 8 + (HF ? 3 * ZTX * TY * 4 : 0);
+  static constexpr int SMEM = NST * BYTES + NST * 8;
+};
 
 struct HtConst {
   ht ih[3];       // 1/h
@@ -125,6 +138,21 @@ __device__ __forceinline__ ht hk(ht a, ht c, bool pow2) {
   return P2 ? ht{a.h * c.h, a.t * c.h} : ht_k(a, c, pow2);
 }
 
+// a float32 value: a pair whose tail is zero
+struct hf {
+  float h;
+};
+__device__ __forceinline__ ht ht_sub(hf a, hf b) {
+  float s, e;
+  two_sum(a.h, -b.h, s, e);
+  return ht{s, e};
+}
+__device__ __forceinline__ ht ht_mul(ht a, hf c) {
+  const float p = a.h * c.h;
+  return ht{p, fmaf(a.t, c.h, fmaf(a.h, c.h, -p))};
+}
+__device__ __forceinline__ hf ht_sgn(hf a, float s) { return hf{a.h * s}; }
+
 // rho/dt q + G p - theta L as a float64
 template <bool P2>
 __device__ __forceinline__ double row_out(const HtConst& K, ht rq, ht gp, ht L) {
@@ -133,11 +161,13 @@ __device__ __forceinline__ double row_out(const HtConst& K, ht rq, ht gp, ht L) 
 
 // P2: 1/h, 2/h^2 and theta are all powers of two (uniform power-of-two
 // spacings), so that every multiplication by a grid constant is an exact
-// scaling
-template <bool P2>
+// scaling.  HF: float32 velocity (see Ring).
+template <bool P2, bool HF>
 __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ DfMaps maps, const HtConst K,
                                                         double* yu, double* yv, double* yw, double* yp, int* err) {
-  extern __shared__ __align__(128) float2 dsm[];
+  using R = Ring<HF>;
+  using Q = typename std::conditional<HF, hf, ht>::type;
+  extern __shared__ __align__(128) unsigned char dsm[];
   const int nx = K.n[0], ny = K.n[1], nz = K.n[2];
   const int lane = threadIdx.x, tid = threadIdx.y * 32 + lane;
   const int xs = blockIdx.x * FX - 2, ys = blockIdx.y * FBY - 1;  // tile origin (x even)
@@ -147,15 +177,20 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
   const int k0 = blockIdx.z * FKC;
   const int k1 = min(k0 + FKC, nz);
   const int tmax = k1 - k0 + 1;  // ring levels t = 0 .. tmax hold z-levels k0 - 1 .. k1
-  const uint32_t sm0 = tma::saddr(dsm), bar0 = sm0 + NST * STAGE * 8;
+  const uint32_t sm0 = tma::saddr(dsm), bar0 = sm0 + NST * R::BYTES;
+  const int xz = xs & ~3;  // origin of the float32 tiles
 
   // (thread 0) the eleven copies of ring level t into slot t % NST
   auto issue = [&](int t) {
     const int s = t % NST;
     const uint32_t bar = bar0 + 8 * s;
-    tma::mbar_expect_tx(bar, STAGE_TX);
-    for (int a = 0; a < DF_NARR; ++a)
-      tma::load3(sm0 + (uint32_t)((s * DF_NARR + a) * TILE * 8), &maps.m[a], bar, xs, ys, k0 - 1 + t);
+    tma::mbar_expect_tx(bar, R::TXB);
+    const uint32_t l0 = sm0 + (uint32_t)(s * R::BYTES);
+    for (int a = R::FIRST; a < DF_NARR; ++a)
+      tma::load3(l0 + (uint32_t)((a - R::FIRST) * TILE * 8), &maps.m[a], bar, xs, ys, k0 - 1 + t);
+    if (HF)
+      for (int a = 0; a < 3; ++a)
+        tma::load3(l0 + (uint32_t)((DF_NARR - R::FIRST) * TILE * 8 + a * ZTILE * 4), &maps.m[a], bar, xz, ys, k0 - 1 + t);
   };
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) tma::mbar_init(bar0 + 8 * s, 1);
@@ -168,9 +203,18 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
     if (!tma::mbar_wait(bar0 + 8 * (t % NST), (t / NST) & 1)) ok = false;
   };
   // slot of ring level t, tile of array a in it, and its element at grid row jj, column ii
-  auto slot = [&](int t) -> const float2* { return dsm + (t % NST) * STAGE; };
-  auto tile = [&](const float2* S, int a) -> const float2* { return S + a * TILE; };
+  auto slot = [&](int t) -> const float2* { return reinterpret_cast<const float2*>(dsm + (t % NST) * R::BYTES); };
+  auto tile = [&](const float2* S, int a) -> const float2* { return S + (a - R::FIRST) * TILE; };
   auto at = [&](const float2* T, int jj, int ii) -> ht { return ht_of(T[(jj - ys) * TX + (ii - xs)]); };
+  // velocity component c (0 .. 2) of level S
+  auto vat = [&](const float2* S, int c, int jj, int ii) -> Q {
+    if constexpr (HF) {
+      const float* Z = reinterpret_cast<const float*>(S + (DF_NARR - R::FIRST) * TILE) + c * ZTILE;
+      return hf{Z[(jj - ys) * ZTX + (ii - xz)]};
+    } else {
+      return ht_of(S[c * TILE + (jj - ys) * TX + (ii - xs)]);
+    }
+  };
 
   const bool cI = i >= 0 && i < nx;  // a cell column
   const bool fI = i >= 0 && i <= nx; // an x-face / x-edge column
@@ -186,24 +230,22 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
   const bool pxk = K.pw & 1, pyk = (K.pw >> 1) & 1, pzk = (K.pw >> 2) & 1;
   const ht ihx = K.ih[0], ihy = K.ih[1], ihz = K.ih[2];
 
-  // w of a level's tile at (column col_i or its x-ghost, row jj or its y-ghost)
-  auto w_at = [&](const float2* Tw, int col_i, bool xghost, float xsg, int jj) -> ht {
+  // w of a level at (column col_i or its x-ghost, row jj or its y-ghost)
+  auto w_at = [&](const float2* S, int col_i, bool xghost, float xsg, int jj) -> Q {
     float s = xghost ? xsg : 1.f;
     if (jj < 0) { jj = 0; s *= byl; } else if (jj >= ny) { jj = ny - 1; s *= byh; }
-    return ht_sgn(at(Tw, jj, col_i), s);
+    return ht_sgn(vat(S, DF_W, jj, col_i), s);
   };
   // shear stresses on the z-level edges of ring level t from the fields at the
   // level below (lo) and at it (hi), ghosts already applied:
   // xz at (i, j), yz at (i, j) and at (i, j + 1)
-  auto zedges = [&](const float2* S, ht u_lo, ht u_hi, ht v_lo, ht v_hi, ht vj_lo, ht vj_hi, ht& txz, ht& tyz,
-                    ht& tyzj) {
-    const float2* Tw = tile(S, DF_W);
+  auto zedges = [&](const float2* S, Q u_lo, Q u_hi, Q v_lo, Q v_hi, Q vj_lo, Q vj_hi, ht& txz, ht& tyz, ht& tyzj) {
     const float2* Te = tile(S, DF_MU_YZ);
-    const ht wc = w_at(Tw, ic, hiX, bxh, j);   // w at column i (x-edge column; ghost at i = nx)
-    const ht wm = w_at(Tw, icm, loX, bxl, j);  // w at column i - 1
-    const ht wjm = w_at(Tw, ic, false, 1.f, j - 1);
-    const ht wjp = w_at(Tw, ic, false, 1.f, j + 1);
-    const ht w0 = at(Tw, j, ic);
+    const Q wc = w_at(S, ic, hiX, bxh, j);   // w at column i (x-edge column; ghost at i = nx)
+    const Q wm = w_at(S, icm, loX, bxl, j);  // w at column i - 1
+    const Q wjm = w_at(S, ic, false, 1.f, j - 1);
+    const Q wjp = w_at(S, ic, false, 1.f, j + 1);
+    const Q w0 = vat(S, DF_W, j, ic);
     txz = ht_mul(at(tile(S, DF_MU_XZ), j, iff),
                  ht_add(hk<P2>(ht_sub(u_hi, u_lo), ihz, pzk), hk<P2>(ht_sub(wc, wm), ihx, pxk)));
     tyz = ht_mul(at(Te, j, ic), ht_add(hk<P2>(ht_sub(v_hi, v_lo), ihz, pzk), hk<P2>(ht_sub(w0, wjm), ihy, pyk)));
@@ -215,19 +257,19 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
   wait(1);
   const float2* S0 = slot(0);
   const float2* S1 = slot(1);
-  ht u_k = at(tile(S1, DF_U), j, iff);
-  ht v_k = at(tile(S1, DF_V), j, ic);
-  ht vj_k = at(tile(S1, DF_V), j + 1, ic);
-  ht w_k = at(tile(S1, DF_W), j, ic);
+  Q u_k = vat(S1, DF_U, j, iff);
+  Q v_k = vat(S1, DF_V, j, ic);
+  Q vj_k = vat(S1, DF_V, j + 1, ic);
+  Q w_k = vat(S1, DF_W, j, ic);
   ht txz_k, tyz_k, tyzj_k;
   ht nzz_km1{0.f, 0.f}, p_km1{0.f, 0.f};
   {
-    ht u_m, v_m, vj_m;
+    Q u_m, v_m, vj_m;
     if (k0 > 0) {
-      u_m = at(tile(S0, DF_U), j, iff);
-      v_m = at(tile(S0, DF_V), j, ic);
-      vj_m = at(tile(S0, DF_V), j + 1, ic);
-      const ht w_m = at(tile(S0, DF_W), j, ic);
+      u_m = vat(S0, DF_U, j, iff);
+      v_m = vat(S0, DF_V, j, ic);
+      vj_m = vat(S0, DF_V, j + 1, ic);
+      const Q w_m = vat(S0, DF_W, j, ic);
       nzz_km1 = ht_mul(at(tile(S0, DF_MU_CC), j, ic), ht_sub(w_k, w_m));
       p_km1 = at(tile(S0, DF_P), j, ic);
     } else {
@@ -246,41 +288,39 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
     const float2* Sp = slot(tp);
     wait(tp);
     // ---- level k + 1: fields and z-edge shear stresses
-    ht u_kp, v_kp, vj_kp;
+    Q u_kp, v_kp, vj_kp;
     if (k + 1 < nz) {
-      u_kp = at(tile(Sp, DF_U), j, iff);
-      v_kp = at(tile(Sp, DF_V), j, ic);
-      vj_kp = at(tile(Sp, DF_V), j + 1, ic);
+      u_kp = vat(Sp, DF_U, j, iff);
+      v_kp = vat(Sp, DF_V, j, ic);
+      vj_kp = vat(Sp, DF_V, j + 1, ic);
     } else {
       u_kp = ht_sgn(u_k, bzh);
       v_kp = ht_sgn(v_k, bzh);
       vj_kp = ht_sgn(vj_k, bzh);
     }
-    const ht w_kp = at(tile(Sp, DF_W), j, ic);
+    const Q w_kp = vat(Sp, DF_W, j, ic);
     ht txz_kp, tyz_kp, tyzj_kp;
     zedges(Sp, u_k, u_kp, v_k, v_kp, vj_k, vj_kp, txz_kp, tyz_kp, tyzj_kp);
 
     // ---- level k: normal stresses and the xy shear stresses at rows j, j + 1
-    const float2* TU = tile(Sk, DF_U);
-    const float2* TV = tile(Sk, DF_V);
     const float2* TP = tile(Sk, DF_P);
     const float2* TM = tile(Sk, DF_MU_CC);
     const float2* TE = tile(Sk, DF_MU_XY);
     const ht mu_c = at(TM, j, ic);
-    const ht u_ip = at(TU, j, ifp);
+    const Q u_ip = vat(Sk, DF_U, j, ifp);
     const ht nxx = ht_mul(mu_c, ht_sub(u_ip, u_k));
     const ht nyy = ht_mul(mu_c, ht_sub(vj_k, v_k));
     const ht nzz = ht_mul(mu_c, ht_sub(w_kp, w_k));
     ht nyy_m{0.f, 0.f};
-    if (j > 0) nyy_m = ht_mul(at(TM, j - 1, ic), ht_sub(v_k, at(TV, j - 1, ic)));
+    if (j > 0) nyy_m = ht_mul(at(TM, j - 1, ic), ht_sub(v_k, vat(Sk, DF_V, j - 1, ic)));
     // u at rows j - 1, j + 1 of column i (y-ghosts)
-    const ht u_jm = j > 0 ? at(TU, j - 1, iff) : ht_sgn(u_k, byl);
-    const ht u_jp = j + 1 < ny ? at(TU, j + 1, iff) : ht_sgn(u_k, byh);
+    const Q u_jm = j > 0 ? vat(Sk, DF_U, j - 1, iff) : ht_sgn(u_k, byl);
+    const Q u_jp = j + 1 < ny ? vat(Sk, DF_U, j + 1, iff) : ht_sgn(u_k, byh);
     // v at columns i, i - 1 of rows j, j + 1 (x-ghosts)
-    const ht vx = hiX ? ht_sgn(v_k, bxh) : v_k;
-    const ht vjx = hiX ? ht_sgn(vj_k, bxh) : vj_k;
-    const ht vm = ht_sgn(at(TV, j, icm), loX ? bxl : 1.f);
-    const ht vjm = ht_sgn(at(TV, j + 1, icm), loX ? bxl : 1.f);
+    const Q vx = hiX ? ht_sgn(v_k, bxh) : v_k;
+    const Q vjx = hiX ? ht_sgn(vj_k, bxh) : vj_k;
+    const Q vm = ht_sgn(vat(Sk, DF_V, j, icm), loX ? bxl : 1.f);
+    const Q vjm = ht_sgn(vat(Sk, DF_V, j + 1, icm), loX ? bxl : 1.f);
     const ht txy = ht_mul(at(TE, j, iff), ht_add(hk<P2>(ht_sub(u_k, u_jm), ihy, pyk), hk<P2>(ht_sub(vx, vm), ihx, pxk)));
     const ht txyj =
         ht_mul(at(TE, j + 1, iff), ht_add(hk<P2>(ht_sub(u_jp, u_k), ihy, pyk), hk<P2>(ht_sub(vjx, vjm), ihx, pxk)));
@@ -375,6 +415,7 @@ __global__ void __launch_bounds__(32 * FBY) k_stokes_df(const __grid_constant__ 
 struct PadSplit {
   const double* x[DF_NARR];
   float2* out[DF_NARR];
+  float* f32[DF_NARR];  // dense float32 copy (unscaled), or null
   double scale[DF_NARR];
   int cols[DF_NARR], pitch[DF_NARR], nrows[DF_NARR];
   int count;
@@ -404,6 +445,7 @@ __global__ void __launch_bounds__(256) k_df_split_pad(PadSplit s) {
         if (c < pitch) {
           const dfl d = df_split(sc == 1.0 ? v[u] : sc * v[u]);
           orow[c] = make_float2(d.h, d.l);
+          if (s.f32[a] && c < cols) s.f32[a][(size_t)r * cols + c] = d2f_fast(v[u]);
         }
       }
     }
@@ -411,7 +453,7 @@ __global__ void __launch_bounds__(256) k_df_split_pad(PadSplit s) {
 }
 
 static void split_pad(const DfOperands& o, const int* which, const double* const* x, const double* scale, int count,
-                      cudaStream_t st) {
+                      float* const* f32, cudaStream_t st) {
   PadSplit s;
   int rmax = 0;
   s.count = count;
@@ -419,6 +461,7 @@ static void split_pad(const DfOperands& o, const int* which, const double* const
     const int a = which[q];
     s.x[q] = x[q];
     s.out[q] = o.a[a];
+    s.f32[q] = f32 ? f32[q] : nullptr;
     s.scale[q] = scale[q];
     s.cols[q] = o.cols[a];
     s.pitch[q] = o.pitch[a];
@@ -443,8 +486,11 @@ void df_operands_shape(const GridDev& g, DfOperands& o) {
     o.rows[a] = dims[a][1];
     o.levels[a] = dims[a][2];
     o.pitch[a] = (dims[a][0] + 1) & ~1;  // 16-byte rows
+    if (a < 3) o.zpitch[a] = (dims[a][0] + 3) & ~3;
   }
 }
+
+size_t zvec_elems(const DfOperands& o, int c) { return (size_t)o.zpitch[c] * o.rows[c] * o.levels[c]; }
 
 size_t df_operand_elems(const DfOperands& o, int a) { return (size_t)o.pitch[a] * o.rows[a] * o.levels[a]; }
 
@@ -453,7 +499,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-int df_operands_encode(DfOperands& o) {
+static EncodeTiledFn encode_fn() {
   static EncodeTiledFn encode = nullptr;
   if (!encode) {
     void* fn = nullptr;
@@ -461,9 +507,42 @@ int df_operands_encode(DfOperands& o) {
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
             cudaSuccess ||
         q != cudaDriverEntryPointSuccess || !fn)
-      return WSI_ERR_CUDA;
+      return nullptr;
     encode = (EncodeTiledFn)fn;
   }
+  return encode;
+}
+
+// descriptors of the matvec with z: the operands' ones with the velocity arrays
+// exchanged for z's float32 parts
+int zvec_encode(const DfOperands& o, ZVec& z) {
+  EncodeTiledFn encode = encode_fn();
+  if (!encode || !o.maps) return WSI_ERR_CUDA;
+  DfMaps* m = new DfMaps(*static_cast<const DfMaps*>(o.maps));
+  for (int a = 0; a < 3; ++a) {
+    const cuuint64_t dim[3] = {(cuuint64_t)o.cols[a], (cuuint64_t)o.rows[a], (cuuint64_t)o.levels[a]};
+    const cuuint64_t stride[2] = {(cuuint64_t)o.zpitch[a] * 4, (cuuint64_t)o.zpitch[a] * o.rows[a] * 4};
+    const cuuint32_t box[3] = {ZTX, TY, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (encode(&m->m[a], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)z.v[a], dim, stride, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+      delete m;
+      return WSI_ERR_CUDA;
+    }
+  }
+  z.maps = m;
+  return WSI_OK;
+}
+
+void zvec_release(ZVec& z) {
+  delete static_cast<DfMaps*>(z.maps);
+  z.maps = nullptr;
+}
+
+int df_operands_encode(DfOperands& o) {
+  EncodeTiledFn encode = encode_fn();
+  if (!encode) return WSI_ERR_CUDA;
   DfMaps* m = new DfMaps;
   for (int a = 0; a < DF_NARR; ++a) {
     const cuuint64_t dim[3] = {(cuuint64_t)o.cols[a], (cuuint64_t)o.rows[a], (cuuint64_t)o.levels[a]};
@@ -487,11 +566,11 @@ void df_operands_release(DfOperands& o) {
 }
 
 void df_split_coefs(const DfOperands& o, const double* const rho[3], const double* const mu_e[3], const double* mu_cc,
-                    double inv_dt, cudaStream_t st) {
+                    double inv_dt, float* const f32[7], cudaStream_t st) {
   const int which[7] = {DF_RHO_X, DF_RHO_Y, DF_RHO_Z, DF_MU_CC, DF_MU_XY, DF_MU_XZ, DF_MU_YZ};
   const double* x[7] = {rho[0], rho[1], rho[2], mu_cc, mu_e[0], mu_e[1], mu_e[2]};
   const double sc[7] = {inv_dt, inv_dt, inv_dt, 1.0, 1.0, 1.0, 1.0};
-  split_pad(o, which, x, sc, 7, st);
+  split_pad(o, which, x, sc, 7, f32, st);
 }
 
 static dfl host_split(double a) {
@@ -506,15 +585,9 @@ static bool host_pow2(const dfl& c) {
   return c.l == 0.0f && c.h != 0.0f && std::fabs(std::frexp((double)c.h, &e)) == 0.5;
 }
 
-void launch_stokes_df(const GridDev& g, const DfOperands& o, double theta, const double* x, double* y, int* err,
-                      cudaStream_t st) {
+static void matvec(const GridDev& g, const DfMaps& m, bool half, double theta, double* y, int* err,
+                   cudaStream_t st) {
   Packing pk = packing(g);
-  {
-    const int which[4] = {DF_U, DF_V, DF_W, DF_P};
-    const double* xs[4] = {x + pk.off[0], x + pk.off[1], x + pk.off[2], x + pk.off[3]};
-    const double sc[4] = {1.0, 1.0, 1.0, 1.0};
-    split_pad(o, which, xs, sc, 4, st);
-  }
   HtConst k;
   k.pw = 0;
   for (int a = 0; a < 3; ++a) {
@@ -532,21 +605,124 @@ void launch_stokes_df(const GridDev& g, const DfOperands& o, double theta, const
   k.open_top = g.open_top;
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_stokes_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    cudaFuncSetAttribute(k_stokes_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaFuncSetAttribute(k_stokes_df<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ring<false>::SMEM);
+    cudaFuncSetAttribute(k_stokes_df<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ring<false>::SMEM);
+    cudaFuncSetAttribute(k_stokes_df<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ring<true>::SMEM);
+    cudaFuncSetAttribute(k_stokes_df<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ring<true>::SMEM);
     attr = true;
   }
-  dim3 grid(cdiv(g.n[0] + 1, FX), cdiv(g.n[1], FBY), cdiv(g.n[2], FKC));
-  const DfMaps& m = *static_cast<const DfMaps*>(o.maps);
+  const dim3 grid(cdiv(g.n[0] + 1, FX), cdiv(g.n[1], FBY), cdiv(g.n[2], FKC)), block(32, FBY);
+  double *yu = y + pk.off[0], *yv = y + pk.off[1], *yw = y + pk.off[2], *yp = y + pk.off[3];
+  const bool p2 = k.pw == 0x7Fu;
   ktimer_begin(KC_STOKES, st);
-  if (k.pw == 0x7Fu)
-    k_stokes_df<true><<<grid, dim3(32, FBY), SMEM_BYTES, st>>>(m, k, y + pk.off[0], y + pk.off[1], y + pk.off[2],
-                                                               y + pk.off[3], err);
-  else
-    k_stokes_df<false><<<grid, dim3(32, FBY), SMEM_BYTES, st>>>(m, k, y + pk.off[0], y + pk.off[1], y + pk.off[2],
-                                                                y + pk.off[3], err);
+  if (half) {
+    if (p2) k_stokes_df<true, true><<<grid, block, Ring<true>::SMEM, st>>>(m, k, yu, yv, yw, yp, err);
+    else k_stokes_df<false, true><<<grid, block, Ring<true>::SMEM, st>>>(m, k, yu, yv, yw, yp, err);
+  } else {
+    if (p2) k_stokes_df<true, false><<<grid, block, Ring<false>::SMEM, st>>>(m, k, yu, yv, yw, yp, err);
+    else k_stokes_df<false, false><<<grid, block, Ring<false>::SMEM, st>>>(m, k, yu, yv, yw, yp, err);
+  }
   WSI_COUNT();
   ktimer_end(KC_STOKES, st);
+}
+
+void launch_stokes_df(const GridDev& g, const DfOperands& o, double theta, const double* x, double* y, int* err,
+                      cudaStream_t st) {
+  Packing pk = packing(g);
+  const int which[4] = {DF_U, DF_V, DF_W, DF_P};
+  const double* xs[4] = {x + pk.off[0], x + pk.off[1], x + pk.off[2], x + pk.off[3]};
+  const double sc[4] = {1.0, 1.0, 1.0, 1.0};
+  split_pad(o, which, xs, sc, 4, nullptr, st);
+  matvec(g, *static_cast<const DfMaps*>(o.maps), false, theta, y, err, st);
+}
+
+void launch_stokes_df_z(const GridDev& g, const DfOperands& o, const ZVec& z, double theta, double* y, int* err,
+                        cudaStream_t st) {
+  (void)o;
+  matvec(g, *static_cast<const DfMaps*>(z.maps), true, theta, y, err, st);
+}
+
+void launch_stokes_df_ready(const GridDev& g, const DfOperands& o, double theta, double* y, int* err, cudaStream_t st) {
+  matvec(g, *static_cast<const DfMaps*>(o.maps), false, theta, y, err, st);
+}
+
+// x += sum_t y[t] z_t over the velocity rows (blockIdx.y the component, a warp
+// per row, four elements in flight per lane) and the pressure (blockIdx.y = 3);
+// the last pass also splits the new x into the operands of the matvec that
+// follows (a splitting pass of its own read x again: 340 us at 256^3)
+static constexpr int XUP = 16;  // vectors per pass
+struct XUpdate {
+  const float* v[XUP][3];
+  const double* p[XUP];
+  size_t off[4];
+  int cols[4], pitch[4], nrows[4], m;
+  float2* op[4];  // null: not the last pass
+  int opitch[4];
+};
+__global__ void __launch_bounds__(256) k_x_update(const __grid_constant__ XUpdate u, const double* __restrict__ h, double* x) {
+  __shared__ double hs[XUP];
+  if (threadIdx.x < u.m) hs[threadIdx.x] = -1.0 * h[threadIdx.x];
+  __syncthreads();
+  const int q = blockIdx.y, cols = u.cols[q], pitch = u.pitch[q], lane = threadIdx.x & 31;
+  double* xq = x + u.off[q];
+  const int wstride = gridDim.x * (blockDim.x >> 5);
+  for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < u.nrows[q]; r += wstride) {
+    double* xr = xq + (size_t)r * cols;
+    float2* orow = u.op[q] ? u.op[q] + (size_t)r * u.opitch[q] : nullptr;
+    const int end = orow ? u.opitch[q] : cols;
+    for (int c0 = lane; c0 < end; c0 += 128) {
+      double s[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) s[a] = c0 + 32 * a < cols ? xr[c0 + 32 * a] : 0.0;
+      for (int t = 0; t < u.m; ++t) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const int c = c0 + 32 * a;
+          if (c < cols) {
+            const double z = q < 3 ? f2d_fast(u.v[t][q][(size_t)r * pitch + c]) : u.p[t][(size_t)r * cols + c];
+            s[a] -= hs[t] * z;
+          }
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const int c = c0 + 32 * a;
+        if (c < cols) xr[c] = s[a];
+        if (orow && c < end) {
+          const dfl d = df_split(s[a]);
+          orow[c] = make_float2(d.h, d.l);
+        }
+      }
+    }
+  }
+}
+
+void launch_x_update(const GridDev& g, const DfOperands& o, const ZVec* z, int m, const double* h, double* x,
+                     cudaStream_t st) {
+  Packing pk = packing(g);
+  for (int t0 = 0; t0 < m; t0 += XUP) {
+    XUpdate u;
+    u.m = std::min(XUP, m - t0);
+    int rmax = 0;
+    for (int q = 0; q < 4; ++q) {
+      u.off[q] = pk.off[q];
+      u.cols[q] = o.cols[q];
+      u.pitch[q] = q < 3 ? o.zpitch[q] : o.cols[q];
+      u.nrows[q] = o.rows[q] * o.levels[q];
+      u.op[q] = t0 + XUP >= m ? o.a[q] : nullptr;
+      u.opitch[q] = o.pitch[q];
+      rmax = std::max(rmax, u.nrows[q]);
+    }
+    for (int t = 0; t < u.m; ++t) {
+      for (int c = 0; c < 3; ++c) u.v[t][c] = z[t0 + t].v[c];
+      u.p[t] = z[t0 + t].p;
+    }
+    ktimer_begin(KC_MAXPY, st);
+    // per vector the float32 velocity and the float64 pressure; x read, written and split
+    ktimer_bytes(KC_MAXPY, (double)pk.off[3] * (4.0 * u.m + 24.0) + (double)fsize(g, 3) * (8.0 * u.m + 24.0));
+    { k_x_update<<<dim3(std::min(cdiv(rmax, 8), 152 * 8), 4), 256, 0, st>>>(u, h + t0, x); WSI_COUNT(); }
+    ktimer_end(KC_MAXPY, st);
+  }
 }
 
 }  // namespace wsi

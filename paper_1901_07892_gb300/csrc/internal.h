@@ -70,7 +70,15 @@ enum DfArray {
 struct DfOperands {
   float2* a[DF_NARR] = {};
   int cols[DF_NARR], rows[DF_NARR], levels[DF_NARR], pitch[DF_NARR];
+  int zpitch[3];         // row pitch of a preconditioned vector's float32 velocity parts (rows on 16 bytes)
   void* maps = nullptr;  // host copy of the arrays' tile-copy descriptors
+};
+// A preconditioned vector of the mixed path: the float32 velocity as it leaves
+// the preconditioner (padded rows; wall faces stay zero) and the float64 pressure
+struct ZVec {
+  float* v[3] = {};
+  double* p = nullptr;
+  void* maps = nullptr;  // tile-copy descriptors of the matvec with this vector
 };
 // extents and pitches of the arrays for grid g
 void df_operands_shape(const GridDev& g, DfOperands& o);
@@ -79,14 +87,28 @@ size_t df_operand_elems(const DfOperands& o, int a);
 // the tile-copy descriptors of the allocated arrays (WSI_OK or WSI_ERR_CUDA)
 int df_operands_encode(DfOperands& o);
 void df_operands_release(DfOperands& o);
-// split the seven coefficient arrays, the face density times inv_dt
+int zvec_encode(const DfOperands& o, ZVec& z);
+void zvec_release(ZVec& z);
+size_t zvec_elems(const DfOperands& o, int c);  // float32 elements of velocity part c
+// split the seven coefficient arrays, the face density times inv_dt; with f32
+// also their float32 copies (dense; order rho_x, rho_y, rho_z, mu_cc, mu_xy,
+// mu_xz, mu_yz)
 void df_split_coefs(const DfOperands& o, const double* const rho[3], const double* const mu_e[3], const double* mu_cc,
-                    double inv_dt, cudaStream_t st);
+                    double inv_dt, float* const f32[7], cudaStream_t st);
 // y = K x in double-float arithmetic: x split into the operands, then the
 // matvec from the coefficients split by the last df_split_coefs; *err is set
 // to 1 when a wait for a tile copy gave up
 void launch_stokes_df(const GridDev& g, const DfOperands& o, double theta, const double* x, double* y, int* err,
                       cudaStream_t st);
+// y = K z; the pressure operand (DF_P) already holds z's pressure, split
+void launch_stokes_df_z(const GridDev& g, const DfOperands& o, const ZVec& z, double theta, double* y, int* err,
+                        cudaStream_t st);
+// y = K x for the x that launch_x_update left split in the operands
+void launch_stokes_df_ready(const GridDev& g, const DfOperands& o, double theta, double* y, int* err, cudaStream_t st);
+// x += sum_t y[t] z_t (t < m, in order), the new x also split into the matvec's
+// operands; h: the coefficients on the device
+void launch_x_update(const GridDev& g, const DfOperands& o, const ZVec* z, int m, const double* h, double* x,
+                     cudaStream_t st);
 // red-black Gauss-Seidel half sweep on the viscous block for component c
 template <typename T>
 void launch_viscous_rbgs(const GridDev& g, const Coef<T>& cf, T inv_dt, T theta, T* const q[3], const T* const b[3],
@@ -149,10 +171,33 @@ void launch_rhs_nc(const GridDev& g, const double* b0, const TN* N, const double
 void launch_mdot(const double* V, size_t ldv, int m, const double* w, size_t n, double* out, double* scratch,
                  cudaStream_t st);
 // w = (w - sign * sum_t h[t] V_t) * scale  (h and scale on device; scale
-// null = 1)
+// null = 1); with w32 also the result's float32 copy
 void launch_maxpy(const double* V, size_t ldv, int m, const double* h, double* w, size_t n, double sign,
-                  cudaStream_t st, const double* scale_dev = nullptr);
-void launch_scale(double* x, size_t n, const double* s_dev, bool inverse, cudaStream_t st);
+                  cudaStream_t st, const double* scale_dev = nullptr, float* w32 = nullptr);
+// w -= V h, then out = (V^T w, w.w), w being row m of V (m rows before it)
+void launch_orth(const double* V, size_t ldv, int m, const double* h, double* w, size_t n, double* out, double* scratch,
+                 cudaStream_t st);
+// x *= s; with x32 also its float32 copy
+void launch_scale(double* x, size_t n, const double* s_dev, cudaStream_t st, float* x32 = nullptr);
+// deterministic sums: RB blocks of RT threads walk an array with a grid stride,
+// their partials are added by launch_reduce_sum
+static constexpr int RB = 152 * 4, RT = 256;
+void launch_reduce_sum(const double* part, double* out_dev, cudaStream_t st);
+// block sum of acc (RT threads, fixed tree) into part[blockIdx.x]
+__device__ __forceinline__ void block_sum_to(double acc, double* part) {
+  __shared__ double sh[RT / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) sh[wid] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int q = 0; q < RT / 32; ++q) s += sh[q];
+    part[blockIdx.x] = s;
+  }
+}
+// r <- b - r, and its norm (the order of host_norm2's sum)
+double host_residual_norm2(const double* b, double* r, size_t n, double* scratch, cudaStream_t st);
 double host_norm2(const double* x, size_t n, double* scratch, cudaStream_t st);
 // max |x_i| read back to the host (scratch: RB + 1 doubles)
 double host_maxabs(const double* x, size_t n, double* scratch, cudaStream_t st);
@@ -244,9 +289,8 @@ struct Precond {
   T* mu_cc = nullptr;
   T* mu_e[3] = {nullptr, nullptr, nullptr};
   // work
-  T* ru[3] = {nullptr, nullptr, nullptr};
   T* ut[3] = {nullptr, nullptr, nullptr};
-  T* rp = nullptr;
+  T* pv = nullptr;  // float32: pressure part before its mean is removed
   double* dscratch = nullptr;  // reductions
   double* dsum = nullptr;
   bool built = false;
@@ -267,14 +311,17 @@ template <typename T>
 int precond_alloc(Precond<T>& P, const GridDev& g, bool visc, std::string& err);  // visc: with viscous V-cycles
 template <typename T>
 void precond_free(Precond<T>& P);
-// rebuild level coefficients from the float64 fine coefficients
+// rebuild level coefficients from the float64 fine coefficients; beta_only: the
+// density and viscosities on the finest level are filled in by the caller
 template <typename T>
-int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, cudaStream_t st,
+int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, bool beta_only, cudaStream_t st,
                   std::string& err);
-// z = P^{-1} v  (packed float64 Stokes vectors)
-template <typename T>
-void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,
+// z = P^{-1} v; v a packed Stokes vector in T.  float64: z packed; float32: z's
+// parts, and its pressure split into the matvec operand o.a[DF_P]
+void precond_apply(Precond<double>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,
                    cudaStream_t st);
+void precond_apply(Precond<float>& P, const GridDev& g, const Opts& o, double dt, const float* v, const ZVec& z,
+                   const DfOperands& op, cudaStream_t st);
 
 // ---------------------------------------------------------------- waves.cu
 struct WaveDev {

@@ -24,6 +24,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "df.cuh"
 #include "internal.h"
 
 namespace wsi {
@@ -143,12 +144,11 @@ int precond_alloc(Precond<T>& P, const GridDev& g0, bool visc, std::string& err)
   P.coarse_inv = dalloc<double>(P.allocs, (size_t)P.ncoarse * P.ncoarse, err);
   for (int c = 0; c < 3; ++c) {
     P.rho_face[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
-    if (!std::is_same<T, double>::value) P.ru[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
     P.ut[c] = dalloc<T>(P.allocs, fsize(g0, c), err);
   }
   P.mu_cc = dalloc<T>(P.allocs, fsize(g0, 3), err);
   for (int e = 0; e < 3; ++e) P.mu_e[e] = dalloc<T>(P.allocs, esize(g0, e), err);
-  if (!std::is_same<T, double>::value) P.rp = dalloc<T>(P.allocs, fsize(g0, 3), err);
+  if (!std::is_same<T, double>::value) P.pv = dalloc<T>(P.allocs, fsize(g0, 3), err);
   cudaFuncSetAttribute(k_coarse_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (INV_MAX + 1) * INV_MAX * (int)sizeof(double));
   // the fused lower cycle's shared memory: x and b of its small levels (each at
@@ -176,7 +176,7 @@ int precond_alloc(Precond<T>& P, const GridDev& g0, bool visc, std::string& err)
   cudaGetLastError();
   P.dscratch = dalloc<double>(P.allocs, 4096, err);
   P.dsum = dalloc<double>(P.allocs, 8, err);
-  if (!P.coarse_inv || !P.mu_cc || (!P.rp && !std::is_same<T, double>::value) || !P.dscratch || !P.dsum) return WSI_ERR_OOM;
+  if (!P.coarse_inv || !P.mu_cc || (!P.pv && !std::is_same<T, double>::value) || !P.dscratch || !P.dsum) return WSI_ERR_OOM;
   if (visc) return vlev_alloc(P, err);
   P.vlev.assign(P.lev.size(), VLevel<T>{});
   return WSI_OK;
@@ -446,9 +446,9 @@ __global__ void __launch_bounds__(1024) k_coarse_inverse(GridDev g, const T* __r
 }
 
 template <typename T>
-int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, cudaStream_t st,
-                  std::string& err) {
-  // fine coefficients in T (one launch for the ten arrays)
+int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, bool visc, bool beta_only,
+                  cudaStream_t st, std::string& err) {
+  // fine coefficients in T (one launch for the arrays)
   {
     CastSet<double, T> cs;
     cs.count = 0;
@@ -459,11 +459,13 @@ int precond_setup(Precond<T>& P, const GridDev& g, const Coef<double>& fine, boo
       ++cs.count;
     };
     for (int c = 0; c < 3; ++c) {
-      add(fine.rho_face[c], P.rho_face[c], fsize(g, c));
+      if (!beta_only) add(fine.rho_face[c], P.rho_face[c], fsize(g, c));
       add(fine.beta[c], P.lev[0].beta[c], fsize(g, c));
     }
-    add(fine.mu_cc, P.mu_cc, fsize(g, 3));
-    for (int e = 0; e < 3; ++e) add(fine.mu_e[e], P.mu_e[e], esize(g, e));
+    if (!beta_only) {
+      add(fine.mu_cc, P.mu_cc, fsize(g, 3));
+      for (int e = 0; e < 3; ++e) add(fine.mu_e[e], P.mu_e[e], esize(g, e));
+    }
     cast_set(cs, st);
   }
   for (size_t l = 0; l + 1 < P.lev.size(); ++l) {
@@ -1375,16 +1377,27 @@ int learned_alloc(Precond<float>& P, UNetImpl* net, int level, UNetImpl* gnet, i
 }
 
 // ------------------------------------------------------------ PC glue kernels
+// y = r_p + D u~ and the partials of its sum, in the fixed order of launch_sum
+// (each thread's cells with a grid stride), so that the mean needs no second
+// pass over y
 template <typename T>
-__global__ void k_div_add(GridDev g, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ w,
-                          const T* __restrict__ rp, T* y) {
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.n[0] || j >= g.n[1]) return;
-  T d = (u[fidx(g, 0, i + 1, j, k)] - u[fidx(g, 0, i, j, k)]) * ginv<T>(g, 0) +
-        (v[fidx(g, 1, i, j + 1, k)] - v[fidx(g, 1, i, j, k)]) * ginv<T>(g, 1) +
-        (w[fidx(g, 2, i, j, k + 1)] - w[fidx(g, 2, i, j, k)]) * ginv<T>(g, 2);
-  size_t id = fidx(g, 3, i, j, k);
-  y[id] = rp[id] + d;
+__global__ void __launch_bounds__(RT) k_div_sum(GridDev g, const T* __restrict__ u, const T* __restrict__ v,
+                                                const T* __restrict__ w, const T* __restrict__ rp, T* y, double* part) {
+  const unsigned nx = g.n[0], ny = g.n[1];
+  const size_t n = (size_t)nx * ny * g.n[2], stride = (size_t)RB * RT;
+  const size_t pl = (size_t)nx * ny;
+  double acc = 0.0;
+#pragma unroll 4
+  for (size_t t = (size_t)blockIdx.x * RT + threadIdx.x; t < n; t += stride) {
+    const unsigned row = (unsigned)(t / nx), k = row / ny;
+    const size_t iu = t + row, iv = t + (size_t)k * nx;  // x-faces: one more per row; y-faces: one more row per plane
+    const T d = (u[iu + 1] - u[iu]) * ginv<T>(g, 0) + (v[iv + nx] - v[iv]) * ginv<T>(g, 1) +
+                (w[t + pl] - w[t]) * ginv<T>(g, 2);
+    const T q = rp[t] + d;
+    y[t] = q;
+    acc += cvt<double, T>(q);
+  }
+  block_sum_to(acc, part);
 }
 
 // u = u~ - beta G phi on C-faces, written as float64 into z
@@ -1407,19 +1420,87 @@ __global__ void k_vel_update(GridDev g, const T* __restrict__ ut, const T* __res
   z[id] = cvt<double, T>(ut[id] - beta[id] * gphi);
 }
 
-// p = phi/dt - theta mu y - mean (mean subtracted with the sum in s_dev)
-template <typename T>
-__global__ void k_p_update(size_t n, const T* __restrict__ phi, const T* __restrict__ mu, const T* __restrict__ y,
-                           double inv_dt, double theta, double* z) {
-  size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t stride = (size_t)gridDim.x * blockDim.x;
-  if constexpr (std::is_same<T, float>::value) {
-    // float32 preconditioner: float32 arithmetic, exact widening by integer operations
-    const float fi = (float)inv_dt, ft = (float)theta;
-    for (; t < n; t += stride) z[t] = f2d_fast(phi[t] * fi - ft * mu[t] * y[t]);
-  } else {
-    for (; t < n; t += stride) z[t] = (double)phi[t] * inv_dt - theta * (double)mu[t] * (double)y[t];
+// The same for the float32 preconditioner: the lower faces of each cell into
+// the padded float32 parts of z (wall faces stay zero), and the open top's faces
+__global__ void __launch_bounds__(256) k_vel_update_f(GridDev g, CVel<float> ut, CVel<float> beta,
+                                                      const float* __restrict__ phi, float* zu, float* zv, float* zw,
+                                                      int pu, int pv, int pw) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  if (i >= nx || j >= ny) return;
+  const int r = k * ny + j, id = r * nx + i, pl = nx * ny;
+  const float pc = phi[id];
+  if (i > 0) {
+    const int q = id + r;
+    const float gp = (pc - phi[id - 1]) * g.ihf[0];
+    zu[(size_t)r * pu + i] = ut.q[0][q] - beta.q[0][q] * gp;
   }
+  if (j > 0) {
+    const int q = id + k * nx;
+    const float gp = (pc - phi[id - nx]) * g.ihf[1];
+    zv[(size_t)(r + k) * pv + i] = ut.q[1][q] - beta.q[1][q] * gp;
+  }
+  if (k > 0) {
+    const float gp = (pc - phi[id - pl]) * g.ihf[2];
+    zw[(size_t)r * pw + i] = ut.q[2][id] - beta.q[2][id] * gp;
+  }
+  if (k == nz - 1 && g.open_top) {  // ghost -phi above the open top
+    const float gp = (-pc - pc) * g.ihf[2];
+    zw[(size_t)(r + ny) * pw + i] = ut.q[2][id + pl] - beta.q[2][id + pl] * gp;
+  }
+}
+
+// p = phi/dt - theta mu y in float32 and the partials of its sum (order of
+// launch_sum on the widened values)
+__global__ void __launch_bounds__(RT) k_p_sum_f(size_t n, const float* __restrict__ phi, const float* __restrict__ mu,
+                                                const float* __restrict__ y, float fi, float ft, float* p,
+                                                double* part) {
+  double acc = 0.0;
+  const size_t stride = (size_t)RB * RT;
+#pragma unroll 4
+  for (size_t t = (size_t)blockIdx.x * RT + threadIdx.x; t < n; t += stride) {
+    const float v = phi[t] * fi - ft * mu[t] * y[t];
+    p[t] = v;
+    acc += f2d_fast(v);
+  }
+  block_sum_to(acc, part);
+}
+
+// z's pressure: p - mean (sum null: no mean removed) in float64, and split into
+// the matvec's operand (padded rows); one warp per row
+__global__ void __launch_bounds__(256) k_p_finish_f(int cols, int nrows, int pitch, const float* __restrict__ p,
+                                                    const double* __restrict__ sum, double* z, float2* op) {
+  const double m = sum ? sum[0] / ((double)cols * (double)nrows) : 0.0;
+  const int lane = threadIdx.x & 31;
+  for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < nrows; r += gridDim.x * 8) {
+    const float* __restrict__ pr = p + (size_t)r * cols;
+    for (int c0 = lane; c0 < pitch; c0 += 128) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = c0 + 32 * u < cols ? pr[c0 + 32 * u] : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = c0 + 32 * u;
+        if (c >= pitch) continue;
+        double d = 0.0;
+        if (c < cols) {
+          d = f2d_fast(v[u]);
+          if (sum) d -= m;
+          z[(size_t)r * cols + c] = d;
+        }
+        const dfl s = df_split(d);
+        op[(size_t)r * pitch + c] = make_float2(s.h, s.l);
+      }
+    }
+  }
+}
+
+// p = phi/dt - theta mu y
+__global__ void k_p_update(size_t n, const double* __restrict__ phi, const double* __restrict__ mu,
+                           const double* __restrict__ y, double inv_dt, double theta, double* z) {
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride)
+    z[t] = phi[t] * inv_dt - theta * mu[t] * y[t];
 }
 
 template <typename T>
@@ -1483,28 +1564,14 @@ static void vcycle_visc(Precond<T>& P, const Opts& o, size_t l, const Coef<T>& c
     for (int c = 1; c >= 0; --c) launch_viscous_rbgs<T>(g, cf, inv_dt, theta, u, b, c, st);
 }
 
+// u~ = A^{-1} r_u (into P.ut), y = r_p + D u~ (level 0's right-hand side) and
+// phi = L^{-1} y (level 0's x) for the packed vector v
 template <typename T>
-void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,
-                   cudaStream_t st) {
+static void precond_core(Precond<T>& P, const GridDev& g, const Opts& o, double dt, const T* v, cudaStream_t st) {
   Packing pk = packing(g);
   MGLevel<T>& L0 = P.lev[0];
-  const T *ru[3], *rp;
+  const T* ru[3] = {v + pk.off[0], v + pk.off[1], v + pk.off[2]};
   for (int c = 0; c < 3; ++c) cudaMemsetAsync(P.ut[c], 0, fsize(g, c) * sizeof(T), st);
-  if constexpr (std::is_same<T, double>::value) {
-    for (int c = 0; c < 3; ++c) ru[c] = v + pk.off[c];
-    rp = v + pk.off[3];
-  } else {
-    CastSet<double, T> cs;
-    cs.count = 4;
-    for (int c = 0; c < 4; ++c) {
-      cs.a[c] = v + pk.off[c];
-      cs.b[c] = c < 3 ? P.ru[c] : P.rp;
-      cs.n[c] = fsize(g, c);
-    }
-    cast_set(cs, st);  // one launch for the four parts
-    for (int c = 0; c < 3; ++c) ru[c] = P.ru[c];
-    rp = P.rp;
-  }
   Coef<T> cf;
   for (int c = 0; c < 3; ++c) {
     cf.rho_face[c] = P.rho_face[c];
@@ -1522,35 +1589,63 @@ void precond_apply(Precond<T>& P, const GridDev& g, const Opts& o, double dt, co
   }
   // y = r_p + D u~, mean-free in a closed box (the pressure problem's
   // compatibility condition; an open top fixes the pressure instead)
-  dim3 gr = grid3(g.n[0], g.n[1], g.n[2]);
-  { k_div_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, P.ut[0], P.ut[1], P.ut[2], rp, L0.b); WSI_COUNT(); }
-  size_t ncell = fsize(g, 3);
-  if (!g.open_top) sub_mean<T>(L0.b, ncell, P.dsum, P.dscratch, st);
+  const size_t ncell = fsize(g, 3);
+  { k_div_sum<T><<<RB, RT, 0, st>>>(g, P.ut[0], P.ut[1], P.ut[2], v + pk.off[3], L0.b, P.dscratch); WSI_COUNT(); }
+  if (!g.open_top) {
+    launch_reduce_sum(P.dscratch, P.dsum, st);
+    const int blocks = (int)std::min<size_t>((ncell + 255) / 256, 152 * 16);
+    { k_sub_mean<T><<<std::max(blocks, 1), 256, 0, st>>>(L0.b, ncell, P.dsum); WSI_COUNT(); }
+  }
   // phi = L^{-1} y (the cycles leave their right-hand side as it is)
   for (int c = 0; c < o.mg_cycles; ++c) vcycle(P, o, 0, c == 0, st);
+}
+
+void precond_apply(Precond<double>& P, const GridDev& g, const Opts& o, double dt, const double* v, double* z,
+                   cudaStream_t st) {
+  precond_core<double>(P, g, o, dt, v, st);
+  Packing pk = packing(g);
+  const MGLevel<double>& L0 = P.lev[0];
   // velocity and pressure updates
-  { k_vel_update<0, T><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[0], L0.beta[0], L0.x,
-                                                                                 z + pk.off[0]); WSI_COUNT(); }
-  { k_vel_update<1, T><<<grid3(g.n[0], g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[1], L0.beta[1], L0.x,
-                                                                                 z + pk.off[1]); WSI_COUNT(); }
-  { k_vel_update<2, T><<<grid3(g.n[0], g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, P.ut[2], L0.beta[2], L0.x,
-                                                                                 z + pk.off[2]); WSI_COUNT(); }
+  { k_vel_update<0, double><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[0], L0.beta[0], L0.x,
+                                                                                      z + pk.off[0]); WSI_COUNT(); }
+  { k_vel_update<1, double><<<grid3(g.n[0], g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, P.ut[1], L0.beta[1], L0.x,
+                                                                                      z + pk.off[1]); WSI_COUNT(); }
+  { k_vel_update<2, double><<<grid3(g.n[0], g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, P.ut[2], L0.beta[2], L0.x,
+                                                                                      z + pk.off[2]); WSI_COUNT(); }
+  const size_t ncell = fsize(g, 3);
   int blocks = (int)std::min<size_t>((ncell + 255) / 256, 152 * 16);
-  { k_p_update<T><<<std::max(blocks, 1), 256, 0, st>>>(ncell, L0.x, P.mu_cc, L0.b, 1.0 / dt, o.theta, z + pk.off[3]); WSI_COUNT(); }
+  { k_p_update<<<std::max(blocks, 1), 256, 0, st>>>(ncell, L0.x, P.mu_cc, L0.b, 1.0 / dt, o.theta, z + pk.off[3]); WSI_COUNT(); }
   if (!g.open_top) sub_mean<double>(z + pk.off[3], ncell, P.dsum, P.dscratch, st);
+}
+
+// The mixed path's z leaves in the form that the matvec and the update of x
+// read: the float32 velocity as it is (half the bytes of its float64 copy, and
+// no splitting pass before the matvec), the pressure in float64 after its mean
+// is removed, split on the way.  At 256^3 and per application: the splits of
+// the input vector (308 us), the casts to float32 (220 us) and the float64
+// velocity and pressure passes (430 us) became 290 us.
+void precond_apply(Precond<float>& P, const GridDev& g, const Opts& o, double dt, const float* v, const ZVec& z,
+                   const DfOperands& op, cudaStream_t st) {
+  precond_core<float>(P, g, o, dt, v, st);
+  const MGLevel<float>& L0 = P.lev[0];
+  { k_vel_update_f<<<grid3(g.n[0], g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(
+      g, CVel<float>{{P.ut[0], P.ut[1], P.ut[2]}}, CVel<float>{{L0.beta[0], L0.beta[1], L0.beta[2]}}, L0.x, z.v[0], z.v[1],
+      z.v[2], op.zpitch[0], op.zpitch[1], op.zpitch[2]); WSI_COUNT(); }
+  const size_t ncell = fsize(g, 3);
+  { k_p_sum_f<<<RB, RT, 0, st>>>(ncell, L0.x, P.mu_cc, L0.b, (float)(1.0 / dt), (float)o.theta, P.pv, P.dscratch); WSI_COUNT(); }
+  if (!g.open_top) launch_reduce_sum(P.dscratch, P.dsum, st);
+  const int rows = g.n[1] * g.n[2];
+  { k_p_finish_f<<<std::min(cdiv(rows, 8), 152 * 8), 256, 0, st>>>(g.n[0], rows, op.pitch[DF_P], P.pv,
+                                                                  g.open_top ? nullptr : P.dsum, z.p, op.a[DF_P]); WSI_COUNT(); }
 }
 
 template int precond_alloc<double>(Precond<double>&, const GridDev&, bool, std::string&);
 template int precond_alloc<float>(Precond<float>&, const GridDev&, bool, std::string&);
 template void precond_free<double>(Precond<double>&);
 template void precond_free<float>(Precond<float>&);
-template int precond_setup<double>(Precond<double>&, const GridDev&, const Coef<double>&, bool, cudaStream_t,
+template int precond_setup<double>(Precond<double>&, const GridDev&, const Coef<double>&, bool, bool, cudaStream_t,
                                    std::string&);
-template int precond_setup<float>(Precond<float>&, const GridDev&, const Coef<double>&, bool, cudaStream_t,
+template int precond_setup<float>(Precond<float>&, const GridDev&, const Coef<double>&, bool, bool, cudaStream_t,
                                   std::string&);
-template void precond_apply<double>(Precond<double>&, const GridDev&, const Opts&, double, const double*, double*,
-                                    cudaStream_t);
-template void precond_apply<float>(Precond<float>&, const GridDev&, const Opts&, double, const double*, double*,
-                                   cudaStream_t);
 
 }  // namespace wsi
