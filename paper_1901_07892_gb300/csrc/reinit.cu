@@ -19,14 +19,14 @@
 // each face's difference and minmod are formed once: the pair shares them in x,
 // the march hands them on in z.  phi~ enters through a one-byte code per cell
 // (its sign and the axes along which it changes sign), made once per call;
-// the cells next to the interface are listed at the same time and
-// a second launch per stage gives them their subcell distances (inside the
-// march that path cost registers and instruction cache).  Per stage phi is read once and written once (plus phi^m in the
-// second stage) with the code byte: 9 or 13 bytes per cell in float32.  Bound
-// by instruction issue (190 warp instructions per 32 cells, 76 % of the slots):
-// 57 us per stage at 256 x 256 x 128 and 10 us for the listed cells; one cell per
-// thread, every axis by itself and the subcell path inside it took 326
-// instructions and 84 us.
+// the cells next to the interface are listed at the same time and a second
+// launch per stage gives them their subcell distances (inside the march that
+// path cost registers and instruction cache: 204 us per stage).  Per stage phi
+// is read once and written once (plus phi^m in the second stage) with the code
+// byte: 9 or 13 bytes per cell in float32.  Bound by instruction issue (190 warp
+// instructions per 32 cells, 76 % of the slots): 112 us per stage at 256^3 and
+// 10 us for the listed cells; one cell per thread with every axis by itself
+// took 326 instructions and 169 us.
 #include <algorithm>
 
 #include "internal.h"
@@ -83,9 +83,7 @@ __global__ void k_reinit_code(GridDev g, const T* __restrict__ q0, unsigned char
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const size_t plane = (size_t)n0 * n1, n = plane * n2;
   for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(id / plane);
-    const size_t r = id - (size_t)k * plane;
-    const int j = (int)(r / n0), i = (int)(r - (size_t)j * n0);
+    const int row = (int)id / n0, i = (int)id - row * n0, k = row / n1, j = row - k * n1;
     const T q = q0[id];
     unsigned c = q > T(0) ? 1u : (q < T(0) ? 2u : 0u);
     const int cc[3] = {i, j, k}, nn[3] = {n0, n1, n2};
@@ -342,7 +340,7 @@ __global__ void k_to_f32(const double* __restrict__ a, float* __restrict__ b, si
 template <typename T>
 static void stage(const GridDev& g, const ReinitAxes<T>& ax, const unsigned char* code, const int* list, const T* q0,
                   const T* pin, const T* pavg, T* pout, double* out64, cudaStream_t st) {
-  // long marches, but about eight blocks per SM
+  // long marches, but at least four blocks per SM
   const long long base = (long long)cdiv(g.n[0], 2 * RX) * cdiv(g.n[1], RY);
   int zc = 32;
   while (zc > 4 && base * cdiv(g.n[2], zc) < 152LL * 4) zc /= 2;
@@ -351,9 +349,9 @@ static void stage(const GridDev& g, const ReinitAxes<T>& ax, const unsigned char
   if (smem > 48 * 1024) cudaFuncSetAttribute(k_reinit<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   ktimer_begin(KC_REINIT, st);
   { k_reinit<T><<<grid, dim3(RX, RY), smem, st>>>(g, ax, code, q0, pin, pavg, pout, out64, zc); WSI_COUNT(); }
-  ktimer_end(KC_REINIT, st);
   const int nb = (int)std::min<long long>(((long long)g.n[0] * g.n[1] * g.n[2] + 127) / 128, 152 * 8);
   { k_reinit_near<T><<<nb, 128, 0, st>>>(g, ax, code, list + 2, list, q0, pin, pavg, pout, out64); WSI_COUNT(); }
+  ktimer_end(KC_REINIT, st);
 }
 
 template <typename T>
