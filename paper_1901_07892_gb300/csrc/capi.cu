@@ -1939,11 +1939,9 @@ int wsi_pressure_solve(wsi_ctx* c, const double* y, double* x, double rtol, int 
   double* xb = c->V + n;  // iterate before a learned cycle
   double rn = ynorm, prev = ynorm, rho_plain = 1.0;
   int cycles = 0;
+  double rmean = 0.0;  // of the residual in a closed box
   while (true) {
-    launch_pressure<double>(g, bt, xv, r, st);
-    launch_lincomb(n, 1.0, yv, -1.0, r, 0.0, nullptr, r, st);
-    demean(r);
-    rn = host_norm2(r, n, c->red, st);
+    rn = host_pressure_residual(g, bt, xv, yv, r, c->V + 2 * n, g.open_top ? nullptr : &rmean, st);
     if (!std::isfinite(rn) && !last_learned) return fail(c, WSI_ERR_NAN, "non-finite pressure residual");
     if (last_learned && !(rn <= rho_plain * prev)) {
       cudaMemcpyAsync(xv, xb, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -1959,12 +1957,23 @@ int wsi_pressure_solve(wsi_ctx* c, const double* y, double* x, double rtol, int 
     if (use) cudaMemcpyAsync(xb, xv, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
     if (c->mixed()) {
       MGLevel<float>& L0 = c->P32.lev[0];
-      launch_lincomb_to_f32(n, 1.0 / rn, r, 0.0, nullptr, 0.0, nullptr, L0.b, st);
+      // scaled to order one for float32: by a power of two for the linear cycle,
+      // to norm one for the network and for residuals out of float32's range
+      int e = 0;
+      frexp(rn, &e);
+      const bool pow2 = !learned && e > -40 && e < 100;
+      if (pow2) {
+        launch_shift_scale_f32(n, r, rmean, e, L0.b, st);
+      } else {
+        launch_shift(n, r, rmean, st);
+        launch_lincomb_to_f32(n, 1.0 / rn, r, 0.0, nullptr, 0.0, nullptr, L0.b, st);
+      }
       precond_vcycle<float>(c->P32, c->opts, true, st);
-      launch_lincomb_mix(n, 1.0, xv, rn, L0.x, 0.0, L0.x, xv, st);
+      launch_axpy_f32(n, pow2 ? ldexp(1.0, e) : rn, L0.x, xv, st);
     } else {
       MGLevel<double>& L0 = c->P64.lev[0];
       cudaMemcpyAsync(L0.b, r, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
+      launch_shift(n, L0.b, rmean, st);
       precond_vcycle<double>(c->P64, c->opts, true, st);
       launch_lincomb(n, 1.0, xv, 1.0, L0.x, 0.0, nullptr, xv, st);
     }

@@ -51,6 +51,11 @@ void launch_viscous_residual(const GridDev& g, const Coef<T>& cf, T inv_dt, T th
                              const T* const b[3], T* const r[3], cudaStream_t st);
 template <typename T>
 void launch_pressure(const GridDev& g, const T* const beta[3], const T* p, T* out, cudaStream_t st);
+// r = y - D beta G x on cells; returns its norm, after its mean is removed (and
+// returned in *mean) where mean is given; r itself keeps its mean.  scratch:
+// as many doubles as there are cells, and 8 more
+double host_pressure_residual(const GridDev& g, const double* const beta[3], const double* x, const double* y, double* r,
+                              double* scratch, double* mean, cudaStream_t st);
 template <typename T>
 void launch_grad(const GridDev& g, const T* p, T* const out[3], cudaStream_t st);
 template <typename T>
@@ -133,6 +138,11 @@ void launch_rk_velocities_f32(size_t n, const double* un, const double* unm1, co
                               float* un32, cudaStream_t st);
 void launch_lincomb_mix(size_t n, double a, const double* x, double b, const float* y, double c, const float* z,
                         double* out, cudaStream_t st);
+// y = 2^-e (x - m) and x += 2^e y in float32 / float64, e within the range of
+// float32; x -= m
+void launch_shift_scale_f32(size_t n, const double* x, double m, int e, float* y, cudaStream_t st);
+void launch_axpy_f32(size_t n, double a, const float* y, double* x, cudaStream_t st);
+void launch_shift(size_t n, double* x, double m, cudaStream_t st);
 // z-chunk of the plane-marching stencil kernels for an ex x ey x ez box of
 // points (32 x 8 tiles): long marches, yet about 8 blocks per SM
 int transport_chunk(int ex, int ey, int ez);

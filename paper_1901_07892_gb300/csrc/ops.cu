@@ -397,6 +397,140 @@ void launch_pressure(const GridDev& g, const T* const beta[3], const T* p, T* ou
   { k_pressure<T><<<grid3(g.n[0], g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, beta[0], beta[1], beta[2], p, out); WSI_COUNT(); }
 }
 
+// r = y - D beta G x in float64 with the partials of its sum and square sum.
+// Float64-pipe bound, so every flux beta dx is formed once: along x the upper
+// face comes from the next lane, along y from the next row through shared
+// memory, along z it is carried up the march; a ninth warp forms the fluxes
+// through the tile's upper edges (x: one lane per row, y: one per column).  14
+// operations per cell where five passes (k_pressure, the difference, its sum,
+// the removal of its mean, its norm) took 23, 562 us in k_pressure alone: 495 us at
+// 256^3 (at the float64 rate 14.5 operations take 450).
+static constexpr int QX = 32, QY = 8, QZ = 16;
+// the block's barrier, met from two places of the code (the ninth warp's loop and
+// the others')
+__device__ __forceinline__ void tile_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * (QY + 1)) : "memory"); }
+
+__global__ void __launch_bounds__(32 * (QY + 1)) k_pressure_residual(GridDev g, const double* __restrict__ bx,
+                                                                     const double* __restrict__ by,
+                                                                     const double* __restrict__ bz,
+                                                                     const double* __restrict__ x,
+                                                                     const double* __restrict__ y, double* r,
+                                                                     int zchunk, double* part) {
+  __shared__ double sF[2][QY + 1][32];  // flux through the lower y face
+  __shared__ double sX[2][QY];          // flux through the tile's upper x edge
+  __shared__ double sh[2][QY];
+  const int lane = threadIdx.x, ty = threadIdx.y;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const int x0 = blockIdx.x * QX, y0 = blockIdx.y * QY;
+  const int k0 = blockIdx.z * zchunk, k1 = min(k0 + zchunk, nz);
+  const int i = x0 + lane, j = y0 + ty;
+  const double wx = g.ih2[0], wy = g.ih2[1], wz = g.ih2[2];
+  const size_t pl = (size_t)nx * ny, px = (size_t)(nx + 1) * ny, py = (size_t)nx * (ny + 1);
+  double s1 = 0.0, s2 = 0.0;
+  if (ty == QY) {
+    // upper edges: the row j = y0 + QY, and column x0 + QX of rows y0 + lane
+    const bool row = i < nx && j < ny, col = lane < QY && y0 + lane < ny && x0 + QX < nx;
+    size_t id = row ? (size_t)k0 * pl + (size_t)j * nx + i : 0, iy = row ? fidx(g, 1, i, j, k0) : 0;
+    size_t ic = col ? (size_t)k0 * pl + (size_t)(y0 + lane) * nx + x0 + QX : 0;
+    size_t ix = col ? fidx(g, 0, x0 + QX, y0 + lane, k0) : 0;
+    for (int k = k0; k < k1; ++k) {
+      sF[k & 1][QY][lane] = row ? by[iy] * (x[id] - x[id - nx]) : 0.0;
+      if (lane < QY) sX[k & 1][lane] = col ? bx[ix] * (x[ic] - x[ic - 1]) : 0.0;
+      id += pl;
+      iy += py;
+      ic += pl;
+      ix += px;
+      tile_sync();
+    }
+    tile_sync();
+    if (lane >= 2) return;
+    double a = 0.0;
+    for (int w = 0; w < QY; ++w) a += sh[lane][w];
+    part[2 * (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) + lane] = a;
+    return;
+  }
+  const bool cell = i < nx && j < ny;
+  size_t id = cell ? (size_t)k0 * pl + (size_t)j * nx + i : 0;
+  size_t ix = cell ? fidx(g, 0, i, j, k0) : 0, iy = cell ? fidx(g, 1, i, j, k0) : 0;
+  double xc = cell ? x[id] : 0.0, fz = 0.0;
+  if (cell && k0 > 0) fz = bz[id] * (xc - x[id - pl]);
+  for (int k = k0; k < k1; ++k) {
+    const double xn = cell && k + 1 < nz ? x[id + pl] : 0.0;
+    double fx = 0.0, fy = 0.0;
+    if (cell && i > 0) fx = bx[ix] * (xc - x[id - 1]);
+    if (cell && j > 0) fy = by[iy] * (xc - x[id - nx]);
+    sF[k & 1][ty][lane] = fy;
+    double fxr = __shfl_down_sync(0xffffffffu, fx, 1);  // (zero beyond the grid)
+    tile_sync();
+    if (cell) {
+      if (lane == 31) fxr = sX[k & 1][ty];
+      const double fyr = sF[k & 1][ty + 1][lane];
+      double fzr = 0.0;
+      if (k + 1 < nz) fzr = bz[id + pl] * (xn - xc);
+      else if (g.open_top) fzr = -2.0 * bz[id + pl] * xc;  // ghost -p above the open top
+      const double v = fma(fx - fxr, wx, fma(fy - fyr, wy, fma(fz - fzr, wz, y[id])));
+      r[id] = v;
+      s1 += v;
+      s2 = fma(v, v, s2);
+      fz = fzr;
+      xc = xn;
+    }
+    id += pl;
+    ix += px;
+    iy += py;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s1 += __shfl_down_sync(0xffffffffu, s1, o);
+    s2 += __shfl_down_sync(0xffffffffu, s2, o);
+  }
+  if (lane == 0) {
+    sh[0][ty] = s1;
+    sh[1][ty] = s2;
+  }
+  tile_sync();
+}
+
+__global__ void __launch_bounds__(1024) k_reduce_pairs(const double* __restrict__ part, size_t n, double* out) {
+  __shared__ double sh[2][32];
+  double a = 0.0, b = 0.0;
+  for (size_t t = threadIdx.x; t < n; t += 1024) {
+    a += part[2 * t];
+    b += part[2 * t + 1];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    b += __shfl_down_sync(0xffffffffu, b, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = a;
+    sh[1][threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double s = 0.0;
+    for (int w = 0; w < 32; ++w) s += sh[threadIdx.x][w];
+    out[threadIdx.x] = s;
+  }
+}
+
+double host_pressure_residual(const GridDev& g, const double* const beta[3], const double* x, const double* y, double* r,
+                              double* scratch, double* mean, cudaStream_t st) {
+  const int bx = cdiv(g.n[0], QX), by = cdiv(g.n[1], QY);
+  int zc = QZ;  // shorter marches where the grid is small
+  while (zc > 2 && (long long)bx * by * cdiv(g.n[2], zc) < 152 * 4) zc /= 2;
+  const dim3 grid(bx, by, cdiv(g.n[2], zc));
+  const size_t nb = (size_t)grid.x * grid.y * grid.z;
+  { k_pressure_residual<<<grid, dim3(32, QY + 1), 0, st>>>(g, beta[0], beta[1], beta[2], x, y, r, zc, scratch + 2); WSI_COUNT(); }
+  { k_reduce_pairs<<<1, 1024, 0, st>>>(scratch + 2, nb, scratch); WSI_COUNT(); }
+  double h[2] = {0.0, 0.0};
+  cudaMemcpyAsync(h, scratch, sizeof(h), cudaMemcpyDeviceToHost, st);
+  cudaStreamSynchronize(st);
+  if (!mean) return sqrt(h[1]);
+  const double n = (double)g.n[0] * g.n[1] * g.n[2];
+  *mean = h[0] / n;
+  return sqrt(fmax(h[1] - h[0] * *mean, h[1] == h[1] ? 0.0 : h[1]));
+}
+
 template <int C, typename T>
 __global__ void k_grad(GridDev g, const T* __restrict__ p, T* out) {
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 
+#include "df.cuh"
 #include "internal.h"
 
 namespace wsi {
@@ -496,6 +497,37 @@ __global__ void k_lincomb_mix(size_t n, double a, const double* __restrict__ x, 
 void launch_lincomb_mix(size_t n, double a, const double* x, double b, const float* y, double c, const float* z,
                         double* out, cudaStream_t st) {
   { k_lincomb_mix<<<lc_blocks(n), 256, 0, st>>>(n, a, x, b, y, c, z, out); WSI_COUNT(); }
+}
+
+// The mean is taken off in float32 pairs and the scale is a power of two, so
+// the result carries one rounding and no float64 operation (1/64 of the
+// float32 rate) is spent.
+__global__ void k_shift_scale_f(size_t n, const double* __restrict__ x, dfl m, float f, float* y) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
+    const dfl a = df_split(x[t]);
+    float s, e;
+    two_sum(a.h, -m.h, s, e);
+    y[t] = f * (s + (e + (a.l - m.l)));
+  }
+}
+void launch_shift_scale_f32(size_t n, const double* x, double m, int e, float* y, cudaStream_t st) {
+  dfl d;
+  d.h = (float)m;
+  d.l = (float)(m - (double)d.h);
+  { k_shift_scale_f<<<lc_blocks(n), 256, 0, st>>>(n, x, d, ldexpf(1.0f, -e), y); WSI_COUNT(); }
+}
+__global__ void k_axpy_f(size_t n, double a, const float* __restrict__ y, double* x) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
+    x[t] = fma(a, f2d_fast(y[t]), x[t]);
+}
+void launch_axpy_f32(size_t n, double a, const float* y, double* x, cudaStream_t st) {
+  { k_axpy_f<<<lc_blocks(n), 256, 0, st>>>(n, a, y, x); WSI_COUNT(); }
+}
+__global__ void k_shift(size_t n, double* x, double m) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) x[t] -= m;
+}
+void launch_shift(size_t n, double* x, double m, cudaStream_t st) {
+  { k_shift<<<lc_blocks(n), 256, 0, st>>>(n, x, m); WSI_COUNT(); }
 }
 
 // ================================================================ level set
