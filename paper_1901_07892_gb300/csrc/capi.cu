@@ -95,7 +95,7 @@ struct wsi_ctx {
   double *vel = nullptr, *vel_old = nullptr, *p = nullptr, *phi = nullptr, *psi = nullptr;
   // step scratch
   double *vel_k = nullptr, *vel_half = nullptr, *u1 = nullptr, *u2 = nullptr, *rs1 = nullptr, *rs2 = nullptr,
-         *R = nullptr, *Cc = nullptr, *phi_k = nullptr, *phi_new = nullptr, *phi_half = nullptr, *psi_k = nullptr,
+         *Cc = nullptr, *phi_k = nullptr, *phi_new = nullptr, *phi_half = nullptr, *psi_k = nullptr,
          *psi_new = nullptr, *b = nullptr, *x = nullptr, *rho_cc_tmp = nullptr;
   // Krylov
   int m = 20;
@@ -148,7 +148,7 @@ struct wsi_ctx {
   float* in_gs32 = nullptr;
   // float32 shadows of the explicitly transported fields (mixed path)
   float *vn32 = nullptr, *u1_32 = nullptr, *u2_32 = nullptr, *rn32 = nullptr, *r1_32 = nullptr, *r2_32 = nullptr,
-        *R32 = nullptr, *C32 = nullptr, *vh32 = nullptr, *phih32 = nullptr, *mu_cc_n32 = nullptr,
+        *C32 = nullptr, *vh32 = nullptr, *phih32 = nullptr, *mu_cc_n32 = nullptr,
         *mu_e_n32[3] = {nullptr, nullptr, nullptr};
   bool mixed() const { return desc.precision == WSI_PREC_MIXED; }
 };
@@ -256,29 +256,6 @@ PhaseConst phase_const(wsi_ctx* c) {
   pc.inv_mu = c->inv_mu;
   phase_tables(pc);
   return pc;
-}
-
-// 1/a in double-float arithmetic: float32 reciprocal r, residual 1 - a r
-// formed with a split into (hi, lo) and fused multiply-adds, one Newton step;
-// one float64 addition forms the result (~1e-14 relative).  Zero,
-// subnormal-range and non-finite a take the float64 division.
-__global__ void k_recip(size_t n, const double* __restrict__ a, double* b) {
-  size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const double v = a[t];
-  const dfl x = df_split(v);
-  if (!(fabsf(x.h) > 1e-30f) || !(fabsf(x.h) < 1e30f)) {
-    b[t] = 1.0 / v;
-    return;
-  }
-  const float r = 1.0f / x.h;
-  // e = 1 - x r, exactly enough: fma for the leading product, lo part plainly
-  const float e = fmaf(-x.h, r, 1.0f) - x.l * r;
-  b[t] = df_to_double(quick_two_sum(r, r * e));
-}
-
-void recip(wsi_ctx* c, const double* a, double* b, size_t n) {
-  if (n) { k_recip<<<cdiv(n, 256), 256, 0, c->st>>>(n, a, b); WSI_COUNT(); }
 }
 
 int copy_in(wsi_ctx* c, double* dst, const double* src, size_t n) {
@@ -617,8 +594,7 @@ void transport_stage(wsi_ctx* c, int k, double dt, const double* un, const doubl
       launch_lincomb(nv, 1.0, uk, 0.0, nullptr, 0.0, nullptr, c->u1, st);
       launch_lincomb(nv, 0.375, uk, 0.75, un, -0.125, unm1, c->u2, st);
     }
-    double *R[3], *Cq[3], *r1[3], *r2[3];
-    parts(c, c->R, R);
+    double *Cq[3], *r1[3], *r2[3];
     parts(c, c->Cc, Cq);
     parts(c, c->rs1, r1);
     parts(c, c->rs2, r2);
@@ -627,23 +603,14 @@ void transport_stage(wsi_ctx* c, int k, double dt, const double* un, const doubl
     cparts(c, (const double*)c->u1, cu1);
     cparts(c, (const double*)c->u2, cu2);
     const double* crn[3] = {c->rho_n[0], c->rho_n[1], c->rho_n[2]};
-    if (!reuse_stage1) {
-      launch_transport_flux<double>(g, cun, crn, false, R, st);
-      for (int d = 0; d < 3; ++d) launch_lincomb(fsize(g, d), 1.0, c->rho_n[d], -dt, R[d], 0.0, nullptr, r1[d], st);
-    }
+    if (!reuse_stage1) launch_transport_stage<double>(g, cun, crn, 1.0, nullptr, 0.0, -dt, r1, st);
     const double* cr1[3] = {r1[0], r1[1], r1[2]};
-    launch_transport_flux<double>(g, cu1, cr1, false, R, st);
-    for (int d = 0; d < 3; ++d)
-      launch_lincomb(fsize(g, d), 0.75, c->rho_n[d], 0.25, r1[d], -0.25 * dt, R[d], r2[d], st);
+    launch_transport_stage<double>(g, cu1, cr1, 0.75, crn, 0.25, -0.25 * dt, r2, st);
     const double* cr2[3] = {r2[0], r2[1], r2[2]};
-    launch_transport_flux<double>(g, cu2, cr2, false, R, st);
-    for (int d = 0; d < 3; ++d)
-      launch_lincomb(fsize(g, d), 1.0 / 3.0, c->rho_n[d], 2.0 / 3.0, r2[d], -2.0 / 3.0 * dt, R[d], c->rho_face[d],
-                     st);
-    launch_transport_flux<double>(g, cu2, cr2, true, Cq, st, (const double*)g2);
+    launch_transport_last<double>(g, cu2, cr2, 1.0 / 3.0, crn, 2.0 / 3.0, -2.0 / 3.0 * dt, c->rho_face, c->beta, Cq, st,
+                                  (const double*)g2);
   } else {
-    float *R[3], *Cq[3], *r1[3], *r2[3], *rn[3];
-    parts(c, c->R32, R);
+    float *Cq[3], *r1[3], *r2[3], *rn[3];
     parts(c, c->C32, Cq);
     parts(c, c->r1_32, r1);
     parts(c, c->r2_32, r2);
@@ -656,23 +623,18 @@ void transport_stage(wsi_ctx* c, int k, double dt, const double* un, const doubl
     cparts(c, (const float*)c->u1_32, cu1);
     cparts(c, (const float*)c->u2_32, cu2);
     cparts(c, (const float*)c->rn32, crn);
+    const double* crn64[3] = {c->rho_n[0], c->rho_n[1], c->rho_n[2]};
     if (!reuse_stage1) {
       for (int d = 0; d < 3; ++d)
         launch_lincomb_to_f32(fsize(g, d), 1.0, c->rho_n[d], 0.0, nullptr, 0.0, nullptr, rn[d], st);
-      launch_transport_flux<float>(g, cvn, crn, false, R, st);
-      launch_lincomb_f32(nv, 1.0f, c->rn32, (float)-dt, c->R32, 0.0f, nullptr, c->r1_32, st);
+      launch_transport_stage<float>(g, cvn, crn, 1.0, nullptr, 0.0, -dt, r1, st);
     }
     const float* cr1[3] = {r1[0], r1[1], r1[2]};
-    launch_transport_flux<float>(g, cu1, cr1, false, R, st);
-    launch_lincomb_f32(nv, 0.75f, c->rn32, 0.25f, c->r1_32, (float)(-0.25 * dt), c->R32, c->r2_32, st);
+    launch_transport_stage<float>(g, cu1, cr1, 0.75, crn, 0.25, -0.25 * dt, r2, st);
     const float* cr2[3] = {r2[0], r2[1], r2[2]};
-    launch_transport_flux<float>(g, cu2, cr2, false, R, st);
-    for (int d = 0; d < 3; ++d)
-      launch_lincomb_mix(fsize(g, d), 1.0 / 3.0, c->rho_n[d], 2.0 / 3.0, r2[d], -2.0 / 3.0 * dt, R[d],
-                         c->rho_face[d], st);
-    launch_transport_flux<float>(g, cu2, cr2, true, Cq, st, (const float*)g2);
+    launch_transport_last<float>(g, cu2, cr2, 1.0 / 3.0, crn64, 2.0 / 3.0, -2.0 / 3.0 * dt, c->rho_face, c->beta, Cq,
+                                 st, (const float*)g2);
   }
-  for (int d = 0; d < 3; ++d) recip(c, c->rho_face[d], c->beta[d], fsize(g, d));
 }
 
 // phi_out = phi_n - dt Q(u_half, phi_half) with u_half = (vk + vn)/2 and
@@ -765,14 +727,14 @@ int nc_convection(wsi_ctx* c, int k) {
     cparts(c, (const float*)c->vh32, vh);
     cparts(c, (const float*)c->ones, one);
     parts(c, c->C32, N);
-    launch_transport_flux<float>(g, vh, one, true, N, st, (const float*)gh);
+    launch_transport_conv<float>(g, vh, one, N, st, (const float*)gh);
   } else {
     const double *vh[3], *one[3];
     double* N[3];
     cparts(c, (const double*)c->vel_half, vh);
     cparts(c, (const double*)c->ones, one);
     parts(c, c->Cc, N);
-    launch_transport_flux<double>(g, vh, one, true, N, st, (const double*)gh);
+    launch_transport_conv<double>(g, vh, one, N, st, (const double*)gh);
   }
   return WSI_OK;
 }
@@ -902,7 +864,6 @@ int wsi_create_grid(const wsi_grid_desc* d, void* stream, wsi_ctx** out) {
   c->u2 = A(c->nvel);
   c->rs1 = A(c->nvel);
   c->rs2 = A(c->nvel);
-  c->R = A(c->nvel);
   c->Cc = A(c->nvel);
   c->phi_k = A(c->ncell);
   c->phi_new = A(c->ncell);
@@ -925,7 +886,6 @@ int wsi_create_grid(const wsi_grid_desc* d, void* stream, wsi_ctx** out) {
     c->rn32 = F(c->nvel);
     c->r1_32 = F(c->nvel);
     c->r2_32 = F(c->nvel);
-    c->R32 = F(c->nvel);
     c->C32 = F(c->nvel);
     c->vh32 = F(c->nvel);
     c->phih32 = F(c->ncell);

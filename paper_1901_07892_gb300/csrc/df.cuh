@@ -130,6 +130,19 @@ __device__ __forceinline__ dfl df_sqrt(dfl x) {
   return quick_two_sum(s, d.h / (2.0f * s));
 }
 
+// 1/v in double-float arithmetic: float32 reciprocal r, residual 1 - v r
+// formed with a split into (hi, lo) and fused multiply-adds, one Newton step;
+// one float64 addition forms the result (~1e-14 relative).  Zero,
+// subnormal-range and non-finite v take the float64 division.
+__device__ __forceinline__ double recip_df(double v) {
+  const dfl x = df_split(v);
+  if (!(fabsf(x.h) > 1e-30f) || !(fabsf(x.h) < 1e30f)) return 1.0 / v;
+  const float r = 1.0f / x.h;
+  // e = 1 - x r, exactly enough: fma for the leading product, lo part plainly
+  const float e = fmaf(-x.h, r, 1.0f) - x.l * r;
+  return df_to_double(quick_two_sum(r, r * e));
+}
+
 // Unnormalised head/tail pairs: a value is h + t with the head h formed
 // error-free (exact differences by Knuth's two-sum, exact products by fused
 // multiply-add) and everything smaller gathered in the float32 tail t,

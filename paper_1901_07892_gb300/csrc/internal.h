@@ -119,12 +119,24 @@ template <typename T>
 void launch_viscous_rbgs(const GridDev& g, const Coef<T>& cf, T inv_dt, T theta, T* const q[3], const T* const b[3],
                          int color, cudaStream_t st);
 
-// transport.cu (Sec. 4.2.2): R or C on all three face arrays, storage and
-// arithmetic in T; inlet_w: the tangential data of vel's w on a Dirichlet
-// inlet's x- plane ((nz+1) x ny, used for C), or null
+// transport.cu (Sec. 4.2.2): the divergence R of the mass flux of rho with vel,
+// and C of the momentum flux, on all three face arrays, storage and arithmetic
+// in T; inlet_w: the tangential data of vel's w on a Dirichlet inlet's x- plane
+// ((nz+1) x ny, used for C), or null
+// a Runge-Kutta stage: out = a base + b rho + c R (base null: rho + c R)
 template <typename T>
-void launch_transport_flux(const GridDev& g, const T* const vel[3], const T* const rho[3], bool with_velocity,
-                           T* const out[3], cudaStream_t st, const T* inlet_w = nullptr);
+void launch_transport_stage(const GridDev& g, const T* const vel[3], const T* const rho[3], double a,
+                            const T* const base[3], double b, double c, T* const out[3], cudaStream_t st);
+// the last stage in float64, rho_out = a base + b rho + c R and its reciprocal
+// beta_out, and C into conv
+template <typename T>
+void launch_transport_last(const GridDev& g, const T* const vel[3], const T* const rho[3], double a,
+                           const double* const base[3], double b, double c, double* const rho_out[3],
+                           double* const beta_out[3], T* const conv[3], cudaStream_t st, const T* inlet_w);
+// C alone
+template <typename T>
+void launch_transport_conv(const GridDev& g, const T* const vel[3], const T* const rho[3], T* const conv[3],
+                           cudaStream_t st, const T* inlet_w);
 // out = a*x + b*y + c*z elementwise over n (any of y, z may be null)
 void launch_lincomb(size_t n, double a, const double* x, double b, const double* y, double c, const double* z,
                     double* out, cudaStream_t st);

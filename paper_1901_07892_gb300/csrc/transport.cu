@@ -27,24 +27,40 @@ static constexpr int BX = 32, BY = 8;
 
 // Division-free bounded CUI: with num = qC - qU and den = qD - qU,
 // t = num/den lies in a branch interval iff num*sign(den) lies in den-scaled
-// bounds, and qU + t_f den = qU + {3 num, 5 num/6 + den/3, den, num}.
-template <typename T>
-__device__ __forceinline__ T cui(T qU, T qC, T qD) {
-  T den = qD - qU;
-  T num = qC - qU;
-  if (den == T(0)) return qC;
-  T a = den > T(0) ? num : -num;  // num * sign(den)
-  T D = den > T(0) ? den : -den;  // t = a / D
-  T f;
-  if (a > T(0) && T(13) * a <= T(2) * D)
-    f = T(3) * num;
-  else if (T(13) * a > T(2) * D && T(5) * a <= T(4) * D)
-    f = num * T(5.0 / 6.0) + den * T(1.0 / 3.0);
-  else if (T(5) * a > T(4) * D && a <= D)
-    f = den;
-  else
-    f = num;
-  return qU + f;
+// bounds, and qU + t_f den = qU + {3 num, 5 num/6 + den/3, den, num}.  The
+// bounds 2/13 and 4/5 are tested as 6.5 a <= D and 1.25 a <= D (powers of two
+// of 13 a <= 2 D and 5 a <= 4 D: the same roundings, two products less); none
+// holds for NaN, which takes the last case.
+// Without branches: neighbouring cells take different cases.  up: the flow is
+// in the positive direction; there the steep case rounds once, against it the
+// product by itself (float32 results are kept to the bit, whichever way the
+// cases are told apart).
+__device__ __forceinline__ float cui(float qU, float qC, float qD, bool up) {
+  const float den = qD - qU, num = qC - qU;
+  // num * sign(den), so that t = a / |den| (den = 0 is told apart below)
+  const float a = __int_as_float(__float_as_int(num) ^ (__float_as_int(den) & 0x80000000)), D = fabsf(den);
+  const bool p = a > 0.0f, c1 = p && 6.5f * a <= D, c2 = p && 1.25f * a <= D, c3 = p && a <= D;
+  const float f = c1 ? 3.0f * num : (c2 ? num * (float)(5.0 / 6.0) + den * (float)(1.0 / 3.0) : (c3 ? den : num));
+  const float q = c1 && up ? fmaf(3.0f, num, qU) : qU + f;
+  return den == 0.0f ? qC : q;
+}
+// float64: the comparisons are made on the bit patterns (as signed integers a
+// value of either sign orders correctly against one that is not negative), and
+// the cases differ in two factors: seven operations on the narrow pipe
+__device__ __forceinline__ double cui(double qU, double qC, double qD, bool) {
+  const double den = qD - qU, num = qC - qU;
+  const long long TOP = (long long)0x8000000000000000ull;
+  const long long bd = __double_as_longlong(den), bn = __double_as_longlong(num);
+  const bool pos = bd > 0;  // (den > 0; zero and NaN below)
+  const long long D = pos ? bd : bd ^ TOP;
+  const double a = __longlong_as_double(pos ? bn : bn ^ TOP);
+  const long long i0 = pos ? bn : bn ^ TOP, i1 = __double_as_longlong(6.5 * a), i2 = __double_as_longlong(1.25 * a);
+  const bool c1 = i0 > 0 && i1 <= D, c2 = i1 > D && i2 <= D, c3 = i2 > D && i0 <= D;
+  const long long INF = 0x7FF0000000000000ll;
+  if ((bd & ~TOP) > INF) return qU + num;  // den is NaN
+  const double A = c1 ? 3.0 : (c2 ? 5.0 / 6.0 : (c3 ? 0.0 : 1.0));
+  const double B = c2 ? 1.0 / 3.0 : (c3 ? 1.0 : 0.0);
+  return (bd & ~TOP) == 0 ? qC : qU + fma(A, num, B * den);
 }
 
 // Entry m of the C-face array along axis D extended by two ghost layers: the
@@ -82,7 +98,8 @@ __device__ __forceinline__ int mirror_index(const GridDev& g, int m, T& s) {
 // limited value from the four taps for advective velocity adv
 template <typename T>
 __device__ __forceinline__ T lim4(T t0, T t1, T t2, T t3, T adv) {
-  return adv > T(0) ? cui<T>(t0, t1, t2) : cui<T>(t3, t2, t1);
+  const bool pos = adv > T(0);
+  return cui(pos ? t0 : t3, pos ? t1 : t2, pos ? t2 : t1, pos);
 }
 
 // advective velocity at the D-direction CV face at position m of the C-face
@@ -116,50 +133,102 @@ __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_gro
 template <int N>
 __device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Per z-plane the block stages the transported field (and, for C, the
-// velocity component) of its tile with a two-entry halo in x and y into a
-// ring of NPL plane slots in shared memory, by asynchronous copies issued
-// three planes ahead (the ghosts beyond walls are mirrored through the copies'
-// source addresses; the velocity ghosts' signs, and the inlet data across a
-// Dirichlet inlet, are applied by the staging thread once its copies have
-// landed).  The four limiter taps of every x- and y-flux then come from plane
-// k's slot, the z taps of a thread's own column from the slots of planes
-// k-1 .. k+2 (a plane beyond a wall reads its mirror image's slot with the
-// mirror's sign).  Advective velocities are loaded one plane ahead into
-// registers.  Two block barriers per plane: one publishes the plane, one the
-// x- and y-fluxes.
-static constexpr int NPL = 6;  // planes k-2 .. k+3
+// What a launch does with the divergence R of the mass flux of rho, and that of
+// the momentum flux:
+// TR_STAGE  out = a base + b rho + c R (base null: rho + c R), a Runge-Kutta
+//           stage of the density in T
+// TR_CONV   conv = the momentum flux' divergence alone
+// TR_LAST   both, with the velocity's limiter on the same mass flux: the last
+//           stage in float64 (rho64 = a64 base64 + b64 rho + c64 R, beta64 its
+//           reciprocal) and conv
+enum { TR_STAGE, TR_CONV, TR_LAST };
+template <typename T>
+struct TransportOut {
+  const T* base;
+  T a, b, c;
+  T* out;
+  const double* base64;
+  double a64, b64, c64;
+  double *rho64, *beta64;
+  T* conv;
+};
+
+// a x + b y + c z and y + c z with the roundings of the elementwise sums in
+// float32 (the first product is the one that is fused) and float64 (the last)
+__device__ __forceinline__ float stage_sum(float a, float x, float b, float y, float c, float z) {
+  return fmaf(c, z, fmaf(a, x, __fmul_rn(b, y)));
+}
+__device__ __forceinline__ double stage_sum(double a, double x, double b, double y, double c, double z) {
+  return fma(c, z, fma(b, y, a * x));
+}
+__device__ __forceinline__ float stage_sum(float y, float c, float z) { return __fadd_rn(y, __fmul_rn(c, z)); }
+__device__ __forceinline__ double stage_sum(double y, double c, double z) { return fma(c, z, y); }
+
+__device__ __forceinline__ double stage64(double a, double x, double b, float y, double c, float z) {
+  return a * x + b * f2d_fast(y) + c * f2d_fast(z);
+}
+__device__ __forceinline__ double stage64(double a, double x, double b, double y, double c, double z) {
+  return fma(c, z, fma(b, y, a * x));
+}
+
+// A block advances a tile of 32 x 8 faces up a z-chunk.  Per plane the tile of
+// the transported field (and, for the convective term, of the velocity
+// component) with a two-entry halo in x and y is in a ring of NPL plane slots in
+// shared memory, filled by asynchronous copies up to NPL planes ahead (ghosts
+// beyond walls are mirrored through the copies' source addresses; the velocity
+// ghosts' signs, and the inlet data across a Dirichlet inlet, are applied by the
+// thread that copied them once the copies have landed).  Every flux is formed
+// once: a thread forms the three through the upper faces of its entry, a ninth
+// warp those through the tile's lower x and y edges; the lower x-flux comes by
+// shuffle, the lower y-flux through shared memory, the lower z-flux is the one of
+// the plane before, as the z taps are carried in registers.  The raw advective
+// velocities are loaded one plane ahead.  One barrier per plane: it publishes
+// the edge and y-fluxes of plane k and the staged plane k + 3.  Faces of the last
+// column (C = 0) or row (C = 1) lie on a wall, where R = 0: where they would
+// start a tile of their own their neighbours' threads write them.
+// Bound by instruction issue (82 % of the slots at 256 x 256 x 64, the limiters'
+// compares and selects a third of the instructions).  At 256^3 in float32 a stage
+// takes 166 us per component with its sum, the last stage 345 us with the
+// momentum flux, its sum and the reciprocal.  One launch per flux kind, edges by
+// the first lane and row and two branches per limiter took 240-274 and 400 us,
+// formed the last stage's mass flux twice, and the sums took 26, 106 and 50 us
+// more.  In float64 (128 x 64 x 64): 76 and 151 us, before 217 and 456.
+static constexpr int TNT = BX * (BY + 1);
 
 // inl (C == 2 with the velocity only, else null): tangential data of w on
 // the x- plane of a Dirichlet inlet, (nz+1) x ny; the ghosts of w across it
 // are then 2 inl - (mirror image)
-template <int C, bool WITHV, typename T>
-__global__ void __launch_bounds__(BX* BY) k_transport(GridDev g, CVel<T> vel, const T* __restrict__ rho, T* out,
-                                                      int zchunk, const T* __restrict__ inl) {
-  constexpr int HX = BX + 4, HY = BY + 4, NS = (HX * HY + BX * BY - 1) / (BX * BY);
-  constexpr int PL = HX * HY;
+template <int C, int MODE, typename T>
+__global__ void __launch_bounds__(TNT, sizeof(T) == 4 ? (MODE == TR_STAGE ? 4 : 3) : 2)
+    k_transport(GridDev g, CVel<T> vel, const T* __restrict__ rho, TransportOut<T> o, int zchunk,
+                const T* __restrict__ inl) {
+  constexpr bool V = MODE != TR_STAGE;
+  constexpr int NF = MODE == TR_LAST ? 2 : 1;   // fluxes handed on: mass, momentum
+  constexpr int NPL = sizeof(T) == 4 ? 8 : 4;   // ring slots
+  constexpr int HX = BX + 4, HY = BY + 4, PL = HX * HY, NS = (PL + TNT - 1) / TNT;
   __shared__ __align__(16) T sR[NPL][PL];
-  __shared__ __align__(16) T sQ[WITHV ? NPL : 1][WITHV ? PL : 1];
-  __shared__ T sFx[BY][BX + 1];
-  __shared__ T sFy[BY + 1][BX];
+  __shared__ __align__(16) T sQ[V ? NPL : 1][V ? PL : 1];
+  __shared__ T sFy[2][NF][BY + 1][BX];
+  __shared__ T sXe[2][NF][BY];
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
+  const bool edge = ty == BY;
+  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
   const int i = x0 + tx, j = y0 + ty;
   const int e0 = ext(g, C, 0), e1 = ext(g, C, 1), e2 = ext(g, C, 2);
-  const bool inside = i < e0 && j < e1;
+  const bool inside = !edge && i < e0 && j < e1;
   const int k0 = blockIdx.z * zchunk;
   const int k1 = min(k0 + zchunk, e2);
-  const int ox = (C == 0) ? -1 : 0, oy = (C == 1) ? -1 : 0, oz = (C == 2) ? -1 : 0;
   const size_t plane = (size_t)e0 * e1;
   const T* __restrict__ qc = vel.q[C];
   // staged entries of this thread: in-plane offset (mirrored) and velocity sign
   int soff[NS];
   T ssg[NS];
-  constexpr bool INL = C == 2 && WITHV;
+  constexpr bool INL = C == 2 && V;
   int sinl[INL ? NS : 1];  // inlet data row of an x-ghost entry, else -1
 #pragma unroll
   for (int r = 0; r < NS; ++r) {
-    const int t = tid + r * BX * BY;
+    const int t = tid + r * TNT;
     soff[r] = -1;
     ssg[r] = T(1);
     if (INL) sinl[r] = -1;
@@ -173,185 +242,203 @@ __global__ void __launch_bounds__(BX* BY) k_transport(GridDev g, CVel<T> vel, co
       if (INL && inl && x0 - 2 + hx < 0) sinl[r] = my;
     }
   }
-  // ring slot of plane p (k0 - 2 <= p; planes k - 2 .. k + 3 are distinct)
-  auto slot = [&](int p) { return (p - k0 + 2) % NPL; };
-  // copies of plane p into its slot (planes outside the array: none); one
-  // group per call
+  // copies of plane p (k0 <= p; above the array its mirror image) into its slot;
+  // one group per call
   auto issue = [&](int p) {
-    if (p >= 0 && p < e2) {
-      const int s = slot(p);
+    if (p <= k1 + 1) {
+      const int s = (p - k0) & (NPL - 1);
+      T sz;
+      const size_t pz = (size_t)mirror_index<C, 2, T>(g, p, sz) * plane;
 #pragma unroll
       for (int r = 0; r < NS; ++r) {
-        const int t = tid + r * BX * BY;
+        const int t = tid + r * TNT;
         if (soff[r] >= 0) {
-          const size_t a = (size_t)p * plane + soff[r];
-          cpa<T>(&sR[s][t], rho + a);
-          if (WITHV) cpa<T>(&sQ[WITHV ? s : 0][WITHV ? t : 0], qc + a);
+          cpa<T>(&sR[s][t], rho + pz + soff[r]);
+          if (V) cpa<T>(&sQ[V ? s : 0][V ? t : 0], qc + pz + soff[r]);
         }
       }
     }
     cpa_commit();
   };
   // signs and inlet data of this thread's entries of plane p, once landed
+  // (planes above the array: only their inner columns are read)
   auto fix = [&](int p) {
-    if (!WITHV || p < 0 || p >= e2) return;
-    const int s = slot(p);
+    if (!V || p >= e2 || p > k1 + 1) return;
+    const int s = (p - k0) & (NPL - 1);
 #pragma unroll
     for (int r = 0; r < NS; ++r) {
-      const int t = tid + r * BX * BY;
+      const int t = tid + r * TNT;
       if (soff[r] < 0) continue;
       const bool inl_here = INL && sinl[INL ? r : 0] >= 0;
       if (ssg[r] == T(1) && !inl_here) continue;
-      T q = ssg[r] * sQ[WITHV ? s : 0][WITHV ? t : 0];
+      T q = ssg[r] * sQ[V ? s : 0][V ? t : 0];
       if (inl_here) q += T(2) * inl[(size_t)p * e1 + sinl[INL ? r : 0]];
-      sQ[WITHV ? s : 0][WITHV ? t : 0] = q;
+      sQ[V ? s : 0][V ? t : 0] = q;
     }
   };
-  // z taps of this thread's column at plane m (mirrored beyond the walls)
-  const int own = (ty + 2) * HX + (tx + 2);
-  auto ztap = [&](int m, T& r_, T& q_) {
-    T sz;
-    const int mm = mirror_index<C, 2, T>(g, m, sz);
-    const int s = slot(mm);
-    r_ = sR[s][own];
-    q_ = WITHV ? sz * sQ[WITHV ? s : 0][WITHV ? own : 0] : T(0);
-  };
-  // fluxes this thread forms at plane k, and their advective velocities: the
-  // two entries of each are found at offsets that move by one z-level of
-  // their array per plane (computed once; 32-bit, every array holds fewer
-  // than 2^31 entries)
-  struct Adv {
-    T xh, xl, yh, yl, zh;
-  };
-  const int mxh = i + ox + 1, mxl = i + ox, myh = j + oy + 1, myl = j + oy;
-  const bool fxh0 = inside && (C != 0 || mxh <= g.n[0] - 1), fxl0 = inside && tx == 0 && (C != 0 || mxl >= 0);
-  const bool fyh0 = inside && (C != 1 || myh <= g.n[1] - 1), fyl0 = inside && ty == 0 && (C != 1 || myl >= 0);
-  // offset at level k0 of the first entry, and the distance to the second
-  auto adv_off = [&](int D, int m, int& d) -> int {
-    int a[3] = {clampi(i, 0, g.n[0]), clampi(j, 0, g.n[1]), k0};
-    a[D] = m;
-    if (C == D) {
-      d = C == 0 ? 1 : (C == 1 ? g.n[0] : g.n[0] * g.n[1]);
-      return (int)fidx(g, C, a[0], a[1], a[2]);
-    }
-    d = -(C == 0 ? 1 : (C == 1 ? (g.n[0] + (D == 0)) : (g.n[0] + (D == 0)) * (g.n[1] + (D == 1))));
-    return (int)fidx(g, D, a[0], a[1], a[2]);
-  };
-  int dxh = 0, dxl = 0, dyh = 0, dyl = 0, dzh = 0;
-  const int oxh = fxh0 ? adv_off(0, mxh, dxh) : 0, oxl = fxl0 ? adv_off(0, mxl, dxl) : 0;
-  const int oyh = fyh0 ? adv_off(1, myh, dyh) : 0, oyl = fyl0 ? adv_off(1, myl, dyl) : 0;
-  const int ozh = inside ? adv_off(2, k0 + oz + 1, dzh) : 0;
-  // one z-level of the u, v, w arrays
-  const int lx = (g.n[0] + 1) * g.n[1], ly = g.n[0] * (g.n[1] + 1), lz = g.n[0] * g.n[1];
+  // The entries whose upper x- and y-fluxes this thread forms: its own, in the
+  // ninth warp those below the tile's edges; whether there is a flux at all (not
+  // through a wall, nor for a face on a wall), and where its two advective
+  // velocities are: offsets at level k0 that move by one level of their array
+  // per plane (32-bit: every array holds fewer than 2^31 entries)
+  const int xi = edge ? x0 - 1 : i, xj = edge ? y0 + (tx & (BY - 1)) : j, yj = edge ? y0 - 1 : j;
+  const int mx = xi + (C == 0 ? 0 : 1), my = yj + (C == 1 ? 0 : 1);
+  const bool wi = i == 0 || i == n0, wj = j == 0 || j == n1;
+  const bool fx = (edge ? tx < BY : i < e0) && xj < e1 && (C != 0 || (mx >= 0 && mx < n0)) &&
+                  (C != 1 || (xj != 0 && xj != n1));
+  const bool fy = i < e0 && yj < e1 && (C != 1 || (my >= 0 && my < n1)) && (C != 0 || !wi);
+  const bool fz = inside && (C != 0 || !wi) && (C != 1 || !wj);
+  const int lx = (n0 + 1) * n1, ly = n0 * (n1 + 1), lz = n0 * n1;  // one z-level of u, v, w
+  const int dx = C == 0 ? 1 : (C == 1 ? -(n0 + 1) : -lx);
+  const int dy = C == 1 ? n0 : (C == 0 ? -1 : -ly);
+  const int dz = C == 2 ? lz : (C == 0 ? -1 : -n0);
+  int ax = fx ? (int)fidx(g, 0, mx, xj, k0) : 0;
+  int ay = fy ? (int)fidx(g, 1, i, my, k0) : 0;
+  int az = fz ? (int)fidx(g, 2, i, j, k0 + (C == 2 ? 0 : 1)) : 0;
   const T* __restrict__ U_ = vel.q[0];
   const T* __restrict__ V_ = vel.q[1];
   const T* __restrict__ W_ = vel.q[2];
-  auto adv_load = [&](int k) {
-    Adv a{T(0), T(0), T(0), T(0), T(0)};
-    const int idC = (C == 0) ? i : ((C == 1) ? j : k);
-    const bool wall = idC == 0 || idC == g.n[C];
-    const int dk = k - k0;
-    if ((C == 0) || !wall) {
-      if (fxh0) { const int o = oxh + dk * lx; a.xh = T(0.5) * (U_[o] + U_[o + dxh]); }
-      if (fxl0) { const int o = oxl + dk * lx; a.xl = T(0.5) * (U_[o] + U_[o + dxl]); }
+  T u0 = T(0), u1 = T(0), v0 = T(0), v1 = T(0), w0 = T(0), w1 = T(0);
+  auto load = [&](int k) {  // of plane k; called for consecutive planes
+    const bool kw = C == 2 && (k == 0 || k == n2);
+    u0 = u1 = v0 = v1 = w0 = w1 = T(0);
+    if (fx && !kw) {
+      u0 = U_[ax];
+      u1 = U_[ax + dx];
     }
-    if ((C == 1) || !wall) {
-      if (fyh0) { const int o = oyh + dk * ly; a.yh = T(0.5) * (V_[o] + V_[o + dyh]); }
-      if (fyl0) { const int o = oyl + dk * ly; a.yl = T(0.5) * (V_[o] + V_[o + dyl]); }
+    if (fy && !kw) {
+      v0 = V_[ay];
+      v1 = V_[ay + dy];
     }
-    if (inside && ((C == 2) || !wall) && (C != 2 || k + oz + 1 <= g.n[2] - 1)) {
-      const int o = ozh + dk * lz;
-      a.zh = T(0.5) * (W_[o] + W_[o + dzh]);
+    if (fz && (C != 2 || k < n2)) {
+      w0 = W_[az];
+      w1 = W_[az + dz];
     }
-    return a;
+    ax += lx;
+    ay += ly;
+    az += lz;
   };
+  const int own = (ty + 2) * HX + tx + 2;
+  const int ox = edge ? ((tx & (BY - 1)) + 2) * HX + 1 : own;
+  const int oy = edge ? HX + tx + 2 : own;
 
-  // prologue: planes k0-2 .. k0+2 in flight, advective velocities of plane k0
 #pragma unroll 1
-  for (int p = k0 - 2; p <= k0 + 2; ++p) issue(p);
-  Adv cur = adv_load(k0);
-  T Fz_lo = T(0);
+  for (int p = k0; p < k0 + NPL; ++p) issue(p);
+  load(k0);
+  // own column: planes k0 - 2 and k0 - 1 from memory
+  const size_t col = (size_t)min(j, e1 - 1) * e0 + min(i, e0 - 1);
+  T ra, rm, qa = T(0), qm = T(0);
+  {
+    T sa, sm;
+    const size_t pa = (size_t)mirror_index<C, 2, T>(g, k0 - 2, sa) * plane + col;
+    const size_t pm = (size_t)mirror_index<C, 2, T>(g, k0 - 1, sm) * plane + col;
+    ra = rho[pa];
+    rm = rho[pm];
+    if (V) {
+      qa = sa * qc[pa];
+      qm = sm * qc[pm];
+    }
+  }
+  cpa_wait<NPL - 3>();  // planes k0 .. k0 + 2
+#pragma unroll 1
+  for (int p = k0; p <= k0 + 2; ++p) fix(p);
+  __syncthreads();
+  T rc = sR[0][own], rp = sR[1][own], qo = T(0), qp = T(0);
+  if (V) {
+    T sp;
+    mirror_index<C, 2, T>(g, k0 + 1, sp);
+    qo = sQ[0][V ? own : 0];
+    qp = sp * sQ[V ? 1 : 0][V ? own : 0];
+  }
+  T zlo[2] = {T(0), T(0)};
+  if (fz && (C != 2 || k0 > 0)) {
+    const T adv = adv_at<C, 2, T>(g, vel, i, j, k0, C == 2 ? k0 - 1 : k0);
+    if (adv != T(0)) {
+      zlo[0] = adv * lim4<T>(ra, rm, rc, rp, adv);
+      if (V) zlo[1] = zlo[0] * lim4<T>(qa, qm, qo, qp, adv);
+    }
+  }
+  size_t id = (size_t)k0 * plane + (size_t)j * e0 + i;
+  // face through the last column or row, next to this one
+  const bool twin = inside && ((C == 0 && tx == BX - 1 && i == n0 - 1) || (C == 1 && ty == BY - 1 && j == n1 - 1));
+  auto emit = [&](size_t at, T self, T R, T M, T base, double base64) {
+    if (MODE == TR_STAGE) {
+      o.out[at] = o.base ? stage_sum(o.a, base, o.b, self, o.c, R) : stage_sum(self, o.c, R);
+    } else if (MODE == TR_LAST) {
+      const double v = stage64(o.a64, base64, o.b64, self, o.c64, R);
+      o.rho64[at] = v;
+      o.beta64[at] = recip_df(v);
+    }
+    if (V) o.conv[at] = M;
+  };
+#pragma unroll 1
   for (int k = k0; k < k1; ++k) {
-    issue(k + 3);
-    const Adv nxt = k + 1 < k1 ? adv_load(k + 1) : Adv{T(0), T(0), T(0), T(0), T(0)};
-    cpa_wait<1>();  // planes up to k + 2 have landed (this thread's copies)
-    if (k == k0) {
-#pragma unroll 1
-      for (int p = k0 - 2; p <= k0 + 2; ++p) fix(p);
-    } else {
-      fix(k + 2);
+    const T axv = T(0.5) * (u0 + u1), ayv = T(0.5) * (v0 + v1), azv = T(0.5) * (w0 + w1);
+    if (k + 1 < k1) load(k + 1);
+    T base = T(0);
+    double base64 = 0.0;
+    if (MODE == TR_STAGE && o.base && inside) base = o.base[id];
+    if (MODE == TR_LAST && inside) base64 = o.base64[id];
+    const int s = (k - k0) & (NPL - 1), s2 = (k + 2 - k0) & (NPL - 1), par = k & 1;
+    const T* R_ = sR[s];
+    const T* Q_ = sQ[V ? s : 0];
+    const T rq = sR[s2][own];
+    T qq = T(0);
+    if (V) {
+      T sz;
+      mirror_index<C, 2, T>(g, k + 2, sz);
+      qq = sz * sQ[V ? s2 : 0][V ? own : 0];
     }
-    __syncthreads();  // plane k + 2 published
-    const int s = slot(k);
-    const int idC = (C == 0) ? i : ((C == 1) ? j : k);
-    const bool wall = idC == 0 || idC == g.n[C];
-    T Fz_hi = T(0);
-    if (inside) {
-      const T* R_ = sR[s];
-      const T* Q_ = sQ[WITHV ? s : 0];
-      // x-fluxes: hi through the CV face above i (taps i-1 .. i+2), lo below (taps i-2 .. i+1)
-      T hi = T(0), lo = T(0);
-      const int hr = (ty + 2) * HX;
-      if (cur.xh != T(0)) {
-        hi = cur.xh * lim4<T>(R_[hr + tx + 1], R_[hr + tx + 2], R_[hr + tx + 3], R_[hr + tx + 4], cur.xh);
-        if (WITHV) hi *= lim4<T>(Q_[hr + tx + 1], Q_[hr + tx + 2], Q_[hr + tx + 3], Q_[hr + tx + 4], cur.xh);
-      }
-      if (cur.xl != T(0)) {
-        lo = cur.xl * lim4<T>(R_[hr + tx], R_[hr + tx + 1], R_[hr + tx + 2], R_[hr + tx + 3], cur.xl);
-        if (WITHV) lo *= lim4<T>(Q_[hr + tx], Q_[hr + tx + 1], Q_[hr + tx + 2], Q_[hr + tx + 3], cur.xl);
-      }
-      sFx[ty][tx + 1] = hi;
-      if (tx == 0) sFx[ty][0] = lo;
-      // y-fluxes
-      hi = T(0);
-      lo = T(0);
-      const int hc = tx + 2;
-      if (cur.yh != T(0)) {
-        hi = cur.yh * lim4<T>(R_[(ty + 1) * HX + hc], R_[(ty + 2) * HX + hc], R_[(ty + 3) * HX + hc],
-                              R_[(ty + 4) * HX + hc], cur.yh);
-        if (WITHV)
-          hi *= lim4<T>(Q_[(ty + 1) * HX + hc], Q_[(ty + 2) * HX + hc], Q_[(ty + 3) * HX + hc],
-                        Q_[(ty + 4) * HX + hc], cur.yh);
-      }
-      if (cur.yl != T(0)) {
-        lo = cur.yl * lim4<T>(R_[ty * HX + hc], R_[(ty + 1) * HX + hc], R_[(ty + 2) * HX + hc],
-                              R_[(ty + 3) * HX + hc], cur.yl);
-        if (WITHV)
-          lo *= lim4<T>(Q_[ty * HX + hc], Q_[(ty + 1) * HX + hc], Q_[(ty + 2) * HX + hc],
-                        Q_[(ty + 3) * HX + hc], cur.yl);
-      }
-      sFy[ty + 1][tx] = hi;
-      if (ty == 0) sFy[0][tx] = lo;
-      // z-fluxes through the CV faces above (taps k-1 .. k+2) and, at the
-      // chunk start, below (taps k-2 .. k+1)
-      if (k == k0) {
-        Fz_lo = T(0);
-        const int mzl = k + oz;
-        if (((C == 2) || !wall) && (C != 2 || mzl >= 0)) {
-          const T adv = adv_at<C, 2, T>(g, vel, i, j, k, mzl);
-          T r4[4], q4[4];
+    // fluxes: [0] mass, [1] momentum
+    T xf[2], yf[2], zf[2];
+    xf[0] = axv * lim4<T>(R_[ox - 1], R_[ox], R_[ox + 1], R_[ox + 2], axv);
+    yf[0] = ayv * lim4<T>(R_[oy - HX], R_[oy], R_[oy + HX], R_[oy + 2 * HX], ayv);
+    zf[0] = azv * lim4<T>(rm, rc, rp, rq, azv);
+    if (axv == T(0)) xf[0] = T(0);
+    if (ayv == T(0)) yf[0] = T(0);
+    if (azv == T(0)) zf[0] = T(0);
+    xf[1] = yf[1] = zf[1] = T(0);
+    if (V) {
+      if (axv != T(0)) xf[1] = xf[0] * lim4<T>(Q_[ox - 1], Q_[ox], Q_[ox + 1], Q_[ox + 2], axv);
+      if (ayv != T(0)) yf[1] = yf[0] * lim4<T>(Q_[oy - HX], Q_[oy], Q_[oy + HX], Q_[oy + 2 * HX], ayv);
+      if (azv != T(0)) zf[1] = zf[0] * lim4<T>(qm, qo, qp, qq, azv);
+    }
+    constexpr int F0 = MODE == TR_CONV ? 1 : 0;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) ztap(k - 2 + q, r4[q], q4[q]);
-          Fz_lo = adv * lim4<T>(r4[0], r4[1], r4[2], r4[3], adv);
-          if (WITHV) Fz_lo *= lim4<T>(q4[0], q4[1], q4[2], q4[3], adv);
-        }
-      }
-      if (cur.zh != T(0)) {
-        T r4[4], q4[4];
+    for (int f = 0; f < NF; ++f) {
+      sFy[par][f][edge ? 0 : ty + 1][tx] = yf[F0 + f];
+      if (edge && tx < BY) sXe[par][f][tx] = xf[F0 + f];
+    }
+    cpa_wait<NPL - 4>();  // planes up to k + 3 have landed (this thread's copies)
+    fix(k + 3);
+    __syncthreads();
+    T res[2] = {T(0), T(0)};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) ztap(k - 1 + q, r4[q], q4[q]);
-        Fz_hi = cur.zh * lim4<T>(r4[0], r4[1], r4[2], r4[3], cur.zh);
-        if (WITHV) Fz_hi *= lim4<T>(q4[0], q4[1], q4[2], q4[3], cur.zh);
-      }
+    for (int f = 0; f < NF; ++f) {
+      T xl = __shfl_up_sync(0xffffffffu, xf[F0 + f], 1);
+      if (tx == 0) xl = sXe[par][f][edge ? 0 : ty];
+      const T yl = sFy[par][f][edge ? 0 : ty][tx];
+      res[F0 + f] = (xf[F0 + f] - xl) * ginv<T>(g, 0) + (yf[F0 + f] - yl) * ginv<T>(g, 1) +
+                    (zf[F0 + f] - zlo[F0 + f]) * ginv<T>(g, 2);
+      zlo[F0 + f] = zf[F0 + f];
     }
-    __syncthreads();  // x- and y-fluxes published
-    if (inside) {
-      const T r = (sFx[ty][tx + 1] - sFx[ty][tx]) * ginv<T>(g, 0) + (sFy[ty + 1][tx] - sFy[ty][tx]) * ginv<T>(g, 1) +
-                  (Fz_hi - Fz_lo) * ginv<T>(g, 2);
-      out[(size_t)k * plane + (size_t)j * e0 + i] = wall ? T(0) : r;
-      Fz_lo = Fz_hi;
+    if (C == 0 ? wi : (C == 1 ? wj : (k == 0 || k == n2))) res[0] = res[1] = T(0);
+    if (inside) emit(id, rc, res[0], res[1], base, base64);
+    if (twin) {
+      const size_t at = id + (C == 0 ? 1 : e0);
+      emit(at, rho[at], T(0), T(0), MODE == TR_STAGE && o.base ? o.base[at] : T(0),
+           MODE == TR_LAST ? o.base64[at] : 0.0);
     }
-    cur = nxt;
+    issue(k + NPL);  // into plane k's slot
+    rm = rc;
+    rc = rp;
+    rp = rq;
+    if (V) {
+      qm = qo;
+      qo = qp;
+      qp = qq;
+    }
+    id += plane;
   }
   cpa_wait<0>();  // no copies in flight when the block ends
 }
@@ -365,42 +452,85 @@ int transport_chunk(int ex, int ey, int ez) {
   return c;
 }
 
-template <bool WITHV, typename T>
-static void transport_all(const GridDev& g, const CVel<T>& v, const T* const rho[3], T* const out[3],
-                          const T* inlet_w, cudaStream_t st) {
-  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-  int zc = transport_chunk(n0 + 1, n1, n2);
-  { k_transport<0, WITHV, T><<<dim3(cdiv(n0 + 1, BX), cdiv(n1, BY), cdiv(n2, zc)), dim3(BX, BY), 0, st>>>(
-      g, v, rho[0], out[0], zc, nullptr); WSI_COUNT(); }
-  zc = transport_chunk(n0, n1 + 1, n2);
-  { k_transport<1, WITHV, T><<<dim3(cdiv(n0, BX), cdiv(n1 + 1, BY), cdiv(n2, zc)), dim3(BX, BY), 0, st>>>(
-      g, v, rho[1], out[1], zc, nullptr); WSI_COUNT(); }
-  zc = transport_chunk(n0, n1, n2 + 1);
-  { k_transport<2, WITHV, T><<<dim3(cdiv(n0, BX), cdiv(n1, BY), cdiv(n2 + 1, zc)), dim3(BX, BY), 0, st>>>(
-      g, v, rho[2], out[2], zc, WITHV ? inlet_w : nullptr); WSI_COUNT(); }
+template <int C, int MODE, typename T>
+static void transport_one(const GridDev& g, const CVel<T>& v, const T* rho, const TransportOut<T>& o, const T* inl,
+                          cudaStream_t st) {
+  // (the last column or row, see k_transport, gets no tile of its own)
+  const int ex = C == 0 && g.n[0] % BX == 0 ? g.n[0] : ext(g, C, 0);
+  const int ey = C == 1 && g.n[1] % BY == 0 ? g.n[1] : ext(g, C, 1);
+  const int ez = ext(g, C, 2), zc = transport_chunk(ex, ey, ez);
+  { k_transport<C, MODE, T><<<dim3(cdiv(ex, BX), cdiv(ey, BY), cdiv(ez, zc)), dim3(BX, BY + 1), 0, st>>>(g, v, rho, o, zc,
+                                                                                                       inl); WSI_COUNT(); }
 }
 
-template <typename T>
-void launch_transport_flux(const GridDev& g, const T* const vel[3], const T* const rho[3], bool with_velocity,
-                           T* const out[3], cudaStream_t st, const T* inlet_w) {
+template <int MODE, typename T>
+static void transport_all(const GridDev& g, const T* const vel[3], const T* const rho[3], const TransportOut<T> o[3],
+                          const T* inlet_w, cudaStream_t st) {
   CVel<T> v{{vel[0], vel[1], vel[2]}};
   ktimer_begin(KC_TRANSPORT, st);
   {
-    // algorithmic bytes: per component rho_C, u, v, w (advective
-    // velocities), q_C with the velocity, the result
+    // algorithmic bytes: per component rho_C, u, v, w (advective velocities),
+    // q_C and the result with the momentum flux; the stage's other input and
+    // its results
     const double F = (double)(fsize(g, 0) + fsize(g, 1) + fsize(g, 2));
-    ktimer_bytes(KC_TRANSPORT, sizeof(T) * F * (with_velocity ? 6.0 : 5.0));
+    const double b = sizeof(T) * (MODE == TR_STAGE ? (o[0].base ? 6.0 : 5.0) : 6.0) + (MODE == TR_LAST ? 24.0 : 0.0);
+    ktimer_bytes(KC_TRANSPORT, F * b);
   }
-  if (with_velocity)
-    transport_all<true, T>(g, v, rho, out, inlet_w, st);
-  else
-    transport_all<false, T>(g, v, rho, out, nullptr, st);
+  transport_one<0, MODE, T>(g, v, rho[0], o[0], nullptr, st);
+  transport_one<1, MODE, T>(g, v, rho[1], o[1], nullptr, st);
+  transport_one<2, MODE, T>(g, v, rho[2], o[2], inlet_w, st);
   ktimer_end(KC_TRANSPORT, st);
 }
-template void launch_transport_flux<double>(const GridDev&, const double* const[3], const double* const[3], bool,
-                                            double* const[3], cudaStream_t, const double*);
-template void launch_transport_flux<float>(const GridDev&, const float* const[3], const float* const[3], bool,
-                                           float* const[3], cudaStream_t, const float*);
+
+template <typename T>
+void launch_transport_stage(const GridDev& g, const T* const vel[3], const T* const rho[3], double a,
+                            const T* const base[3], double b, double c, T* const out[3], cudaStream_t st) {
+  TransportOut<T> o[3] = {};
+  for (int d = 0; d < 3; ++d) {
+    o[d].base = base ? base[d] : nullptr;
+    o[d].a = (T)a;
+    o[d].b = (T)b;
+    o[d].c = (T)c;
+    o[d].out = out[d];
+  }
+  transport_all<TR_STAGE, T>(g, vel, rho, o, nullptr, st);
+}
+
+template <typename T>
+void launch_transport_last(const GridDev& g, const T* const vel[3], const T* const rho[3], double a,
+                           const double* const base[3], double b, double c, double* const rho_out[3],
+                           double* const beta_out[3], T* const conv[3], cudaStream_t st, const T* inlet_w) {
+  TransportOut<T> o[3] = {};
+  for (int d = 0; d < 3; ++d) {
+    o[d].base64 = base[d];
+    o[d].a64 = a;
+    o[d].b64 = b;
+    o[d].c64 = c;
+    o[d].rho64 = rho_out[d];
+    o[d].beta64 = beta_out[d];
+    o[d].conv = conv[d];
+  }
+  transport_all<TR_LAST, T>(g, vel, rho, o, inlet_w, st);
+}
+
+template <typename T>
+void launch_transport_conv(const GridDev& g, const T* const vel[3], const T* const rho[3], T* const conv[3],
+                           cudaStream_t st, const T* inlet_w) {
+  TransportOut<T> o[3] = {};
+  for (int d = 0; d < 3; ++d) o[d].conv = conv[d];
+  transport_all<TR_CONV, T>(g, vel, rho, o, inlet_w, st);
+}
+#define INST_TRANSPORT(T)                                                                                              \
+  template void launch_transport_stage<T>(const GridDev&, const T* const[3], const T* const[3], double,                \
+                                          const T* const[3], double, double, T* const[3], cudaStream_t);               \
+  template void launch_transport_last<T>(const GridDev&, const T* const[3], const T* const[3], double,                 \
+                                         const double* const[3], double, double, double* const[3], double* const[3],   \
+                                         T* const[3], cudaStream_t, const T*);                                         \
+  template void launch_transport_conv<T>(const GridDev&, const T* const[3], const T* const[3], T* const[3],            \
+                                         cudaStream_t, const T*);
+INST_TRANSPORT(double)
+INST_TRANSPORT(float)
+#undef INST_TRANSPORT
 
 template <typename Ti, typename To>
 __global__ void k_lincomb(size_t n, double a, const Ti* __restrict__ x, double b, const Ti* __restrict__ y, double c,
