@@ -114,10 +114,15 @@ void launch_stokes_df_ready(const GridDev& g, const DfOperands& o, double theta,
 // operands; h: the coefficients on the device
 void launch_x_update(const GridDev& g, const DfOperands& o, const ZVec* z, int m, const double* h, double* x,
                      cudaStream_t st);
-// red-black Gauss-Seidel half sweep on the viscous block for component c
+// red-black Gauss-Seidel half sweep on the viscous block; vd: the inverse
+// diagonals, or null (then formed by each update)
 template <typename T>
 void launch_viscous_rbgs(const GridDev& g, const Coef<T>& cf, T inv_dt, T theta, T* const q[3], const T* const b[3],
-                         int color, cudaStream_t st);
+                         int color, cudaStream_t st, T* const* vd = nullptr);
+// the inverse diagonals of the viscous block's rows (zero on walls); q: any
+// arrays of the velocity's shape
+void launch_viscous_diag(const GridDev& g, const Coef<double>& cf, double inv_dt, double theta,
+                         const double* const q[3], double* const vd[3], cudaStream_t st);
 
 // transport.cu (Sec. 4.2.2): the divergence R of the mass flux of rho with vel,
 // and C of the momentum flux, on all three face arrays, storage and arithmetic
@@ -285,6 +290,7 @@ struct MGLevel {
   T* cd;            // Chebyshev smoother: direction, and the second buffer pair
   T* cx2;
   T* cd2;
+  T* id;            // float64: inverse diagonal (null in float32)
 };
 
 // one level of the viscous multigrid (levels >= 1; level 0 uses the fine
@@ -313,6 +319,10 @@ struct Precond {
   // work
   T* ut[3] = {nullptr, nullptr, nullptr};
   T* pv = nullptr;  // float32: pressure part before its mean is removed
+  // float64: inverse diagonals of the viscous block, for vd_dt and vd_theta
+  T* vd[3] = {nullptr, nullptr, nullptr};
+  bool vd_set = false;
+  T vd_dt = T(0), vd_theta = T(0);
   double* dscratch = nullptr;  // reductions
   double* dsum = nullptr;
   bool built = false;

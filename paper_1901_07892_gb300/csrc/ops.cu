@@ -236,7 +236,8 @@ __device__ __forceinline__ T strain_at(const GridDev& g, const Coef<T>& cf, cons
   T qm = qc[fidx(g, C, lo3[0], lo3[1], lo3[2])];
   T mu_hi = top ? mu_lo : cf.mu_cc[fidx(g, 3, i, j, k)];
   T qp = top ? qm : qc[fidx(g, C, hi3[0], hi3[1], hi3[2])];
-  T L = T(2) * ihC * ihC * (mu_hi * (qp - q0) - mu_lo * (q0 - qm));
+  const T w = sizeof(T) == 8 ? T(2) * ginv2<T>(g, C) : T(2) * ihC * ihC;
+  T L = w * (mu_hi * (qp - q0) - mu_lo * (q0 - qm));
   T dg = -T(2) * ihC * ihC * (mu_hi + mu_lo);
 #pragma unroll
   for (int D = 0; D < 3; ++D) {
@@ -356,18 +357,69 @@ __global__ void k_viscous_rbgs(GridDev g, Coef<T> cf, T inv_dt, T theta, Vel<T> 
   q.q[C][id] += (b[id] - a) / d;
 }
 
+// The same with the inverse diagonals from memory: the float64 pipe bounds the
+// update, and the diagonal and its division were 25 of its 60 operations (at 128
+// x 64 x 64 36 -> 22 us per component and half sweep).
+template <int C>
+__global__ void k_viscous_rbgs_d(GridDev g, Coef<double> cf, double inv_dt, double theta, Vel<double> q,
+                                 const double* __restrict__ b, const double* __restrict__ vd, int color) {
+  const int j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + color) & 1);
+  if (i >= ext(g, C, 0) || j >= ext(g, C, 1)) return;
+  int id3[3] = {i, j, k};
+  if (!face_row(g, C, id3[C])) return;
+  const size_t id = fidx(g, C, i, j, k);
+  const double* cq[3] = {q.q[0], q.q[1], q.q[2]};
+  const double L = strain_at<C, double>(g, cf, cq, i, j, k, nullptr);
+  const double q0 = q.q[C][id], r = fma(-(cf.rho_face[C][id] * inv_dt), q0, b[id]);
+  q.q[C][id] = fma(fma(theta, L, r), vd[id], q0);
+}
+
+// (q: arrays of the velocity's shape; the operator's value is not used)
+template <int C>
+__global__ void k_viscous_diag(GridDev g, Coef<double> cf, double inv_dt, double theta, CVel<double> q, double* vd) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  if (i >= ext(g, C, 0) || j >= ext(g, C, 1)) return;
+  int id3[3] = {i, j, k};
+  const size_t id = fidx(g, C, i, j, k);
+  double dg = 0.0;
+  if (face_row(g, C, id3[C])) {
+    strain_at<C, double>(g, cf, q.q, i, j, k, &dg);
+    dg = 1.0 / (cf.rho_face[C][id] * inv_dt - theta * dg);
+  }
+  vd[id] = dg;
+}
+
+void launch_viscous_diag(const GridDev& g, const Coef<double>& cf, double inv_dt, double theta,
+                         const double* const q[3], double* const vd[3], cudaStream_t st) {
+  const CVel<double> v{{q[0], q[1], q[2]}};
+  const dim3 blk(BX, BY);
+  { k_viscous_diag<0><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), blk, 0, st>>>(g, cf, inv_dt, theta, v, vd[0]); WSI_COUNT(); }
+  { k_viscous_diag<1><<<grid3(g.n[0], g.n[1] + 1, g.n[2]), blk, 0, st>>>(g, cf, inv_dt, theta, v, vd[1]); WSI_COUNT(); }
+  { k_viscous_diag<2><<<grid3(g.n[0], g.n[1], g.n[2] + 1), blk, 0, st>>>(g, cf, inv_dt, theta, v, vd[2]); WSI_COUNT(); }
+}
+
+template <int C, typename T>
+static void viscous_rbgs_one(const GridDev& g, const Coef<T>& cf, T inv_dt, T theta, const Vel<T>& q, const T* b,
+                             const T* vd, int color, cudaStream_t st) {
+  const dim3 grid = grid3((ext(g, C, 0) + 1) / 2, ext(g, C, 1), ext(g, C, 2)), blk(BX, BY);
+  if constexpr (sizeof(T) == 8) {
+    if (vd) {
+      { k_viscous_rbgs_d<C><<<grid, blk, 0, st>>>(g, cf, inv_dt, theta, q, b, vd, color); WSI_COUNT(); }
+      return;
+    }
+  }
+  { k_viscous_rbgs<C, T><<<grid, blk, 0, st>>>(g, cf, inv_dt, theta, q, b, color); WSI_COUNT(); }
+}
+
 template <typename T>
 void launch_viscous_rbgs(const GridDev& g, const Coef<T>& cf, T inv_dt, T theta, T* const q[3], const T* const b[3],
-                         int color, cudaStream_t st) {
+                         int color, cudaStream_t st, T* const* vd) {
   Vel<T> vq{{q[0], q[1], q[2]}};
   ktimer_begin(KC_RBGS_V, st);
-  { k_viscous_rbgs<0, T><<<grid3((g.n[0] + 2) / 2, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, cf, inv_dt, theta, vq,
-                                                                                         b[0], color); WSI_COUNT(); }
-  { k_viscous_rbgs<1, T><<<grid3((g.n[0] + 1) / 2, g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, cf, inv_dt, theta,
-                                                                                           vq, b[1], color); WSI_COUNT(); }
-  if (g.n[2] > 1)
-    { k_viscous_rbgs<2, T><<<grid3((g.n[0] + 1) / 2, g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, cf, inv_dt, theta,
-                                                                                             vq, b[2], color); WSI_COUNT(); }
+  viscous_rbgs_one<0, T>(g, cf, inv_dt, theta, vq, b[0], vd ? vd[0] : nullptr, color, st);
+  viscous_rbgs_one<1, T>(g, cf, inv_dt, theta, vq, b[1], vd ? vd[1] : nullptr, color, st);
+  if (g.n[2] > 1) viscous_rbgs_one<2, T>(g, cf, inv_dt, theta, vq, b[2], vd ? vd[2] : nullptr, color, st);
   ktimer_end(KC_RBGS_V, st);
 }
 
@@ -775,9 +827,9 @@ template void launch_viscous_residual<double>(const GridDev&, const Coef<double>
 template void launch_viscous_residual<float>(const GridDev&, const Coef<float>&, float, float, const float* const[3],
                                              const float* const[3], float* const[3], cudaStream_t);
 template void launch_viscous_rbgs<double>(const GridDev&, const Coef<double>&, double, double, double* const[3],
-                                          const double* const[3], int, cudaStream_t);
+                                          const double* const[3], int, cudaStream_t, double* const*);
 template void launch_viscous_rbgs<float>(const GridDev&, const Coef<float>&, float, float, float* const[3],
-                                         const float* const[3], int, cudaStream_t);
+                                         const float* const[3], int, cudaStream_t, float* const*);
 template void launch_pressure<double>(const GridDev&, const double* const[3], const double*, double*, cudaStream_t);
 template void launch_pressure<float>(const GridDev&, const float* const[3], const float*, float*, cudaStream_t);
 template void launch_grad<double>(const GridDev&, const double*, double* const[3], cudaStream_t);
