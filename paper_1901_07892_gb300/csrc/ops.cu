@@ -35,6 +35,9 @@ __device__ __forceinline__ int band_code_f(float tf, float bound) {
   return 2;
 }
 
+// FUSED: 1 + phi/eps with one rounding, else the quotient by itself (each caller
+// keeps to one of the two, so that its results are kept to the bit).
+template <bool FUSED>
 __device__ __forceinline__ double heav(double phi, double inv_eps, int& code) {
   const double t = phi * inv_eps;
   const float tf = d2f_fast(t);
@@ -47,7 +50,8 @@ __device__ __forceinline__ double heav(double phi, double inv_eps, int& code) {
     return 1.0;
   }
   code = 2;
-  return 0.5 * (1.0 + t + sin(M_PI * t) / M_PI);
+  const double q = FUSED ? fma(phi, inv_eps, 1.0) : __dadd_rn(1.0, t);
+  return 0.5 * __dadd_rn(q, sin(M_PI * t) / M_PI);
 }
 
 // two-stage blend (Sec. 2): fluid value from phi, then solid from psi; away
@@ -59,78 +63,93 @@ __device__ __forceinline__ double two_stage(double h1, int c1, double h2, int c2
   return zs + (zf - zs) * h2;
 }
 
-__device__ __forceinline__ double cell_at(const GridDev& g, const double* a, int i, int j, int k) {
-  i = clampi(i, 0, g.n[0] - 1);
-  j = clampi(j, 0, g.n[1] - 1);
-  k = clampi(k, 0, g.n[2] - 1);
-  return a[fidx(g, 3, i, j, k)];
+// inside a band: the cell's density and viscosity, a face's density and flow
+// density with their reciprocals (rare: out of line, one copy of the code)
+__device__ __noinline__ void cell_band(const PhaseConst& pc, double a, double b, double* rho, double* mu, double* imu) {
+  int c1, c2;
+  const double h1 = heav<true>(a, pc.inv_eps, c1), h2 = heav<true>(b, pc.inv_eps, c2);
+  if (rho) *rho = two_stage(h1, c1, h2, c2, pc.rho_l, pc.rho_g, pc.rho_s, pc.rho_tab);
+  const double m = two_stage(h1, c1, h2, c2, pc.mu_l, pc.mu_g, pc.mu_s, pc.mu_tab);
+  *mu = m;
+  if (imu) *imu = (c1 < 2 && c2 < 2) ? pc.imu_tab[c1 + 2 * c2] : 1.0 / m;
 }
-
-__global__ void k_mat_cells(GridDev g, PhaseConst pc, const double* __restrict__ phi, const double* __restrict__ psi,
-                            double* rho_cc, double* mu_cc) {
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.n[0] || j >= g.n[1]) return;
-  size_t id = fidx(g, 3, i, j, k);
-  const double a = phi[id], b = psi[id];
-  const float ie = pc.inv_eps_f;
-  const float af = d2f_fast(a), bf = d2f_fast(b);
-  // bound: 2^-20 |t|, far above the float32 rounding of phi and of phi/eps
-  int c1 = band_code_f(af * ie, 9.5367431640625e-07f * fabsf(af * ie)),
-      c2 = band_code_f(bf * ie, 9.5367431640625e-07f * fabsf(bf * ie));
-  if (c1 < 2 && c2 < 2) {
-    if (rho_cc) rho_cc[id] = pc.rho_tab[c1 + 2 * c2];
-    mu_cc[id] = pc.mu_tab[c1 + 2 * c2];
-    if (pc.inv_mu) pc.inv_mu[id] = pc.imu_tab[c1 + 2 * c2];
-    return;
-  }
-  const double h1 = heav(a, pc.inv_eps, c1), h2 = heav(b, pc.inv_eps, c2);
-  if (rho_cc) rho_cc[id] = two_stage(h1, c1, h2, c2, pc.rho_l, pc.rho_g, pc.rho_s, pc.rho_tab);
-  const double mu = two_stage(h1, c1, h2, c2, pc.mu_l, pc.mu_g, pc.mu_s, pc.mu_tab);
-  mu_cc[id] = mu;
-  if (pc.inv_mu) pc.inv_mu[id] = (c1 < 2 && c2 < 2) ? pc.imu_tab[c1 + 2 * c2] : 1.0 / mu;
-}
-
-// face density from face-averaged level sets (wall faces: the interior cell)
-template <int C>
-__global__ void k_mat_faces(GridDev g, PhaseConst pc, const double* __restrict__ phi, const double* __restrict__ psi,
-                            double* rho_face, double* beta, double* rho_flow) {
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= ext(g, C, 0) || j >= ext(g, C, 1)) return;
-  int lo[3] = {i, j, k}, hi[3] = {i, j, k};
-  lo[C] -= 1;
-  const double pl = cell_at(g, phi, lo[0], lo[1], lo[2]), ph = cell_at(g, phi, hi[0], hi[1], hi[2]);
-  size_t id = fidx(g, C, i, j, k);
-  const float ie = pc.inv_eps_f;
-  // bound: 2^-20 (|phi_lo| + |phi_hi|)/eps, far above the float32 rounding of
-  // the two values, their mean and the scaling
-  const float plf = d2f_fast(pl), phf = d2f_fast(ph);
-  int c1 = band_code_f(0.5f * (plf + phf) * ie, 9.5367431640625e-07f * (fabsf(plf) + fabsf(phf)) * ie);
-  double sl = 0.0, sh = 0.0;
-  int c2 = 0;
-  if (rho_face) {
-    sl = cell_at(g, psi, lo[0], lo[1], lo[2]);
-    sh = cell_at(g, psi, hi[0], hi[1], hi[2]);
-    const float slf = d2f_fast(sl), shf = d2f_fast(sh);
-    c2 = band_code_f(0.5f * (slf + shf) * ie, 9.5367431640625e-07f * (fabsf(slf) + fabsf(shf)) * ie);
-  }
-  if (c1 < 2 && c2 < 2) {  // away from both bands: table values only
-    if (rho_face) {
-      rho_face[id] = pc.rho_tab[c1 + 2 * c2];
-      if (beta) beta[id] = pc.beta_tab[c1 + 2 * c2];
-    }
-    if (rho_flow) rho_flow[id] = pc.flow_tab[c1];
-    return;
-  }
+__device__ __noinline__ void face_band(const PhaseConst& pc, double pl, double ph, double sl, double sh, double* rho,
+                                       double* beta, double* flow) {
+  int c1, c2;
   const double pa = 0.5 * (pl + ph);
-  const double h1 = heav(pa, pc.inv_eps, c1);
-  if (rho_face) {
-    const double sa = 0.5 * (sl + sh);
-    const double h2 = heav(sa, pc.inv_eps, c2);
-    const double r = two_stage(h1, c1, h2, c2, pc.rho_l, pc.rho_g, pc.rho_s, pc.rho_tab);
-    rho_face[id] = r;
-    if (beta) beta[id] = (c1 < 2 && c2 < 2) ? pc.beta_tab[c1 + 2 * c2] : 1.0 / r;
+  const double h1 = heav<true>(pa, pc.inv_eps, c1);
+  const double sa = 0.5 * (sl + sh);
+  const double h2 = heav<false>(sa, pc.inv_eps, c2);
+  const double r = two_stage(h1, c1, h2, c2, pc.rho_l, pc.rho_g, pc.rho_s, pc.rho_tab);
+  *rho = r;
+  if (beta) *beta = (c1 < 2 && c2 < 2) ? pc.beta_tab[c1 + 2 * c2] : 1.0 / r;
+  if (flow) *flow = c1 < 2 ? pc.flow_tab[c1] : pc.rho_l + (pc.rho_g - pc.rho_l) * h1;
+}
+
+// Any of the pointers but rho_face may be null.
+struct MatOut {
+  double *rho_cc, *mu_cc;
+  double *rho_face[3], *beta[3], *rho_flow[3];
+};
+
+// Cell densities and viscosities and the face densities (from face-averaged
+// level sets; wall faces: the interior cell) of all three components in one
+// pass: a thread owns a cell and its lower faces, and the upper one at the end of
+// each axis.  Every level-set value is read once from memory: 144 us at 250 x
+// 126 x 130, with a pass for the cells and one per component 195 us.  Latency and
+// the float64 pipe share the time (530 warp instructions per 32 cells, the bands
+// included).
+__global__ void __launch_bounds__(BX* BY, 4) k_materials(GridDev g, const __grid_constant__ PhaseConst pc,
+                                                      const double* __restrict__ phi, const double* __restrict__ psi,
+                                                      const __grid_constant__ MatOut o) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
+  if (i >= n0 || j >= n1) return;
+  // (32-bit offsets: every array holds fewer than 2^31 entries)
+  const int pl = n0 * n1, id = (k * n1 + j) * n0 + i;
+  const int lo[3] = {id - (i > 0 ? 1 : 0), id - (j > 0 ? n0 : 0), id - (k > 0 ? pl : 0)};
+  const double a = phi[id], b = psi[id];
+  double an[3], bn[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    an[d] = phi[lo[d]];
+    bn[d] = psi[lo[d]];
   }
-  if (rho_flow) rho_flow[id] = c1 < 2 ? pc.flow_tab[c1] : pc.rho_l + (pc.rho_g - pc.rho_l) * h1;
+  const float ie = pc.inv_eps_f, eb = 9.5367431640625e-07f;
+  const float af = d2f_fast(a), bf = d2f_fast(b);
+  if (o.mu_cc) {
+    // bound: 2^-20 |t|, far above the float32 rounding of phi and of phi/eps
+    const int c1 = band_code_f(af * ie, eb * fabsf(af * ie)), c2 = band_code_f(bf * ie, eb * fabsf(bf * ie));
+    if (c1 < 2 && c2 < 2) {
+      if (o.rho_cc) o.rho_cc[id] = pc.rho_tab[c1 + 2 * c2];
+      o.mu_cc[id] = pc.mu_tab[c1 + 2 * c2];
+      if (pc.inv_mu) pc.inv_mu[id] = pc.imu_tab[c1 + 2 * c2];
+    } else {
+      cell_band(pc, a, b, o.rho_cc ? o.rho_cc + id : nullptr, o.mu_cc + id, pc.inv_mu ? pc.inv_mu + id : nullptr);
+    }
+  }
+  const int fid[3] = {id + k * n1 + j, id + k * n0, id}, up[3] = {1, n0, pl};
+  const bool last[3] = {i == n0 - 1, j == n1 - 1, k == n2 - 1};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    auto face = [&](int f, double pm, double sm) {
+      // bound: 2^-20 (|phi_lo| + |phi_hi|)/eps, far above the float32 rounding of
+      // the two values, their mean and the scaling
+      const float pf = d2f_fast(pm), sf = d2f_fast(sm);
+      const int c1 = band_code_f(0.5f * (pf + af) * ie, eb * (fabsf(pf) + fabsf(af)) * ie);
+      const int c2 = band_code_f(0.5f * (sf + bf) * ie, eb * (fabsf(sf) + fabsf(bf)) * ie);
+      if (c1 < 2 && c2 < 2) {  // away from both bands: table values only
+        o.rho_face[d][f] = pc.rho_tab[c1 + 2 * c2];
+        if (o.beta[d]) o.beta[d][f] = pc.beta_tab[c1 + 2 * c2];
+        if (o.rho_flow[d]) o.rho_flow[d][f] = pc.flow_tab[c1];
+      } else {
+        face_band(pc, pm, a, sm, b, o.rho_face[d] + f, o.beta[d] ? o.beta[d] + f : nullptr,
+                  o.rho_flow[d] ? o.rho_flow[d] + f : nullptr);
+      }
+    };
+    face(fid[d], an[d], bn[d]);
+    if (last[d]) face(fid[d] + up[d], a, b);
+  }
 }
 
 // Harmonic mean 4 / sum(1/mu) of the 4 cells around an edge (mirror ghosts
@@ -138,35 +157,36 @@ __global__ void k_mat_faces(GridDev g, PhaseConst pc, const double* __restrict__
 // given: a float64 division costs tens of instructions at GB300's float64
 // rate, and each cell feeds twelve edges.  Where the four reciprocals are
 // bit-identical table values the mean comes from the table as well.
-template <int E>
-__global__ void k_mat_edges(GridDev g, PhaseConst pc, const double* __restrict__ mu_cc,
-                            const double* __restrict__ inv_mu, double* mu_e) {
-  // E = 0: xy edges, 1: xz, 2: yz
-  constexpr int A1 = (E == 2) ? 1 : 0;
-  constexpr int A2 = (E == 0) ? 1 : 2;
-  int ex = g.n[0] + (A1 == 0 || A2 == 0), ey = g.n[1] + (A1 == 1 || A2 == 1);
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= ex || j >= ey) return;
-  double v[4];
+// All three edge families in one pass (80 bytes per cell less than three): the
+// seven cells around a corner are read by the corner's thread: 39 us at 250 x
+// 126 x 130, by three passes 62 us.
+__global__ void __launch_bounds__(BX* BY) k_mat_edges(GridDev g, const __grid_constant__ PhaseConst pc,
+                                                      const double* __restrict__ mu_cc,
+                                                      const double* __restrict__ inv_mu, double* e0, double* e1,
+                                                      double* e2) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
+  if (i > n0 || j > n1) return;
+  // the cells above (1) and below (0) the corner along each axis, mirrored at walls
+  const int id = (min(k, n2 - 1) * n1 + min(j, n1 - 1)) * n0 + min(i, n0 - 1);
+  const int dx = i > 0 && i < n0 ? 1 : 0, dy = j > 0 && j < n1 ? n0 : 0, dz = k > 0 && k < n2 ? n0 * n1 : 0;
+  auto at = [&](int o) { return inv_mu ? inv_mu[id - o] : 1.0 / mu_cc[id - o]; };
+  const double v = at(0), vx = at(dx), vy = at(dy), vz = at(dz), vxy = at(dx + dy), vxz = at(dx + dz), vyz = at(dy + dz);
+  auto edge = [&](double* out, double a, double b, double c, double d) {
+    const long long b0 = __double_as_longlong(a);
+    if (b0 == __double_as_longlong(b) && b0 == __double_as_longlong(c) && b0 == __double_as_longlong(d)) {
 #pragma unroll
-  for (int o1 = 0; o1 < 2; ++o1)
-#pragma unroll
-    for (int o2 = 0; o2 < 2; ++o2) {
-      int c[3] = {i, j, k};
-      c[A1] -= o1;
-      c[A2] -= o2;
-      v[2 * o1 + o2] = inv_mu ? cell_at(g, inv_mu, c[0], c[1], c[2]) : 1.0 / cell_at(g, mu_cc, c[0], c[1], c[2]);
+      for (int t = 0; t < 4; ++t)
+        if (b0 == __double_as_longlong(pc.imu_tab[t])) {
+          *out = pc.mue_tab[t];
+          return;
+        }
     }
-  const long long b0 = __double_as_longlong(v[0]);
-  if (b0 == __double_as_longlong(v[1]) && b0 == __double_as_longlong(v[2]) && b0 == __double_as_longlong(v[3])) {
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-      if (b0 == __double_as_longlong(pc.imu_tab[t])) {
-        mu_e[eidx(g, E, i, j, k)] = pc.mue_tab[t];
-        return;
-      }
-  }
-  mu_e[eidx(g, E, i, j, k)] = 4.0 / (((v[0] + v[1]) + v[2]) + v[3]);
+    *out = 4.0 / (((a + b) + c) + d);
+  };
+  if (k < n2) edge(e0 + ((k * (n1 + 1) + j) * (n0 + 1) + i), v, vy, vx, vxy);
+  if (j < n1) edge(e1 + ((k * n1 + j) * (n0 + 1) + i), v, vz, vx, vxz);
+  if (i < n0) edge(e2 + ((k * (n1 + 1) + j) * n0 + i), v, vz, vy, vyz);
 }
 
 void phase_tables(PhaseConst& pc) {
@@ -190,26 +210,21 @@ void phase_tables(PhaseConst& pc) {
 void launch_materials(const GridDev& g, const PhaseConst& pc, const double* phi, const double* psi, double* rho_cc,
                       double* mu_cc, double* const rho_face[3], double* const beta[3], double* const rho_flow[3],
                       double* const mu_e[3], cudaStream_t st) {
-  { k_mat_cells<<<grid3(g.n[0], g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_cc, mu_cc); WSI_COUNT(); }
-  { k_mat_faces<0><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[0], beta[0],
-                                                                             rho_flow[0]); WSI_COUNT(); }
-  { k_mat_faces<1><<<grid3(g.n[0], g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[1], beta[1],
-                                                                             rho_flow[1]); WSI_COUNT(); }
-  { k_mat_faces<2><<<grid3(g.n[0], g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[2], beta[2],
-                                                                             rho_flow[2]); WSI_COUNT(); }
-  { k_mat_edges<0><<<grid3(g.n[0] + 1, g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, mu_cc, pc.inv_mu, mu_e[0]); WSI_COUNT(); }
-  { k_mat_edges<1><<<grid3(g.n[0] + 1, g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, pc, mu_cc, pc.inv_mu, mu_e[1]); WSI_COUNT(); }
-  { k_mat_edges<2><<<grid3(g.n[0], g.n[1] + 1, g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, pc, mu_cc, pc.inv_mu, mu_e[2]); WSI_COUNT(); }
+  MatOut o = {rho_cc, mu_cc, {}, {}, {}};
+  for (int d = 0; d < 3; ++d) {
+    o.rho_face[d] = rho_face[d];
+    o.beta[d] = beta[d];
+    o.rho_flow[d] = rho_flow[d];
+  }
+  { k_materials<<<grid3(g.n[0], g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, o); WSI_COUNT(); }
+  { k_mat_edges<<<grid3(g.n[0] + 1, g.n[1] + 1, g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, pc, mu_cc, pc.inv_mu, mu_e[0],
+                                                                                  mu_e[1], mu_e[2]); WSI_COUNT(); }
 }
 
 void launch_face_density(const GridDev& g, const PhaseConst& pc, const double* phi, const double* psi,
                          double* const rho_face[3], cudaStream_t st) {
-  { k_mat_faces<0><<<grid3(g.n[0] + 1, g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[0], nullptr,
-                                                                             nullptr); WSI_COUNT(); }
-  { k_mat_faces<1><<<grid3(g.n[0], g.n[1] + 1, g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[1], nullptr,
-                                                                             nullptr); WSI_COUNT(); }
-  { k_mat_faces<2><<<grid3(g.n[0], g.n[1], g.n[2] + 1), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, rho_face[2], nullptr,
-                                                                             nullptr); WSI_COUNT(); }
+  MatOut o = {nullptr, nullptr, {rho_face[0], rho_face[1], rho_face[2]}, {}, {}};
+  { k_materials<<<grid3(g.n[0], g.n[1], g.n[2]), dim3(BX, BY), 0, st>>>(g, pc, phi, psi, o); WSI_COUNT(); }
 }
 
 // =========================================================== strain-rate operator
