@@ -271,6 +271,34 @@ int copy_out(wsi_ctx* c, double* dst, const double* src, size_t n) {
   return WSI_OK;
 }
 
+// Whether kernels can take a caller's array as it is: memory of
+// the current device, aligned as the library's own arrays are used (16 bytes).
+// (The calls return only after their stream has been synchronised, so the array
+// outlives its use.)  Everything else goes through a staging copy.
+bool usable(const void* p) {
+  if (!p || ((uintptr_t)p & 15)) return false;
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
+}
+bool overlap(const double* a, size_t na, const double* b, size_t nb) {
+  const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
+  return a0 < b0 + nb * sizeof(double) && b0 < a0 + na * sizeof(double);
+}
+// the caller's array itself where kernels can read it, else its copy in staging
+int use_in(wsi_ctx* c, const double*& use, const double* src, size_t n, double* staging) {
+  if (usable(src)) {
+    use = src;
+    return WSI_OK;
+  }
+  use = staging;
+  return copy_in(c, staging, src, n);
+}
+
 // fill: *fill tells whether the caller still has to fill in the finest level's
 // float32 density and viscosities (df_coef_refresh does both at once)
 int ensure_pc(wsi_ctx* c, bool* fill = nullptr) {
@@ -1305,7 +1333,7 @@ int wsi_apply(wsi_ctx* c, int op, const double* in, double* out, double dt) {
   if (!c->have_phases) return fail(c, WSI_ERR_INVALID_ARG, "no phases set");
   if (!(dt > 0.0)) return fail(c, WSI_ERR_INVALID_ARG, "dt must be positive");
   Coef<double> cf = coef_now(c);
-  double* xin = c->b;
+  const double* xin = nullptr;
   double* xout = c->x;
   size_t nin = 0, nout = 0;
   switch (op) {
@@ -1317,11 +1345,14 @@ int wsi_apply(wsi_ctx* c, int op, const double* in, double* out, double dt) {
     case WSI_OP_DIV: nin = c->nvel; nout = c->ncell; break;
     default: return fail(c, WSI_ERR_INVALID_ARG, "unknown operator");
   }
-  int rc = copy_in(c, xin, in, nin);
+  int rc = use_in(c, xin, in, nin, c->b);
   if (rc) return rc;
+  // (at 250 x 182 x 126 the two copies were 108 of 630 us)
+  const bool direct = usable(out) && !overlap(out, nout, xin, nin);
+  if (direct) xout = out;
   const double* qi[3];
   double* qo[3];
-  vel_parts(c, (const double*)xin, qi);
+  vel_parts(c, xin, qi);
   vel_parts(c, xout, qo);
   switch (op) {
     case WSI_OP_STOKES:
@@ -1338,7 +1369,7 @@ int wsi_apply(wsi_ctx* c, int op, const double* in, double* out, double dt) {
     case WSI_OP_GRAD: launch_grad<double>(c->g, xin, qo, c->st); break;
     case WSI_OP_DIV: launch_div<double>(c->g, qi, xout, 1.0, c->st); break;
   }
-  rc = copy_out(c, out, xout, nout);
+  if (!direct) rc = copy_out(c, out, xout, nout);
   if (rc) return rc;
   rc = cuda_check(c, "apply");
   if (rc == WSI_OK && op == WSI_OP_STOKES) rc = df_check(c);
@@ -1350,30 +1381,37 @@ int wsi_transport(wsi_ctx* c, const double* u_n, const double* u_nm1, const doub
   if (valid_ctx(c)) return WSI_ERR_INVALID_ARG;
   if (!c->have_phases) return fail(c, WSI_ERR_INVALID_ARG, "no phases set");
   size_t nv = c->nvel;
-  // u_n -> vel_half, u^{n-1} -> u1 scratch copy, u_k -> vel_k
-  int rc = copy_in(c, c->vel_half, u_n, nv);
-  if (!rc) rc = copy_in(c, c->rs2, u_nm1, nv);
-  if (!rc && k > 0) rc = copy_in(c, c->vel_k, u_k, nv);
+  // u^{n-1} becomes the stored previous velocity; the two others are read where
+  // they are
+  const double *un = nullptr, *uk = nullptr;
+  int rc = use_in(c, un, u_n, nv, c->vel_half);
+  if (!rc && k > 0) rc = use_in(c, uk, u_k, nv, c->vel_k);
+  if (!rc) rc = copy_in(c, c->vel_old, u_nm1, nv);
   if (rc) return rc;
   PhaseConst pc = phase_const(c);
   launch_materials(c->g, pc, c->phi, c->psi, c->rho_cc_tmp, c->mu_cc_n, c->rho_n, c->beta_n, c->rho_flow_n,
                    c->mu_e_n, c->st);
-  // the stage buffers of the plain path alias rs2 only after u^(1), u^(2)
-  // are formed, so copy u^{n-1} aside first
-  cudaMemcpyAsync(c->vel_old, c->rs2, nv * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
-  transport_stage(c, k, dt, c->vel_half, c->vel_old, c->vel_k, false);
+  transport_stage(c, k, dt, un, c->vel_old, uk, false);
   c->mat_n_valid = false;  // the operator coefficients now hold the transported density
   c->pc_dirty = true;
-  double* rq[3];
-  parts(c, c->b, rq);
-  for (int d = 0; d < 3; ++d)
-    cudaMemcpyAsync(rq[d], c->rho_face[d], fsize(c->g, d) * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
-  if (c->mixed())
-    launch_lincomb_mix(nv, 0.0, c->Cc, 1.0, c->C32, 0.0, c->C32, c->x, c->st);
-  else
-    cudaMemcpyAsync(c->x, c->Cc, nv * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
-  rc = copy_out(c, rho_out, c->b, nv);
-  if (!rc) rc = copy_out(c, C_out, c->x, nv);
+  // (every input has been read by now: the outputs may overlap them)
+  if (usable(rho_out)) {
+    for (int d = 0; d < 3 && !rc; ++d) rc = copy_out(c, rho_out + c->pk.off[d], c->rho_face[d], fsize(c->g, d));
+  } else {
+    double* rq[3];
+    parts(c, c->b, rq);
+    for (int d = 0; d < 3; ++d)
+      cudaMemcpyAsync(rq[d], c->rho_face[d], fsize(c->g, d) * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
+    rc = copy_out(c, rho_out, c->b, nv);
+  }
+  if (rc) return rc;
+  if (!c->mixed()) {
+    rc = copy_out(c, C_out, c->Cc, nv);
+  } else {
+    double* const w = usable(C_out) ? C_out : c->x;
+    launch_widen(c->C32, nv, w, c->st);
+    if (w != C_out) rc = copy_out(c, C_out, w, nv);
+  }
   if (rc) return rc;
   return cuda_check(c, "transport");
 }
@@ -1441,13 +1479,17 @@ int wsi_advect_levelset(wsi_ctx* c, const double* vel, const double* phi_n, cons
   // phi_half = (phi_k + phi_n)/2 with phi_k = 2 phi_half - phi_n; likewise the
   // velocity is passed as u_half = (u_half + u_half)/2
   // (scratch buffers only: the stored level sets are left untouched)
-  int rc = copy_in(c, c->vel_k, vel, c->nvel);
-  if (!rc) rc = copy_in(c, c->psi_new, phi_n, c->ncell);
-  if (!rc) rc = copy_in(c, c->phi_half, phi_half, c->ncell);
+  const double *v = nullptr, *pn = nullptr, *ph = nullptr;
+  int rc = use_in(c, v, vel, c->nvel, c->vel_k);
+  if (!rc) rc = use_in(c, pn, phi_n, c->ncell, c->psi_new);
+  if (!rc) rc = use_in(c, ph, phi_half, c->ncell, c->phi_half);
   if (rc) return rc;
-  launch_lincomb(c->ncell, 2.0, c->phi_half, -1.0, c->psi_new, 0.0, nullptr, c->phi_k, c->st);
-  levelset_stage(c, c->vel_k, c->vel_k, c->phi_k, c->psi_new, dt, c->phi_new);
-  rc = copy_out(c, phi_out, c->phi_new, c->ncell);
+  launch_lincomb(c->ncell, 2.0, ph, -1.0, pn, 0.0, nullptr, c->phi_k, c->st);
+  const bool direct = usable(phi_out) && !overlap(phi_out, c->ncell, pn, c->ncell) &&
+                      !overlap(phi_out, c->ncell, v, c->nvel);
+  double* const dst = direct ? phi_out : c->phi_new;
+  levelset_stage(c, v, v, c->phi_k, pn, dt, dst);
+  if (!direct) rc = copy_out(c, phi_out, dst, c->ncell);
   if (rc) return rc;
   return cuda_check(c, "advect_levelset");
 }

@@ -160,6 +160,8 @@ void launch_lincomb_mix(size_t n, double a, const double* x, double b, const flo
 void launch_shift_scale_f32(size_t n, const double* x, double m, int e, float* y, cudaStream_t st);
 void launch_axpy_f32(size_t n, double a, const float* y, double* x, cudaStream_t st);
 void launch_shift(size_t n, double* x, double m, cudaStream_t st);
+// out = x widened to float64
+void launch_widen(const float* x, size_t n, double* out, cudaStream_t st);
 // z-chunk of the plane-marching stencil kernels for an ex x ey x ez box of
 // points (32 x 8 tiles): long marches, yet about 8 blocks per SM
 int transport_chunk(int ex, int ey, int ez);

@@ -629,6 +629,14 @@ void launch_lincomb_mix(size_t n, double a, const double* x, double b, const flo
   { k_lincomb_mix<<<lc_blocks(n), 256, 0, st>>>(n, a, x, b, y, c, z, out); WSI_COUNT(); }
 }
 
+__global__ void k_widen(const float* __restrict__ x, size_t n, double* out) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
+    out[t] = f2d_fast(x[t]);
+}
+void launch_widen(const float* x, size_t n, double* out, cudaStream_t st) {
+  { k_widen<<<lc_blocks(n), 256, 0, st>>>(x, n, out); WSI_COUNT(); }
+}
+
 // The mean is taken off in float32 pairs and the scale is a power of two, so
 // the result carries one rounding and no float64 operation (1/64 of the
 // float32 rate) is spent.
