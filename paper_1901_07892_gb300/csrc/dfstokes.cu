@@ -417,6 +417,7 @@ struct PadSplit {
   float2* out[DF_NARR];
   float* f32[DF_NARR];  // dense float32 copy (unscaled), or null
   double scale[DF_NARR];
+  int unit[DF_NARR];  // scale is 1 (a float64 comparison per element would bound the pass)
   int cols[DF_NARR], pitch[DF_NARR], nrows[DF_NARR];
   int count;
 };
@@ -426,6 +427,7 @@ __global__ void __launch_bounds__(256) k_df_split_pad(PadSplit s) {
   if (a >= s.count) return;
   const int cols = s.cols[a], pitch = s.pitch[a], nr = s.nrows[a];
   const double sc = s.scale[a];
+  const bool unit = s.unit[a] != 0;
   const int lane = threadIdx.x & 31;
   const int wstride = gridDim.x * (blockDim.x >> 5);
   for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < nr; r += wstride) {
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(256) k_df_split_pad(PadSplit s) {
       for (int u = 0; u < 4; ++u) {
         const int c = c0 + 32 * u;
         if (c < pitch) {
-          const dfl d = df_split(sc == 1.0 ? v[u] : sc * v[u]);
+          const dfl d = df_split(unit ? v[u] : sc * v[u]);
           orow[c] = make_float2(d.h, d.l);
           if (s.f32[a] && c < cols) s.f32[a][(size_t)r * cols + c] = d2f_fast(v[u]);
         }
@@ -463,6 +465,7 @@ static void split_pad(const DfOperands& o, const int* which, const double* const
     s.out[q] = o.a[a];
     s.f32[q] = f32 ? f32[q] : nullptr;
     s.scale[q] = scale[q];
+    s.unit[q] = scale[q] == 1.0;
     s.cols[q] = o.cols[a];
     s.pitch[q] = o.pitch[a];
     s.nrows[q] = o.rows[a] * o.levels[a];
