@@ -42,7 +42,7 @@ FP64_PEAK_DERIVED_GFLOPS = 152 * 2 * 2 * 2.07
 # DRAM bytes per cell of one launch, measured with ncu at 128^3 (dram__bytes_read.sum +
 # dram__bytes_write.sum, profiles/k_stokes_df_tank128.md) for the current kernel revision;
 # scaled by the cells of the workload (empty while no capture of the current revision exists)
-TRAFFIC_PER_CELL = {("stokes", "mixed"): (200.392192e6 + 46.134528e6) / 128 ** 3}
+TRAFFIC_PER_CELL = {}
 KCLASS = {"stokes": 0, "rbgs_p": 1, "rbgs_v": 2, "transport": 3, "mdot": 4, "maxpy": 5, "restrict": 6,
           "prolong": 7, "reinit": 8}
 
@@ -56,7 +56,9 @@ def kernel_model(name, nx, ny, nz, prec_bytes):
     if name == "stokes":
         # read u,v,w,p, rho_face, mu_cc, mu_edges; write 4 outputs: 8 bytes each
         # (float64, or the (hi, lo) float32 pairs of the double-float matvec)
-        byts = 8 * (F + N + F + N + E + F + N)
+        # (mixed: half of the launches read the velocity as float32; counted so
+        # for all of them)
+        byts = 8 * (F + N + F + N + E + F + N) - (0 if prec_bytes == 8 else 4 * F)
         flops = 44 * F + 8 * N
         # float64 arithmetic is bound by the float64 pipe; the double-float
         # matvec of the mixed path is reported against HBM
@@ -69,11 +71,12 @@ def kernel_model(name, nx, ny, nz, prec_bytes):
         byts = prec_bytes * (F + F // 2 + F + N + E + F // 2)
         return byts, 50 * F // 2, "hbm"
     if name == "transport":
-        # launches differ (density only, or with the velocity): the library
-        # sums each launch's algorithmic bytes (wsi_ktimer_bytes): per
-        # component the transported density, the three velocity arrays of the
-        # advective velocities, the transported velocity (convective term)
-        # and the result, in the storage type
+        # launches differ (a density stage, or the last one with the
+        # velocity): the library sums each launch's algorithmic bytes
+        # (wsi_ktimer_bytes): per component the transported density, the three
+        # velocity arrays of the advective velocities, a stage's other input
+        # and its result, the transported velocity and the momentum flux in the
+        # storage type, the last stage's float64 input and results
         return None, None, "hbm"
     if name in ("mdot", "maxpy"):
         # launches differ in the number of basis vectors: the library sums

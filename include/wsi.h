@@ -18,7 +18,10 @@
  *   Faces lying on a wall carry the zero normal velocity; they are not
  *   unknowns and every output writes 0 there.
  * Memory.  Array arguments may be device pointers or host pointers (pageable
- *   or pinned): the library copies with cudaMemcpyDefault on its stream.
+ *   or pinned): the library copies with cudaMemcpyDefault on its stream, or
+ *   (wsi_apply, wsi_transport, wsi_advect_levelset) reads and writes arrays of
+ *   the current device on a 16-byte boundary in place.  Outputs may lie on
+ *   inputs.
  *   The caller keeps ownership of everything it passes; the library copies
  *   what it needs and never keeps a caller pointer after returning.
  *   The context owns all device state it allocates, on the stream given at

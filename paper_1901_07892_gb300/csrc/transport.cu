@@ -5,9 +5,10 @@
 // momentum) is a divergence over face-centred control volumes.  Each flux
 // through a control-volume face is shared by the two C-faces on either side
 // of it, so the kernel computes it once: a 32 x 8 block owns a tile of
-// C-faces in (x, y) and marches up a chunk of z-planes; x- and y-fluxes of a
-// plane go through shared memory (one halo column / row computed by the edge
-// threads), the z-flux of the plane below is kept in a register.  The
+// C-faces in (x, y) and marches up a chunk of z-planes; x-fluxes go to the next
+// lane by shuffle and y-fluxes through shared memory (those through the tile's
+// lower edges come from a ninth warp), the z-flux of the plane below is kept in a
+// register.  The
 // limiter's inputs are staged per plane in shared memory (see k_transport).
 //
 // Storage and arithmetic type T: float64 on the plain path; float32 on the
