@@ -4,6 +4,7 @@
 // ops.cu, mg.cu, krylov.cu and dlm.cu; the host only sequences launches,
 // runs the (m+1) x m Hessenberg least-squares update of FGMRES and solves the
 // 3 x 3 inertia system of a free body.
+#include <cuda.h>
 #include <math.h>
 
 #include <algorithm>
@@ -271,11 +272,26 @@ int copy_out(wsi_ctx* c, double* dst, const double* src, size_t n) {
   return WSI_OK;
 }
 
-// Whether kernels can take a caller's array as it is: memory of
-// the current device, aligned as the library's own arrays are used (16 bytes).
-// (The calls return only after their stream has been synchronised, so the array
-// outlives its use.)  Everything else goes through a staging copy.
-bool usable(const void* p) {
+// cuMemGetAddressRange, reached through the runtime's driver entry point
+typedef CUresult (*AddressRangeFn)(CUdeviceptr*, size_t*, CUdeviceptr);
+AddressRangeFn address_range_fn() {
+  static const AddressRangeFn f = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &q) ==
+                        cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? (AddressRangeFn)fn : (AddressRangeFn) nullptr;
+  }();
+  return f;
+}
+
+// Whether kernels can take a caller's array of n doubles as it is: inside one
+// allocation on the current device, aligned as the library's own arrays are used
+// (16 bytes).  (The calls return only after their stream has been synchronised,
+// so the array outlives its use.)  Everything else goes through a staging copy,
+// whose own checks refuse what is not an array.
+bool usable(const void* p, size_t n) {
   if (!p || ((uintptr_t)p & 15)) return false;
   cudaPointerAttributes at;
   int dev = -1;
@@ -283,7 +299,12 @@ bool usable(const void* p) {
     cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
+  if (at.type != cudaMemoryTypeDevice || cudaGetDevice(&dev) != cudaSuccess || at.device != dev) return false;
+  const AddressRangeFn range = address_range_fn();
+  CUdeviceptr base = 0;
+  size_t bytes = 0;
+  return range && range(&base, &bytes, (CUdeviceptr)p) == CUDA_SUCCESS &&
+         (CUdeviceptr)p + n * sizeof(double) <= base + bytes;
 }
 bool overlap(const double* a, size_t na, const double* b, size_t nb) {
   const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
@@ -291,7 +312,7 @@ bool overlap(const double* a, size_t na, const double* b, size_t nb) {
 }
 // the caller's array itself where kernels can read it, else its copy in staging
 int use_in(wsi_ctx* c, const double*& use, const double* src, size_t n, double* staging) {
-  if (usable(src)) {
+  if (usable(src, n)) {
     use = src;
     return WSI_OK;
   }
@@ -1348,7 +1369,7 @@ int wsi_apply(wsi_ctx* c, int op, const double* in, double* out, double dt) {
   int rc = use_in(c, xin, in, nin, c->b);
   if (rc) return rc;
   // (at 250 x 182 x 126 the two copies were 108 of 630 us)
-  const bool direct = usable(out) && !overlap(out, nout, xin, nin);
+  const bool direct = usable(out, nout) && !overlap(out, nout, xin, nin);
   if (direct) xout = out;
   const double* qi[3];
   double* qo[3];
@@ -1395,7 +1416,7 @@ int wsi_transport(wsi_ctx* c, const double* u_n, const double* u_nm1, const doub
   c->mat_n_valid = false;  // the operator coefficients now hold the transported density
   c->pc_dirty = true;
   // (every input has been read by now: the outputs may overlap them)
-  if (usable(rho_out)) {
+  if (usable(rho_out, nv)) {
     for (int d = 0; d < 3 && !rc; ++d) rc = copy_out(c, rho_out + c->pk.off[d], c->rho_face[d], fsize(c->g, d));
   } else {
     double* rq[3];
@@ -1408,7 +1429,7 @@ int wsi_transport(wsi_ctx* c, const double* u_n, const double* u_nm1, const doub
   if (!c->mixed()) {
     rc = copy_out(c, C_out, c->Cc, nv);
   } else {
-    double* const w = usable(C_out) ? C_out : c->x;
+    double* const w = usable(C_out, nv) ? C_out : c->x;
     launch_widen(c->C32, nv, w, c->st);
     if (w != C_out) rc = copy_out(c, C_out, w, nv);
   }
@@ -1485,7 +1506,7 @@ int wsi_advect_levelset(wsi_ctx* c, const double* vel, const double* phi_n, cons
   if (!rc) rc = use_in(c, ph, phi_half, c->ncell, c->phi_half);
   if (rc) return rc;
   launch_lincomb(c->ncell, 2.0, ph, -1.0, pn, 0.0, nullptr, c->phi_k, c->st);
-  const bool direct = usable(phi_out) && !overlap(phi_out, c->ncell, pn, c->ncell) &&
+  const bool direct = usable(phi_out, c->ncell) && !overlap(phi_out, c->ncell, pn, c->ncell) &&
                       !overlap(phi_out, c->ncell, v, c->nvel);
   double* const dst = direct ? phi_out : c->phi_new;
   levelset_stage(c, v, v, c->phi_k, pn, dt, dst);
