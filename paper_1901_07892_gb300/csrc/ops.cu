@@ -8,6 +8,8 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
+#include <limits>
 
 #include "internal.h"
 
@@ -595,7 +597,9 @@ double host_pressure_residual(const GridDev& g, const double* const beta[3], con
   if (!mean) return sqrt(h[1]);
   const double n = (double)g.n[0] * g.n[1] * g.n[2];
   *mean = h[0] / n;
-  return sqrt(fmax(h[1] - h[0] * *mean, h[1] == h[1] ? 0.0 : h[1]));
+  // (sums that overflow or hold a NaN are no small residual: inf - inf below)
+  if (!std::isfinite(h[0]) || !std::isfinite(h[1])) return std::numeric_limits<double>::infinity();
+  return sqrt(std::max(h[1] - h[0] * *mean, 0.0));
 }
 
 template <int C, typename T>
