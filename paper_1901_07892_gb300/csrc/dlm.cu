@@ -517,11 +517,14 @@ __global__ void __launch_bounds__(32 * CW, 8) k_interp_cells(GridDev g, const do
               const float2 a = V[ky * nx + kx];
               sr = df_add(sr, df_mul(wx[kx], dfl{a.x, a.y}));
             }
+            // (a row or plane of weight zero is left out, as in k_interp_list:
+            // what it holds need not be finite)
             const float2 a = W[ty * 4 + ky];
-            sz = df_add(sz, df_mul(dfl{a.x, a.y}, sr));
+            const dfl t = df_add(sz, df_mul(dfl{a.x, a.y}, sr));
+            if (a.x != 0.0f) sz = t;
           }
           const float2 a = W[tz * 4 + kz];
-          s = df_mul(dfl{a.x, a.y}, sz);
+          if (a.x != 0.0f) s = df_mul(dfl{a.x, a.y}, sz);
         }
         // z taps in order: lane kz = 0 adds its three neighbours'
         dfl tot = s;
