@@ -221,11 +221,12 @@ __device__ __forceinline__ void coarsen_face(const GridDev& gf, const GridDev& g
   bc[fidx(gc, C, i, j, k)] = s / T(span[0] * span[1] * span[2]);
 }
 
-// the three face arrays in one launch: blockIdx.z walks the z-planes of each
+// the three face arrays in one launch, one after another along blockIdx.x (y and z
+// of a grid end at 65535, and the planes of one array may use all of that)
 template <typename T>
 __global__ void k_coarsen_faces(GridDev gf, GridDev gc, int r0, int r1, int r2, CVel<T> f, Vel<T> c) {
-  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, n2 = gc.n[2] + 1;
-  const int q = blockIdx.z / n2, k = blockIdx.z - q * n2;
+  const int nb = gridDim.x / 3, q = blockIdx.x / nb;
+  const int i = (blockIdx.x - q * nb) * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
   if (q == 0) coarsen_face<0, T>(gf, gc, r0, r1, r2, f.q[0], c.q[0], i, j, k);
   else if (q == 1) coarsen_face<1, T>(gf, gc, r0, r1, r2, f.q[1], c.q[1], i, j, k);
   else coarsen_face<2, T>(gf, gc, r0, r1, r2, f.q[2], c.q[2], i, j, k);
@@ -233,7 +234,7 @@ __global__ void k_coarsen_faces(GridDev gf, GridDev gc, int r0, int r1, int r2, 
 
 template <typename T>
 static void coarsen_faces(const MGLevel<T>& F, const GridDev& gc, const T* const f[3], T* const c[3], cudaStream_t st) {
-  const dim3 grid(cdiv(gc.n[0] + 1, BX), cdiv(gc.n[1] + 1, BY), 3 * (gc.n[2] + 1));
+  const dim3 grid(3 * cdiv(gc.n[0] + 1, BX), cdiv(gc.n[1] + 1, BY), gc.n[2] + 1);
   { k_coarsen_faces<T><<<grid, dim3(BX, BY), 0, st>>>(F.g, gc, F.r[0], F.r[1], F.r[2], CVel<T>{{f[0], f[1], f[2]}},
                                                       Vel<T>{{c[0], c[1], c[2]}}); WSI_COUNT(); }
 }
