@@ -768,31 +768,18 @@ __global__ void k_rbgs_p(PLevel<T> p, T* x, int color) {
 
 // Four neighbouring cells at a time (rows of a multiple of four cells, so that
 // every row of a cell or y/z-face array starts on a 16-byte boundary; x-face
-// rows have one element more and are read one by one)
-template <typename T>
+// rows have one element more and are read one by one).  float32 only, as the three
+// kernels that use them: in float64 the pipe bounds an update, and two in a row per
+// thread cost 5 % more.
 struct Quad {
-  T v[4];
+  float v[4];
 };
-template <typename T>
-__device__ __forceinline__ Quad<T> load4(const T* a) {
-  Quad<T> q;
-  if constexpr (sizeof(T) == 4) {
-    const float4 f = *reinterpret_cast<const float4*>(a);
-    q.v[0] = f.x, q.v[1] = f.y, q.v[2] = f.z, q.v[3] = f.w;
-  } else {
-    const double2 f = reinterpret_cast<const double2*>(a)[0], h = reinterpret_cast<const double2*>(a)[1];
-    q.v[0] = f.x, q.v[1] = f.y, q.v[2] = h.x, q.v[3] = h.y;
-  }
-  return q;
+__device__ __forceinline__ Quad load4(const float* a) {
+  const float4 f = *reinterpret_cast<const float4*>(a);
+  return Quad{{f.x, f.y, f.z, f.w}};
 }
-template <typename T>
-__device__ __forceinline__ void store4(T* a, const Quad<T>& q) {
-  if constexpr (sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(a) = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]);
-  } else {
-    reinterpret_cast<double2*>(a)[0] = make_double2(q.v[0], q.v[1]);
-    reinterpret_cast<double2*>(a)[1] = make_double2(q.v[2], q.v[3]);
-  }
+__device__ __forceinline__ void store4(float* a, const Quad& q) {
+  *reinterpret_cast<float4*>(a) = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]);
 }
 
 // One colour of a red-black sweep, four cells (two of the colour) per thread:
@@ -800,10 +787,9 @@ __device__ __forceinline__ void store4(T* a, const Quad<T>& q) {
 // colour's values go back as they were read).  ZERO: x is zero on entry and not
 // read.  HBM-bound: x, b and the three coefficient arrays stream once per half
 // sweep, 24 bytes per cell; at 256^3 58.6 us, 6.9 TB/s (one cell per
-// thread, 64-bit indices: 98 us).  float32 only: in float64 the pipe bounds the
-// update and two updates in a row per thread cost 5 % more.
-template <typename T, bool ZERO>
-__global__ void __launch_bounds__(256) k_rbgs_p4(PLevel<T> p, T* x, int color) {
+// thread, 64-bit indices: 98 us).
+template <bool ZERO>
+__global__ void __launch_bounds__(256) k_rbgs_p4(PLevel<float> p, float* x, int color) {
   const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nq = nx >> 2;
   const int t = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
   const int j = t / nq;
@@ -811,9 +797,9 @@ __global__ void __launch_bounds__(256) k_rbgs_p4(PLevel<T> p, T* x, int color) {
   const int i0 = 4 * (t - j * nq), pl = nx * ny;
   const int r = k * ny + j, id = r * nx + i0, oy = id + k * nx, ox = id + r;
   const int q = (j + k + color) & 1;  // cells i0 + q and i0 + q + 2
-  const Quad<T> b = load4(p.b + id);
-  Quad<T> xc, xyl, xyh, xzl, xzh, yl, yh, zl, zh;
-  T xe = T(0), fx[4];
+  const Quad b = load4(p.b + id);
+  Quad xc, xyl, xyh, xzl, xzh, yl, yh, zl, zh;
+  float xe = 0.0f, fx[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) fx[a] = p.bx[ox + q + a];
   yl = load4(p.by + oy);
@@ -829,16 +815,16 @@ __global__ void __launch_bounds__(256) k_rbgs_p4(PLevel<T> p, T* x, int color) {
     if (q ? i0 + 4 < nx : i0 > 0) xe = q ? x[id + 4] : x[id - 1];
   } else {
 #pragma unroll
-    for (int a = 0; a < 4; ++a) xc.v[a] = T(0);
+    for (int a = 0; a < 4; ++a) xc.v[a] = 0.0f;
   }
   auto update = [&](auto QC) {
     constexpr int Q = decltype(QC)::value;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int m = Q + 2 * h;  // place in the quad
-      const Faces<T> f{fx[2 * h + 1], fx[2 * h], yh.v[m], yl.v[m], zh.v[m], zl.v[m]};
-      xc.v[m] = gs_value<T>(p, f, i0 + m, j, k, b.v[m], T(0), [&](int a, int c, int d) {
-        if (ZERO) return T(0);
+      const Faces<float> f{fx[2 * h + 1], fx[2 * h], yh.v[m], yl.v[m], zh.v[m], zl.v[m]};
+      xc.v[m] = gs_value<float>(p, f, i0 + m, j, k, b.v[m], 0.0f, [&](int a, int c, int d) {
+        if (ZERO) return 0.0f;
         if (a == 1) return m == 3 ? xe : xc.v[m < 3 ? m + 1 : 3];
         if (a == -1) return m == 0 ? xe : xc.v[m > 0 ? m - 1 : 0];
         if (c == 1) return xyh.v[m];
@@ -892,41 +878,40 @@ __global__ void k_prolong_add(GridDev gf, GridDev gc, int r0, int r1, int r2, co
 // The same with every axis coarsened, two coarse cells (a fine quad of 2 x 2
 // rows) per thread: 56 loads for 16 fine cells instead of 224 (84 -> 56 us at
 // 256^3).
-template <typename T>
-__global__ void __launch_bounds__(128) k_restrict_res4(PLevel<T> p, const T* __restrict__ x, T* bcoarse) {
+__global__ void __launch_bounds__(128) k_restrict_res4(PLevel<float> p, const float* __restrict__ x, float* bcoarse) {
   const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nq = nx >> 2, m1 = ny >> 1;
   const int t = blockIdx.x * 128 + threadIdx.x, K = blockIdx.y;
   const int J = t / nq;
   if (J >= m1) return;
   const int i0 = 4 * (t - J * nq), j0 = 2 * J, k0 = 2 * K, pl = nx * ny;
-  T s[2] = {T(0), T(0)};
+  float s[2] = {0.0f, 0.0f};
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int k = k0 + c;
-    Quad<T> xr[4];  // rows j0 - 1 .. j0 + 2
+    Quad xr[4];  // rows j0 - 1 .. j0 + 2
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       const int j = j0 - 1 + a;
       if (j >= 0 && j < ny) xr[a] = load4(x + (k * ny + j) * nx + i0);
     }
-    Quad<T> fy[3];
+    Quad fy[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) fy[a] = load4(p.by + (k * (ny + 1) + j0 + a) * nx + i0);
 #pragma unroll
     for (int bb = 0; bb < 2; ++bb) {
       const int j = j0 + bb, r = k * ny + j, id = r * nx + i0;
-      const Quad<T> b = load4(p.b + id), zl = load4(p.bz + id), zh = load4(p.bz + id + pl);
-      Quad<T> xzl, xzh;
+      const Quad b = load4(p.b + id), zl = load4(p.bz + id), zh = load4(p.bz + id + pl);
+      Quad xzl, xzh;
       if (k > 0) xzl = load4(x + id - pl);
       if (k + 1 < nz) xzh = load4(x + id + pl);
-      const T xm = i0 > 0 ? x[id - 1] : T(0), xp = i0 + 4 < nx ? x[id + 4] : T(0);
-      T fx[5];
+      const float xm = i0 > 0 ? x[id - 1] : 0.0f, xp = i0 + 4 < nx ? x[id + 4] : 0.0f;
+      float fx[5];
 #pragma unroll
       for (int a = 0; a < 5; ++a) fx[a] = p.bx[id + r + a];
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const Faces<T> f{fx[m + 1], fx[m], fy[bb + 1].v[m], fy[bb].v[m], zh.v[m], zl.v[m]};
-        s[m >> 1] += b.v[m] - lap_value<T>(p, f, i0 + m, j, k, [&](int da, int db, int dc) {
+        const Faces<float> f{fx[m + 1], fx[m], fy[bb + 1].v[m], fy[bb].v[m], zh.v[m], zl.v[m]};
+        s[m >> 1] += b.v[m] - lap_value<float>(p, f, i0 + m, j, k, [&](int da, int db, int dc) {
           if (da == 1) return m == 3 ? xp : xr[bb + 1].v[m < 3 ? m + 1 : 3];
           if (da == -1) return m == 0 ? xm : xr[bb + 1].v[m > 0 ? m - 1 : 0];
           if (db == 1) return xr[bb + 2].v[m];
@@ -939,14 +924,13 @@ __global__ void __launch_bounds__(128) k_restrict_res4(PLevel<T> p, const T* __r
     }
   }
   const int o = (K * m1 + J) * (nx >> 1) + (i0 >> 1);
-  bcoarse[o] = s[0] / T(8);
-  bcoarse[o + 1] = s[1] / T(8);
+  bcoarse[o] = s[0] / 8.0f;
+  bcoarse[o + 1] = s[1] / 8.0f;
 }
 
 // x_fine += P x_coarse with every axis coarsened, four fine cells per thread
 // (16 coarse loads instead of 32; 149 -> 44 us per cycle over all levels at 256^3)
-template <typename T>
-__global__ void __launch_bounds__(256) k_prolong_add4(int nx, int ny, int m2, const T* __restrict__ xc, T* xf) {
+__global__ void __launch_bounds__(256) k_prolong_add4(int nx, int ny, int m2, const float* __restrict__ xc, float* xf) {
   const int nq = nx >> 2, t = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y, j = t / nq;
   if (j >= ny) return;
   const int i0 = 4 * (t - j * nq), mx = nx >> 1, my = ny >> 1;
@@ -954,20 +938,20 @@ __global__ void __launch_bounds__(256) k_prolong_add4(int nx, int ny, int m2, co
   const int J1 = clampi((j & 1) ? J0 + 1 : J0 - 1, 0, my - 1), K1 = clampi((k & 1) ? K0 + 1 : K0 - 1, 0, m2 - 1);
   const int Im = max(I0 - 1, 0), Ip = min(I0 + 2, mx - 1);
   const int id = (k * ny + j) * nx + i0;
-  Quad<T> f = load4(xf + id), s;
+  Quad f = load4(xf + id), s;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) s.v[m] = T(0);
+  for (int m = 0; m < 4; ++m) s.v[m] = 0.0f;
 #pragma unroll
   for (int cz = 0; cz < 2; ++cz)
 #pragma unroll
     for (int cy = 0; cy < 2; ++cy) {
-      const T* row = xc + ((cz ? K1 : K0) * my + (cy ? J1 : J0)) * mx;
-      const T a[4] = {row[Im], row[I0], row[I0 + 1], row[Ip]};
+      const float* row = xc + ((cz ? K1 : K0) * my + (cy ? J1 : J0)) * mx;
+      const float a[4] = {row[Im], row[I0], row[I0 + 1], row[Ip]};
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const T wyz = (cy ? T(0.25) : T(0.75)) * (cz ? T(0.25) : T(0.75));
-        s.v[m] += T(0.75) * wyz * a[1 + (m >> 1)];
-        s.v[m] += T(0.25) * wyz * a[(m & 1) ? 2 + (m >> 1) : (m >> 1)];
+        const float wyz = (cy ? 0.25f : 0.75f) * (cz ? 0.25f : 0.75f);
+        s.v[m] += 0.75f * wyz * a[1 + (m >> 1)];
+        s.v[m] += 0.25f * wyz * a[(m & 1) ? 2 + (m >> 1) : (m >> 1)];
       }
     }
 #pragma unroll
@@ -1295,11 +1279,16 @@ template <typename T>
 static void half_sweep(MGLevel<T>& L, int color, bool zero, cudaStream_t st) {
   const GridDev& g = L.g;
   ktimer_begin(KC_RBGS_P, st);
-  if (sizeof(T) == 4 && g.n[0] % 4 == 0) {
-    const dim3 grid(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]);
-    if (zero) k_rbgs_p4<T, true><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
-    else k_rbgs_p4<T, false><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
-  } else {
+  bool done = false;
+  if constexpr (sizeof(T) == 4) {
+    if (g.n[0] % 4 == 0) {
+      const dim3 grid(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]);
+      if (zero) k_rbgs_p4<true><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
+      else k_rbgs_p4<false><<<grid, 256, 0, st>>>(plevel(L), L.x, color);
+      done = true;
+    }
+  }
+  if (!done) {
     if (zero) cudaMemsetAsync(L.x, 0, fsize(g, 3) * sizeof(T), st);
     k_rbgs_p<T><<<grid_rb(g), dim3(BX, BY), 0, st>>>(plevel(L), L.x, color);
   }
@@ -1361,19 +1350,23 @@ static void coarse_part(Precond<T>& P, const Opts& o, size_t l, bool zero, cudaS
   const GridDev& gc = Cl.g;
   ktimer_begin(KC_RESTRICT, st);
   const bool quads = sizeof(T) == 4 && g.n[0] % 4 == 0 && L.r[0] == 2 && L.r[1] == 2 && L.r[2] == 2;
-  if (quads)
-    k_restrict_res4<T><<<dim3(cdiv((long long)(g.n[0] / 4) * gc.n[1], 128), gc.n[2]), 128, 0, st>>>(plevel(L), L.x, Cl.b);
-  else
+  if constexpr (sizeof(T) == 4) {
+    if (quads)
+      k_restrict_res4<<<dim3(cdiv((long long)(g.n[0] / 4) * gc.n[1], 128), gc.n[2]), 128, 0, st>>>(plevel(L), L.x, Cl.b);
+  }
+  if (!quads)
     k_restrict_res<T><<<grid3(gc.n[0], gc.n[1], gc.n[2]), dim3(BX, BY), 0, st>>>(plevel(L), gc.n[0], gc.n[1], L.r[0],
                                                                               L.r[1], L.r[2], L.x, Cl.b);
   WSI_COUNT();
   ktimer_end(KC_RESTRICT, st);
   vcycle(P, o, l + 1, true, st);
   ktimer_begin(KC_PROLONG, st);
-  if (quads)
-    k_prolong_add4<T><<<dim3(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]), 256, 0, st>>>(g.n[0], g.n[1], gc.n[2],
-                                                                                               Cl.x, L.x);
-  else
+  if constexpr (sizeof(T) == 4) {
+    if (quads)
+      k_prolong_add4<<<dim3(cdiv((long long)(g.n[0] / 4) * g.n[1], 256), g.n[2]), 256, 0, st>>>(g.n[0], g.n[1], gc.n[2],
+                                                                                              Cl.x, L.x);
+  }
+  if (!quads)
     k_prolong_add<T><<<gr, dim3(BX, BY), 0, st>>>(g, gc, L.r[0], L.r[1], L.r[2], Cl.x, L.x);
   WSI_COUNT();
   ktimer_end(KC_PROLONG, st);
