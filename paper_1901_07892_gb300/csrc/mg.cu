@@ -394,9 +394,15 @@ static void spd_inverse(std::vector<double>& A, int n) {
 // The dense coarsest operator M = -L + c 1 1^T of the level and its inverse
 // (Gauss-Jordan in place, no pivoting: M is symmetric positive definite), one
 // block, the matrix in shared memory; the same operations as the host form
-// above.  float64-pipe bound, n^3 multiply-adds on one SM: about 80 us at 64
-// cells, but nothing waits for it on the host (read back, inverted there and
-// sent down it cost two synchronisations and about 0.4 ms per set-up).
+// below, in a launch that the host doesn't wait for (read back, inverted there and
+// sent down it costs two synchronisations).  Bound by the float64 pipe of one SM and
+// the chain of n pivots (a division, three barriers and n^2 multiply-adds each), so
+// only what the pivots need goes to that pipe: the reciprocal by one thread (by all
+// of them 73 us more at 64 cells), the test for zero on the bits, and the columns of
+// a row in whole warps (unrolled by lane, the last chunk split the warp: 1140 us at
+// 125 cells).  154 us at 64 cells, 757 at 125 (232 and 900 before).  A set-up and one
+// cycle of 4 x 4 x 4 cells 317 us (404; inverted on the host 330), of 8^3 340 (430,
+// 455), 40^3 1120 (1276, 1460), 44 x 28 x 8 1620 (1790, 1800).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_coarse_inverse(GridDev g, const T* __restrict__ bx, const T* __restrict__ by,
                                                          const T* __restrict__ bz, int n, double* inv) {
@@ -437,17 +443,21 @@ __global__ void __launch_bounds__(1024) k_coarse_inverse(GridDev g, const T* __r
   for (int w = 0; w < 32; ++w) dmax = fmax(dmax, dmax_w[w]);
   const double creg = g.open_top ? 0.0 : dmax / n;
   for (int t = tid; t < n * n; t += 1024) W[t] += creg;
+  __shared__ double rpiv;  // reciprocal of the pivot
   for (int p = 0; p < n; ++p) {
     __syncthreads();
-    const double id = 1.0 / W[p * n + p];
-    for (int r = tid; r < n; r += 1024) col[r] = W[r * n + p];
+    if (tid < n) col[tid] = W[tid * n + p];
+    if (tid == 1023) rpiv = 1.0 / W[p * n + p];  // (a warp of its own)
     __syncthreads();
-    for (int c = tid; c < n; c += 1024) W[p * n + c] = c == p ? id : W[p * n + c] * id;
+    if (tid < n) W[p * n + tid] = tid == p ? rpiv : W[p * n + tid] * rpiv;
     __syncthreads();
     for (int r = warp; r < n; r += 32) {
       const double f = col[r];
-      if (r == p || f == 0.0) continue;
-      for (int c = lane; c < n; c += 32) W[r * n + c] = fma(-f, W[p * n + c], c == p ? 0.0 : W[r * n + c]);
+      if (r == p || (__double_as_longlong(f) << 1) == 0) continue;
+      for (int c0 = 0; c0 < n; c0 += 32) {
+        const int c = c0 + lane;
+        if (c < n) W[r * n + c] = fma(-f, W[p * n + c], c == p ? 0.0 : W[r * n + c]);
+      }
     }
   }
   __syncthreads();
