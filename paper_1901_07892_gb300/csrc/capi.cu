@@ -183,7 +183,7 @@ bool ensure_bins(wsi_ctx* c, int n) {
     b.cnt = (int*)dalloc(c, c->ncell / 2 + 1);
     b.bcnt = (int*)dalloc(c, c->ncell / 2 + 1);
     b.ctr = (int*)dalloc(c, BIN_CTR_BYTES / 8);
-    b.fmx = (unsigned long long*)(b.ctr + 4);
+    b.fmx = (unsigned long long*)(b.ctr + 6);
     if (!b.cnt || !b.bcnt || !b.ctr) {
       b.cnt = nullptr;
       return false;
@@ -566,7 +566,7 @@ int dlm_project(wsi_ctx* c, double* velv, const double* Xuse) {
   Body& B = c->body;
   if (!ensure_spread_work(c) || !ensure_bins(c, B.n)) return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
   launch_marker_mean_box(Xuse, B.n, B.xc, c->mbox, B.scratch, c->st);
-  launch_marker_bins(c->g, Xuse, B.n, c->bins, c->st);
+  launch_marker_bins(c->g, Xuse, B.n, c->bins, true, c->st);
   launch_ib_interp(c->g, velv, Xuse, B.n, c->bins, B.U, c->st);
   // the fitted motion of a fully locked body is not used
   bool locked = true;
@@ -1534,7 +1534,7 @@ int wsi_interp(wsi_ctx* c, const double* vel, const double* X, int n, double* U)
   int rc = copy_in(c, c->vel_half, vel, c->nvel);
   if (!rc) rc = copy_in(c, dX, X, (size_t)n * 3);
   if (rc) return rc;
-  launch_marker_bins(c->g, dX, n, c->bins, c->st);
+  launch_marker_bins(c->g, dX, n, c->bins, false, c->st);
   launch_ib_interp(c->g, c->vel_half, dX, n, c->bins, dU, c->st);
   launch_marker_bins_clear(n, c->bins, c->st);
   rc = copy_out(c, U, dU, (size_t)n * 3);
@@ -1566,7 +1566,7 @@ int wsi_spread(wsi_ctx* c, const double* F, const double* X, int n, double dV, d
     if (n > 0) {
       double mm[6];
       launch_marker_mean_box(dX, n, c->red, c->mbox, c->red + 8, c->st);
-      launch_marker_bins(c->g, dX, n, c->bins, c->st);
+      launch_marker_bins(c->g, dX, n, c->bins, true, c->st);
       launch_force_max(dF, n, c->bins, c->st);
       cudaMemcpyAsync(mm, c->mbox, sizeof(mm), cudaMemcpyDeviceToHost, c->st);
       cudaStreamSynchronize(c->st);

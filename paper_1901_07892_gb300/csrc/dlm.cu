@@ -94,15 +94,34 @@ __device__ __forceinline__ void marker_taps(const GridDev& g, const double* __re
   }
 }
 
-// Irregular markers (outside the grid or not finite; none in an ordinary run):
-// one thread per marker of the list, all three components; separable sums
+// Markers of sparse cells get a warp per cell or, where there are at least this many
+// of them, a thread each: the warp has the lower latency, the thread does less work.
+// From markers at random over 96^3, the kernels of a call with a warp per cell and
+// with a thread per marker: interpolation 10000 53 and 100 us, 16500 71 and 91, 30000
+// 116 and 86, 300000 766 and 328; spreading 30000 125 and 171, 100000 251 and 254,
+// 300000 561 and 463.  (Cells of four or more: a million markers with a thread each
+// up to one, two and three to a cell 1281, 1038 and 1014 us, a warp each 1759.)
+static constexpr int INTERP_LIST_MIN = 24576, SPREAD_LIST_MIN = 131072;
+
+// The t-th marker of those that get a thread each: the irregular ones and, where
+// there are list_min or more of them, those of sparse cells (total: how many)
+__device__ __forceinline__ int list_total(const int* __restrict__ ctr, int list_min) {
+  return ctr[BIN_IRR] + (ctr[BIN_SPARSE] >= list_min ? ctr[BIN_SPARSE] : 0);
+}
+__device__ __forceinline__ int list_marker(int t, int n, const int* __restrict__ irr, const int* __restrict__ perm,
+                                           const int* __restrict__ ctr) {
+  return t < ctr[BIN_IRR] ? irr[t] : perm[n - 1 - (t - ctr[BIN_IRR])];
+}
+
+// One thread per marker, all three components; separable sums
 // sum_z w_z sum_y w_y sum_x w_x q in double-float, one float64 addition per
 // component at the end
-__global__ void __launch_bounds__(128) k_interp_list(GridDev g, CVel<double> vel, const double* __restrict__ X,
-                                                     const int* __restrict__ list, const int* __restrict__ ctr,
-                                                     double* U) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ctr[BIN_IRR]; t += gridDim.x * blockDim.x) {
-    const int m = list[t];
+__global__ void __launch_bounds__(128) k_interp_list(GridDev g, CVel<double> vel, const double* __restrict__ X, int n,
+                                                     const int* __restrict__ irr, const int* __restrict__ perm,
+                                                     const int* __restrict__ ctr, double* U) {
+  const int total = list_total(ctr, INTERP_LIST_MIN);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int m = list_marker(t, n, irr, perm, ctr);
     MarkerTaps T;
     marker_taps(g, X, m, T);
 #pragma unroll
@@ -113,11 +132,11 @@ __global__ void __launch_bounds__(128) k_interp_list(GridDev g, CVel<double> vel
       const double* __restrict__ q = vel.q[c];
       const size_t sx = (size_t)(g.n[0] + (c == 0)), sy = sx * (size_t)(g.n[1] + (c == 1));
       dfl s = df_from_float(0.0f);
-#pragma unroll 1
+#pragma unroll
       for (int kz = 0; kz < 4; ++kz) {
         if (tz.w[kz].h == 0.0f) continue;
         dfl sz = df_from_float(0.0f);
-#pragma unroll 1
+#pragma unroll
         for (int ky = 0; ky < 4; ++ky) {
           if (ty.w[ky].h == 0.0f) continue;
           const double* row = q + (size_t)tz.idx[kz] * sy + (size_t)ty.idx[ky] * sx;
@@ -167,15 +186,16 @@ __device__ __forceinline__ int spread_exponent(const int* __restrict__ ctr, cons
 }
 
 __global__ void __launch_bounds__(128) k_spread_list(GridDev g, const double* __restrict__ F,
-                                                     const double* __restrict__ X, const int* __restrict__ list,
-                                                     const int* __restrict__ ctr,
+                                                     const double* __restrict__ X, int n, const int* __restrict__ irr,
+                                                     const int* __restrict__ perm, const int* __restrict__ ctr,
                                                      const unsigned long long* __restrict__ fmx, double scale,
                                                      Vel<unsigned long long> acc) {
-  if (ctr[BIN_IRR] == 0) return;
+  const int total = list_total(ctr, SPREAD_LIST_MIN);
+  if (total == 0) return;
   const int E = spread_exponent(ctr, fmx, scale);
   const dfl sc = df_split(scale);
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ctr[BIN_IRR]; t += gridDim.x * blockDim.x) {
-    const int m = list[t];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int m = list_marker(t, n, irr, perm, ctr);
     MarkerTaps T;
     marker_taps(g, X, m, T);
 #pragma unroll
@@ -186,10 +206,10 @@ __global__ void __launch_bounds__(128) k_spread_list(GridDev g, const double* __
       unsigned long long* q = acc.q[c];
       const size_t sx = (size_t)(g.n[0] + (c == 0)), sy = sx * (size_t)(g.n[1] + (c == 1));
       const dfl f = df_mul(df_split(F[3 * m + c]), sc);
-#pragma unroll 1
+#pragma unroll
       for (int kz = 0; kz < 4; ++kz) {
         if (tz.w[kz].h == 0.0f) continue;
-#pragma unroll 1
+#pragma unroll
         for (int ky = 0; ky < 4; ++ky) {
           if (ty.w[ky].h == 0.0f) continue;
           const dfl wyz = df_mul(tz.w[kz], ty.w[ky]);
@@ -221,23 +241,31 @@ __device__ __forceinline__ int bound_cell(const GridDev& g, const double* __rest
 // positions; bcnt counts by the float64 ones, which may differ on a cell face.
 __global__ void __launch_bounds__(256) k_bin_count(GridDev g, const double* __restrict__ X, int n, int* cnt, int* bcnt,
                                                    int* cellof, int* rank, int* irr, int* ctr) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= n) return;
-  atomicAdd(&bcnt[bound_cell(g, X, m)], 1);
-  int c[3];
-  bool in = true;
+  const int m = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const bool valid = m < n;
+  int c[3] = {0, 0, 0};
+  bool in = valid;
+  if (valid) {
+    if (bcnt) atomicAdd(&bcnt[bound_cell(g, X, m)], 1);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const dfl x = df_split(X[3 * m + d]);
-    c[d] = df_floor(df_mul(x, df_split(g.ih[d])));
-    in = in && fabsf(x.h) < 1e30f && c[d] >= 0 && c[d] < g.n[d];
+    for (int d = 0; d < 3; ++d) {
+      const dfl x = df_split(X[3 * m + d]);
+      c[d] = df_floor(df_mul(x, df_split(g.ih[d])));
+      in = in && fabsf(x.h) < 1e30f && c[d] >= 0 && c[d] < g.n[d];
+    }
   }
-  if (!in) {
-    irr[atomicAdd(&ctr[BIN_IRR], 1)] = m;
-    cellof[m] = -1;
-    rank[m] = 0;
-    return;
+  const unsigned out = __ballot_sync(0xffffffffu, valid && !in);
+  if (out) {  // places in the irregular list, one atomic per warp
+    int first = 0;
+    if (lane == 0) first = atomicAdd(&ctr[BIN_IRR], __popc(out));
+    first = __shfl_sync(0xffffffffu, first, 0);
+    if (valid && !in) {
+      irr[first + __popc(out & ((1u << lane) - 1u))] = m;
+      cellof[m] = -1;
+      rank[m] = 0;
+    }
   }
+  if (!in) return;
   const int cell = (int)fidx(g, 3, c[0], c[1], c[2]);
   cellof[m] = cell;
   rank[m] = atomicAdd(&cnt[cell], 1);
@@ -247,48 +275,67 @@ __global__ void __launch_bounds__(256) k_bin_count(GridDev g, const double* __re
 // places in the cell list, one for each CELL_MAX of its markers: what one warp works
 // on (3000 markers in one cell by one warp: interpolation 1600 us, spreading 3340;
 // shared out 50 and 107.  With 32 instead of 64 a lattice of 64 to a cell, a million
-// markers, is 5 % slower).  Two atomics per block; cnt then holds the range's start.
-// Also the largest of the bound's counts.
-static constexpr int CELL_MAX = 64;
+// markers, is 5 % slower).  Sparse cells, of at most CELL_FEW markers, take their
+// ranges and places from the other end of the same arrays.  Five atomics per block;
+// cnt then holds the range's start.  Also the largest of the bound's counts (bcnt not
+// null).
+static constexpr int CELL_MAX = 64, CELL_FEW = 3;
 __global__ void __launch_bounds__(256) k_bin_alloc(GridDev g, const double* __restrict__ X, int n,
                                                    const int* __restrict__ bcnt, const int* __restrict__ cellof,
                                                    const int* __restrict__ rank, int* cnt, int* lcell, int* lstart, int* lcnt, int* ctr) {
-  __shared__ int sm[8], sc[8], sx[8], base[2];
+  __shared__ int sm[8], sc[8], sf[8], sx[8], base[4];
   const int m = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cell = m < n ? cellof[m] : -1;
   const bool first = cell >= 0 && rank[m] == 0;
-  const int k = first ? cnt[cell] : 0, nb = (k + CELL_MAX - 1) / CELL_MAX;
-  int a = k, b = nb, x = m < n ? bcnt[bound_cell(g, X, m)] : 0;  // inclusive scans of markers and cells
+  const int k = first ? cnt[cell] : 0;
+  const bool few = first && k <= CELL_FEW;
+  const int ka = few ? 0 : k, nb = (ka + CELL_MAX - 1) / CELL_MAX;
+  // inclusive scans: markers and places of the others, markers and cells (in the
+  // upper half) of the sparse ones
+  int a = ka, b = nb, f = few ? k + (1 << 16) : 0, x = bcnt && m < n ? bcnt[bound_cell(g, X, m)] : 0;
   for (int o = 1; o < 32; o <<= 1) {
-    const int ua = __shfl_up_sync(0xffffffffu, a, o), ub = __shfl_up_sync(0xffffffffu, b, o);
+    const int ua = __shfl_up_sync(0xffffffffu, a, o), ub = __shfl_up_sync(0xffffffffu, b, o),
+              uf = __shfl_up_sync(0xffffffffu, f, o);
     if (lane >= o) {
       a += ua;
       b += ub;
+      f += uf;
     }
     x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
   }
   if (lane == 31) {
     sm[wid] = a;
     sc[wid] = b;
+    sf[wid] = f;
     sx[wid] = x;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int ta = 0, tb = 0, tx = 0;
+    int ta = 0, tb = 0, tf = 0, tx = 0;
     for (int w = 0; w < 8; ++w) {
-      const int va = sm[w], vb = sc[w];
+      const int va = sm[w], vb = sc[w], vf = sf[w];
       sm[w] = ta;
       sc[w] = tb;
+      sf[w] = tf;
       ta += va;
       tb += vb;
+      tf += vf;
       tx = max(tx, sx[w]);
     }
     base[0] = atomicAdd(&ctr[BIN_TOTAL], ta);
     base[1] = atomicAdd(&ctr[BIN_CELLS], tb);
+    base[2] = atomicAdd(&ctr[BIN_SPARSE], tf & 0xffff);
+    base[3] = atomicAdd(&ctr[BIN_SPARSE_CELLS], tf >> 16);
     atomicMax(&ctr[BIN_CMAX], tx);
   }
   __syncthreads();
-  if (first) {
+  if (few) {
+    const int v = sf[wid] + f, start = n - base[2] - (v & 0xffff), slot = n - base[3] - (v >> 16);
+    lcell[slot] = cell;
+    lstart[slot] = start;
+    lcnt[slot] = k;
+    cnt[cell] = start;
+  } else if (first) {
     const int start = base[0] + sm[wid] + a - k, slot = base[1] + sc[wid] + b - nb;
     for (int q = 0; q < nb; ++q) {
       lcell[slot + q] = cell;
@@ -299,35 +346,38 @@ __global__ void __launch_bounds__(256) k_bin_alloc(GridDev g, const double* __re
   }
 }
 
-// Pass 3: markers in cell order; the bound's counts back to zero
+// Pass 3: markers in cell order; the bound's counts (bcnt not null) back to zero
 __global__ void __launch_bounds__(256) k_bin_fill(GridDev g, const double* __restrict__ X, int n,
                                                   const int* __restrict__ cellof, const int* __restrict__ rank,
                                                   const int* __restrict__ cnt, int* bcnt, int* perm) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
-  bcnt[bound_cell(g, X, m)] = 0;
+  if (bcnt) bcnt[bound_cell(g, X, m)] = 0;
   const int cell = cellof[m];
   if (cell >= 0) perm[cnt[cell] + rank[m]] = m;
 }
 
-void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBins& b, cudaStream_t st) {
+void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBins& b, bool spread, cudaStream_t st) {
   if (n <= 0) return;
   cudaMemsetAsync(b.ctr, 0, BIN_CTR_BYTES, st);
   const int blocks = cdiv(n, 256);
-  { k_bin_count<<<blocks, 256, 0, st>>>(g, X, n, b.cnt, b.bcnt, b.cellof, b.rank, b.irr, b.ctr); WSI_COUNT(); }
-  { k_bin_alloc<<<blocks, 256, 0, st>>>(g, X, n, b.bcnt, b.cellof, b.rank, b.cnt, b.lcell, b.lstart, b.lcnt,
+  int* const bcnt = spread ? b.bcnt : nullptr;  // (only spreading has a quantum)
+  { k_bin_count<<<blocks, 256, 0, st>>>(g, X, n, b.cnt, bcnt, b.cellof, b.rank, b.irr, b.ctr); WSI_COUNT(); }
+  { k_bin_alloc<<<blocks, 256, 0, st>>>(g, X, n, bcnt, b.cellof, b.rank, b.cnt, b.lcell, b.lstart, b.lcnt,
                                            b.ctr); WSI_COUNT(); }
-  { k_bin_fill<<<blocks, 256, 0, st>>>(g, X, n, b.cellof, b.rank, b.cnt, b.bcnt, b.perm); WSI_COUNT(); }
+  { k_bin_fill<<<blocks, 256, 0, st>>>(g, X, n, b.cellof, b.rank, b.cnt, bcnt, b.perm); WSI_COUNT(); }
 }
 
-// counts of the listed cells back to zero for the next binning
-__global__ void k_bin_clear(const int* __restrict__ lcell, const int* __restrict__ ctr, int* cnt) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ctr[BIN_CELLS]; t += gridDim.x * blockDim.x) cnt[lcell[t]] = 0;
+// counts of the cells back to zero for the next binning
+__global__ void k_bin_clear(int n, const int* __restrict__ lcell, const int* __restrict__ ctr, int* cnt) {
+  const int nc = ctr[BIN_CELLS], total = nc + ctr[BIN_SPARSE_CELLS];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x)
+    cnt[lcell[t < nc ? t : n - 1 - (t - nc)]] = 0;
 }
 
 void launch_marker_bins_clear(int n, const MarkerBins& b, cudaStream_t st) {
   if (n <= 0) return;
-  { k_bin_clear<<<std::min(cdiv(n, 256), 152 * 4), 256, 0, st>>>(b.lcell, b.ctr, b.cnt); WSI_COUNT(); }
+  { k_bin_clear<<<std::min(cdiv(n, 256), 152 * 4), 256, 0, st>>>(n, b.lcell, b.ctr, b.cnt); WSI_COUNT(); }
 }
 
 // ------------------------------------------------------------- cell transfers
@@ -460,7 +510,7 @@ __device__ __forceinline__ void batch_weights(const GridDev& g, const double* __
 // separable sums.  1.49 million markers (eight to a cell) at 256 x 128 x 128:
 // 661 us (one thread per marker, 192 loads and splits each: 1153 us).
 __global__ void __launch_bounds__(32 * CW, 8) k_interp_cells(GridDev g, const double* __restrict__ vel,
-                                                          const double* __restrict__ X, const int* __restrict__ perm,
+                                                          const double* __restrict__ X, int n, const int* __restrict__ perm,
                                                           const int* __restrict__ lcell,
                                                           const int* __restrict__ lstart,
                                                           const int* __restrict__ lcnt, const int* __restrict__ ctr,
@@ -468,11 +518,11 @@ __global__ void __launch_bounds__(32 * CW, 8) k_interp_cells(GridDev g, const do
   __shared__ float2 sv[CW][300];
   __shared__ BatchWeights sb[CW];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ncells = ctr[BIN_CELLS];
+  const int nlist = ctr[BIN_CELLS], ncells = nlist + (ctr[BIN_SPARSE] < INTERP_LIST_MIN ? ctr[BIN_SPARSE_CELLS] : 0);
   CellFaces cf;
   cf.init(g, lane);
-  for (int l = blockIdx.x * CW + w; l < ncells; l += gridDim.x * CW) {
-    const int cnt = lcnt[l];
+  for (int e = blockIdx.x * CW + w; e < ncells; e += gridDim.x * CW) {
+    const int l = e < nlist ? e : n - 1 - (e - nlist), cnt = lcnt[l];
     const int* pm = perm + lstart[l];
     cf.move(g, lcell[l]);
     __syncwarp();
@@ -551,7 +601,7 @@ __global__ void __launch_bounds__(32 * CW, 8) k_interp_cells(GridDev g, const do
 // marker the products F w_x and w_y w_z are formed once and shared.  Same
 // markers as above: 1114 us (192 global atomics per marker: 2468 us).
 __global__ void __launch_bounds__(32 * CW, 6) k_spread_cells(GridDev g, const double* __restrict__ F,
-                                                          const double* __restrict__ X, const int* __restrict__ perm,
+                                                          const double* __restrict__ X, int n, const int* __restrict__ perm,
                                                           const int* __restrict__ lcell,
                                                           const int* __restrict__ lstart,
                                                           const int* __restrict__ lcnt, const int* __restrict__ ctr,
@@ -561,14 +611,14 @@ __global__ void __launch_bounds__(32 * CW, 6) k_spread_cells(GridDev g, const do
   __shared__ float2 sp[CW][MB][60];  // F w_x of the three components (4 each), then w_z w_y (16 each)
   __shared__ long long sa[CW][300];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ncells = ctr[BIN_CELLS];
+  const int nlist = ctr[BIN_CELLS], ncells = nlist + (ctr[BIN_SPARSE] < SPREAD_LIST_MIN ? ctr[BIN_SPARSE_CELLS] : 0);
   const int E = spread_exponent(ctr, fmx, scale);
   const dfl sc = df_split(scale);
   CellFaces cf;
   cf.init(g, lane);
   for (int s = lane; s < 300; s += 32) sa[w][s] = 0;
-  for (int l = blockIdx.x * CW + w; l < ncells; l += gridDim.x * CW) {
-    const int cnt = lcnt[l];
+  for (int e = blockIdx.x * CW + w; e < ncells; e += gridDim.x * CW) {
+    const int l = e < nlist ? e : n - 1 - (e - nlist), cnt = lcnt[l];
     const int* pm = perm + lstart[l];
     cf.move(g, lcell[l]);
     for (int b0 = 0; b0 < cnt; b0 += MB) {
@@ -653,14 +703,17 @@ __global__ void k_unfix(GridDev g, SpreadBox b, Vel<unsigned long long> acc, con
 // warps for the cell kernels: a warp per cell (at most a cell per marker) up
 // to sixteen blocks per SM
 static int cell_blocks(int n) { return std::min(cdiv(n, CW), 152 * 16); }
-static constexpr int LIST_BLOCKS = 8;  // irregular markers are rare
+// blocks of 128 for the markers that get a thread each (the host doesn't know how
+// many; with eight blocks 20000 markers outside the box took 1140 us to interpolate
+// and 600 to spread, now 68 and 104)
+static int list_blocks(int n) { return std::min(cdiv(n, 128), 152 * 4); }
 
 void launch_ib_interp(const GridDev& g, const double* vel, const double* X, int n, const MarkerBins& b,
                       double* U, cudaStream_t st) {
   if (n <= 0) return;
   CVel<double> v{{vel, vel + fsize(g, 0), vel + fsize(g, 0) + fsize(g, 1)}};
-  { k_interp_cells<<<cell_blocks(n), 32 * CW, 0, st>>>(g, vel, X, b.perm, b.lcell, b.lstart, b.lcnt, b.ctr, U); WSI_COUNT(); }
-  { k_interp_list<<<LIST_BLOCKS, 128, 0, st>>>(g, v, X, b.irr, b.ctr, U); WSI_COUNT(); }
+  { k_interp_cells<<<cell_blocks(n), 32 * CW, 0, st>>>(g, vel, X, n, b.perm, b.lcell, b.lstart, b.lcnt, b.ctr, U); WSI_COUNT(); }
+  { k_interp_list<<<list_blocks(n), 128, 0, st>>>(g, v, X, n, b.irr, b.perm, b.ctr, U); WSI_COUNT(); }
 }
 
 SpreadBox spread_box(const GridDev& g, const double mm[6]) {
@@ -711,9 +764,9 @@ void launch_ib_spread(const GridDev& g, const double* F, const double* X, int n,
   Vel<double> v{{vel, vel + fsize(g, 0), vel + fsize(g, 0) + fsize(g, 1)}};
   const long long nb = (long long)(box.hi[0] - box.lo[0] + 2) * (box.hi[1] - box.lo[1] + 2) * (box.hi[2] - box.lo[2] + 2);
   const int blocks = (int)std::min<long long>((nb + 255) / 256, 152 * 4);
-  { k_spread_cells<<<cell_blocks(n), 32 * CW, 0, st>>>(g, F, X, b.perm, b.lcell, b.lstart, b.lcnt, b.ctr, b.fmx, scale,
+  { k_spread_cells<<<cell_blocks(n), 32 * CW, 0, st>>>(g, F, X, n, b.perm, b.lcell, b.lstart, b.lcnt, b.ctr, b.fmx, scale,
                                                        accv); WSI_COUNT(); }
-  { k_spread_list<<<LIST_BLOCKS, 128, 0, st>>>(g, F, X, b.irr, b.ctr, b.fmx, scale, acc); WSI_COUNT(); }
+  { k_spread_list<<<list_blocks(n), 128, 0, st>>>(g, F, X, n, b.irr, b.perm, b.ctr, b.fmx, scale, acc); WSI_COUNT(); }
   { k_unfix<<<dim3(blocks, 3), 256, 0, st>>>(g, box, acc, b.ctr, b.fmx, scale, v); WSI_COUNT(); }
 }
 

@@ -408,18 +408,20 @@ void precond_coarse_part(Precond<T>& P, const Opts& o, int l, cudaStream_t st);
 
 // ---------------------------------------------------------------- dlm.cu
 // Markers binned by the cell that holds them: sorted order (perm), the list of
-// non-empty cells (cell, first place in perm, count) and the irregular markers
-// (outside the grid or not finite), with device counters.  cnt and bcnt (one per
-// cell) are zero between uses.
-enum { BIN_CELLS = 0, BIN_TOTAL = 1, BIN_IRR = 2, BIN_CMAX = 3 };
-static constexpr int BIN_CTR_BYTES = 4 * 4 + 8;  // the four counters and fmx
+// cells (cell, first place in perm, count) and the irregular markers (outside the
+// grid or not finite), with device counters.  Sparse cells have their places at the
+// end of the list and their markers at the end of perm.  cnt and bcnt (one per cell)
+// are zero between uses.
+enum { BIN_CELLS = 0, BIN_TOTAL = 1, BIN_IRR = 2, BIN_CMAX = 3, BIN_SPARSE = 4, BIN_SPARSE_CELLS = 5 };
+static constexpr int BIN_CTR_BYTES = 6 * 4 + 8;  // the counters and fmx
 struct MarkerBins {
   int cap = 0;  // markers the arrays hold
   int *cnt = nullptr, *bcnt = nullptr, *cellof = nullptr, *rank = nullptr, *perm = nullptr, *lcell = nullptr, *lstart = nullptr,
       *lcnt = nullptr, *irr = nullptr, *ctr = nullptr;
   unsigned long long* fmx = nullptr;  // bits of max|F|, zeroed with the counters
 };
-void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBins& b, cudaStream_t st);
+// spread: the markers will be spread too (else interpolated only)
+void launch_marker_bins(const GridDev& g, const double* X, int n, const MarkerBins& b, bool spread, cudaStream_t st);
 void launch_marker_bins_clear(int n, const MarkerBins& b, cudaStream_t st);
 // vel: packed velocity vector
 void launch_ib_interp(const GridDev& g, const double* vel, const double* X, int n, const MarkerBins& b,

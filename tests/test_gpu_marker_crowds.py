@@ -60,3 +60,30 @@ def test_crowds(counts, outside):
         for q in (p[: len(p) // 2], p[:1]):
             assert np.array_equal(ctx.interp(flat, X[q]).reshape(-1, 3), U[q])
     ctx.close()
+
+
+@pytest.mark.parametrize("n,out", [(24000, 0), (30000, 100), (140000, 3000)])
+def test_many_sparse(n, out):
+    """Markers at random, mostly by ones and twos to a cell: few enough for a warp per
+    cell, enough for a thread each to interpolate, and to spread as well."""
+    c = inputs.Case(nx=66, ny=60, nz=64, lx=1.1, ly=1.0, lz=1.0)
+    g = Grid(c.nx, c.ny, c.nz, c.lx, c.ly, c.lz, c.bc)
+    rng = np.random.default_rng(n)
+    X = rng.uniform(0, 1, (n, 3)) * np.array([c.lx, c.ly, c.lz])
+    X[rng.permutation(n)[:out], 1] = -0.3 * c.ly / c.ny
+    ctx = wsi.Context(c.nx, c.ny, c.nz, c.lx, c.ly, c.lz, c.bc, c.gravity)
+    vel = [rng.standard_normal(g.face_shape(d)) * g.interior_face_mask(d) for d in range(3)]
+    flat = np.concatenate([a.ravel() for a in vel])
+    U = ctx.interp(flat, X).reshape(-1, 3)
+    ref = oib.interpolate(g, vel, X)
+    assert np.abs(U - ref).max() < 1e-11 * np.abs(ref).max()
+    p = rng.permutation(n)
+    assert np.array_equal(ctx.interp(flat, X[p]).reshape(-1, 3), U[p])
+    assert np.array_equal(ctx.interp(flat, X[p[:2000]]).reshape(-1, 3), U[p[:2000]])
+    F = rng.standard_normal(X.shape)
+    S = ctx.spread(F, X, 2e-4)
+    ref = np.concatenate([a.ravel() for a in oib.spread(g, F, X, 2e-4)])
+    mag = np.concatenate([a.ravel() for a in oib.spread(g, np.abs(F), X, 2e-4)])
+    assert np.abs(S - ref).max() < 1e-12 * np.abs(mag).max()
+    assert np.array_equal(ctx.spread(F[p], X[p], 2e-4), S)
+    ctx.close()
