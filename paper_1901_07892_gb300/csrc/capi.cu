@@ -133,6 +133,8 @@ struct wsi_ctx {
   unsigned long long* sacc = nullptr;  // deterministic spreading: one integer per face (on first use)
   MarkerBins bins;                // markers sorted by cell (grown on first use)
   void* bins_mem = nullptr;
+  double* mstage = nullptr;       // wsi_interp, wsi_spread: the caller's markers and their values (grown on first use)
+  int mstage_cap = 0;
   double* mbox = nullptr;         // 6 doubles: marker extent
   UNetImpl* gunet_impl = nullptr;  // initial-guess network (wsi_attach_unet_guess)
   int gunet_level = 0;
@@ -203,6 +205,23 @@ bool ensure_bins(wsi_ctx* c, int n) {
   int** q[7] = {&b.cellof, &b.rank, &b.perm, &b.lcell, &b.lstart, &b.lcnt, &b.irr};
   for (int a = 0; a < 7; ++a) *q[a] = p + (size_t)a * n;
   b.cap = n;
+  return true;
+}
+
+// device copies of n markers and of three values each
+bool ensure_marker_stage(wsi_ctx* c, int n) {
+  if (n <= c->mstage_cap) return true;
+  double* p = nullptr;
+  if (cudaMalloc(&p, (size_t)n * 6 * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (c->mstage) {
+    cudaStreamSynchronize(c->st);
+    cudaFree(c->mstage);
+  }
+  c->mstage = p;
+  c->mstage_cap = n;
   return true;
 }
 
@@ -988,6 +1007,7 @@ void wsi_destroy(wsi_ctx* c) {
   precond_free<double>(c->P64);
   precond_free<float>(c->P32);
   cudaFree(c->bins_mem);
+  cudaFree(c->mstage);
   for (ZVec& z : c->zv) zvec_release(z);
   df_operands_release(c->df);
   for (void* p : c->allocs) cudaFree(p);
@@ -1527,10 +1547,9 @@ int wsi_reinit(wsi_ctx* c, double* phi, int iters) {
 int wsi_interp(wsi_ctx* c, const double* vel, const double* X, int n, double* U) {
   if (valid_ctx(c)) return WSI_ERR_INVALID_ARG;
   if (n <= 0) return WSI_OK;
-  if (!ensure_bins(c, n)) return fail(c, WSI_ERR_OOM, "out of device memory for markers");
-  double* dX = dalloc(c, (size_t)n * 3);
-  double* dU = dalloc(c, (size_t)n * 3);
-  if (!dX || !dU) return fail(c, WSI_ERR_OOM, "out of device memory");
+  if (!ensure_bins(c, n) || !ensure_marker_stage(c, n)) return fail(c, WSI_ERR_OOM, "out of device memory for markers");
+  double* dX = c->mstage;
+  double* dU = dX + (size_t)n * 3;
   int rc = copy_in(c, c->vel_half, vel, c->nvel);
   if (!rc) rc = copy_in(c, dX, X, (size_t)n * 3);
   if (rc) return rc;
@@ -1538,24 +1557,20 @@ int wsi_interp(wsi_ctx* c, const double* vel, const double* X, int n, double* U)
   launch_ib_interp(c->g, c->vel_half, dX, n, c->bins, dU, c->st);
   launch_marker_bins_clear(n, c->bins, c->st);
   rc = copy_out(c, U, dU, (size_t)n * 3);
-  cudaStreamSynchronize(c->st);
-  // release the temporaries (last two allocations)
-  cudaFree(dX);
-  cudaFree(dU);
-  c->allocs.resize(c->allocs.size() - 2);
-  if (rc) return rc;
+  if (rc) {
+    cudaStreamSynchronize(c->st);  // the caller's arrays may still be read
+    return rc;
+  }
   return cuda_check(c, "interp");
 }
 
 int wsi_spread(wsi_ctx* c, const double* F, const double* X, int n, double dV, double* vel) {
   if (valid_ctx(c)) return WSI_ERR_INVALID_ARG;
-  // the work arrays first: the two staging buffers below must stay the last
-  // two allocations (they are released at the end)
-  if (!ensure_spread_work(c) || !ensure_bins(c, std::max(n, 1)))
+  const int room = std::max(n, 1);
+  if (!ensure_spread_work(c) || !ensure_bins(c, room) || !ensure_marker_stage(c, room))
     return fail(c, WSI_ERR_OOM, "out of device memory for spreading");
-  double* dX = dalloc(c, (size_t)std::max(n, 1) * 3);
-  double* dF = dalloc(c, (size_t)std::max(n, 1) * 3);
-  if (!dX || !dF) return fail(c, WSI_ERR_OOM, "out of device memory");
+  double* dX = c->mstage;
+  double* dF = dX + (size_t)room * 3;
   int rc = WSI_OK;
   if (n > 0) {
     rc = copy_in(c, dX, X, (size_t)n * 3);
@@ -1575,11 +1590,10 @@ int wsi_spread(wsi_ctx* c, const double* F, const double* X, int n, double dV, d
     }
     rc = copy_out(c, vel, c->vel_half, c->nvel);
   }
-  cudaStreamSynchronize(c->st);
-  cudaFree(dX);
-  cudaFree(dF);
-  c->allocs.resize(c->allocs.size() - 2);
-  if (rc) return rc;
+  if (rc) {
+    cudaStreamSynchronize(c->st);  // the caller's arrays may still be read
+    return rc;
+  }
   return cuda_check(c, "spread");
 }
 
