@@ -40,9 +40,9 @@ PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # 2 flop x 2.07 GHz); used only when the measurement (wsi_fma_peak) fails
 FP64_PEAK_DERIVED_GFLOPS = 152 * 2 * 2 * 2.07
 # DRAM bytes per cell of one launch, measured with ncu at 128^3 (dram__bytes_read.sum +
-# dram__bytes_write.sum, profiles/k_stokes_df_tank128.md) for the current kernel revision;
-# scaled by the cells of the workload (empty while no capture of the current revision exists)
-TRAFFIC_PER_CELL = {}
+# dram__bytes_write.sum, profiles/k_stokes_df_tank128.md) for the current kernel revision, the mean
+# of its two forms; scaled by the cells of the workload
+TRAFFIC_PER_CELL = {("stokes", "mixed"): (199.269632e6 + 46.62784e6 + 170.531584e6 + 46.711808e6) / 2 / 128 ** 3}
 KCLASS = {"stokes": 0, "rbgs_p": 1, "rbgs_v": 2, "transport": 3, "mdot": 4, "maxpy": 5, "restrict": 6,
           "prolong": 7, "reinit": 8}
 

@@ -2,12 +2,12 @@
 // (Sec. 3.3) with the wall-adjoint forms J_BC / S_BC (Sec. 3.3.2).
 //
 // Both transfers work cell by cell.  The markers are binned by the cell that
-// holds them (counting sort; markers outside the grid or not finite go to a
-// short list of their own), and one warp serves the markers of one cell: their
+// holds them (counting sort), and one warp serves up to 64 markers of a cell: their
 // taps cover the same 4 x 5 x 5 faces of each component, so interpolation loads
 // and splits these 300 values once for all of them, and spreading sums their
-// contributions in registers and issues one atomic per face instead of one per
-// marker and tap.  Weights and sums are double-float (float64 accuracy on the
+// contributions in shared memory and issues one atomic per face instead of one per
+// marker and tap.  Markers outside the grid or not finite, and many markers far
+// apart, get a thread each.  Weights and sums are double-float (float64 accuracy on the
 // float32 pipes; GB300's float64 rate is 1/64 of its float32 rate).  Taps that
 // fall beyond a wall are folded onto their mirror image with the ghost sign
 // (tangential: the wall's sign; normal: odd about the wall face, whose own

@@ -40,9 +40,13 @@ template <typename T>
 struct CoarseCycle;
 template <typename T, int NT>
 __global__ void k_coarse_cycle(const __grid_constant__ CoarseCycle<T> c);
-// cells of a level that one block works on in shared memory, and of one that the
-// fused lower cycle takes at all; float64 updates are bound by the narrow pipe of
-// the SMs that take part, so fewer of them go to one block or one cluster
+// Cells of a level that one block works on in shared memory, and of one that the
+// fused lower cycle takes at all.  float64 updates are bound by the narrow pipe of
+// the SMs that take part, so there the whole GPU wins earlier.  Measured per V-cycle
+// in float64, fused from 512, 4096 and 32768 cells down: 16^3 121, 110 and 110 us, 32 x 16 x 16
+// 167, 148 and 136, 32^3 178, 166 and 180, 64^2 161, 132 and 132, 128^2 212, 183 and
+// 176; one block up to 256, 512 and 1024 cells: 16^3 119, 110 and 110, 64^2 132, 132
+// and 124 (float32 16^3 80, 71 and 71, 64^2 82, 82 and 72).
 template <typename T>
 static constexpr int coarse_smem_cells() { return 512; }
 template <typename T>
